@@ -328,13 +328,15 @@ def run_ours(args, rank, world, local_rank):
         e2e["ms_per_step"] = max_over_ranks(e2e["ms_per_step"], dev)
     A.pp_mesh_destroy(m)
     A.pp_destroy(ctx)
+    solves = counts["stage_gmres"] + counts["stage_gmres32"]
+    krylov = iters["gmres_primal"] + iters["gmres_tangent"] + iters["gmres_adjoint"]
     return dict(config=args.config, ms=ms, nu=nu, ne=ne, Nt=Nt, clocks=clocks, iters=iters, split=split, kern=kern,
-                counts=counts, e2e=e2e)
+                counts=counts, e2e=e2e, steps_per_solve=krylov * args.steps / max(solves, 1))
 
 
-# kernel classes timed by the bench: (folded stage operator, fused Arnoldi step)
-KERNELS = {"fp64": ("stage_op", "arnoldi"), "mixed": ("stage_op32", "arnoldi32")}
-PROF_STRIDE = 8   # one launch (one Arnoldi step) in 8 is bracketed by CUDA events
+# kernel classes timed by the bench: (one-launch stage solves, block Jacobian)
+KERNELS = {"fp64": ("stage_gmres", "jacobian"), "mixed": ("stage_gmres32", "jacobian")}
+PROF_STRIDE = 1   # every launch is bracketed by CUDA events (about 1,200 launches of these classes a step)
 
 
 def roofline_for(kernel, res, peaks, fp64_tflops, c, sustained):
@@ -361,7 +363,31 @@ def roofline_for(kernel, res, peaks, fp64_tflops, c, sustained):
                 "launches": launches, "avg_us": t * 1e6, "algorithmic_bytes_per_launch": counted / launches,
                 "note": "basis of one stage solve (<= 41 x N_u words) is L2-resident: a low fraction means "
                         "latency-bound grid reductions, not HBM"}
+    if kernel == "jacobian":
+        # basis contraction of the 4 blocks plus the two tables W = C T per variable pair; the flux
+        # derivatives at the points are not counted
+        nqv, nqf = (p + 2) ** 2, 3 * (p + 2)
+        flops = 2.0 * ne * 16 * (Np * Np * (2 * nqv + 2 * nqf) + 3 * Np * (2 * nqv + 2 * nqf))
+        ach = flops / t / 1e12
+        return {"bound": "alu", "achieved": ach, "peak": fp64_tflops, "unit": "TFLOP/s",
+                "frac": ach / fp64_tflops if fp64_tflops else None, "traffic": None,
+                "kernel": "k_jacobian (element block Jacobian)", "launches": launches, "avg_us": t * 1e6}
     word = 4 if kernel.endswith("32") else 8
+    if kernel.startswith("stage_gmres"):
+        # one launch = one solve of `steps` Krylov steps (mean over the last bench step's solves); a
+        # step reads the 3 blocks and operand slices of every element once
+        steps = res["steps_per_solve"]
+        byts = steps * ne * (3 * nb * nb + 5 * nb) * word
+        note = "%.1f steps per solve; blocks of one solve %.0f MB" % (steps, ne * 3 * nb * nb * word / 1e6)
+        common = {"traffic": MEASURED_TRAFFIC.get((kernel, res["config"])), "launches": launches, "avg_us": t * 1e6,
+                  "kernel": "k_stage_gmres<%d,%s> (whole stage solve, eliminated elements taken out)"
+                  % (nb, "double" if word == 8 else "float"), "hbm_gbs_equiv": byts / t / 1e9, "note": note}
+        if word == 8:
+            ach = 2.0 * steps * ne * 3 * nb * nb / t / 1e12
+            return {"bound": "alu", "achieved": ach, "peak": fp64_tflops, "unit": "TFLOP/s",
+                    "frac": ach / fp64_tflops if fp64_tflops else None, **common}
+        ach = byts / t / 1e9
+        return {"bound": "hbm", "achieved": ach, "peak": hbm, "unit": "GB/s", "frac": ach / hbm, **common}
     # folded operator: 3 blocks + 3 neighbour slices + own slice + output per element
     byts = ne * (3 * nb * nb * word + 5 * nb * word)
     if word == 8:

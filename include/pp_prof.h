@@ -29,7 +29,9 @@ extern "C" {
 #define PP_K_STAGE_OP32 13     /* FP32 folded stage operator of the mixed-precision inner solves */
 #define PP_K_ARNOLDI 14        /* the Gram-Schmidt passes of one FP64 Arnoldi step (3 launches) */
 #define PP_K_ARNOLDI32 15      /* the same in FP32 (mixed-precision inner solves) */
-#define PP_K_COUNT 16
+#define PP_K_STAGE_GMRES 16    /* one whole FP64 stage solve: red-black reduced GMRES and x = D^-1 y */
+#define PP_K_STAGE_GMRES32 17  /* the same in FP32 (mixed-precision inner and Newton solves) */
+#define PP_K_COUNT 18
 
 /* Starts timing every launch of kernel class `kind` (PP_K_NONE stops), and only that class.
    Resets the accumulated totals of every class.  Not thread-safe: one host thread drives

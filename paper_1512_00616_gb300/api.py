@@ -37,7 +37,7 @@ EXPORTED = [
 ]
 PP_K = dict(none=0, jacobian=1, residual=2, stage_matvec=3, block_apply=4, block_inverse=5, krylov=6, other=7,
             stage_matvec32=8, block_apply32=9, krylov32=10, stage_op=11, fold=12, stage_op32=13, arnoldi=14,
-            arnoldi32=15)
+            arnoldi32=15, stage_gmres=16, stage_gmres32=17)
 
 
 class pp_config(C.Structure):

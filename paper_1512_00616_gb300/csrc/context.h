@@ -49,6 +49,7 @@ struct KrylovT {
 };
 using Krylov = KrylovT<double>;
 constexpr int kRing = 4;
+constexpr int kDot = 47;          // d_scalar / h_scalar words: dot product | record of the stage solves (2)
 
 // Motion quantities at one time and their derivatives w.r.t. mu.
 struct Motion {
@@ -73,11 +74,14 @@ struct pp_ctx {
   // reductions
   double* d_partial = nullptr;
   unsigned* d_counter = nullptr;
-  double* d_scalar = nullptr;  // [64]
+  double* d_scalar = nullptr;  // [64]; kDot: a dot product, then the record of the stage solves
   double* h_scalar = nullptr;  // pinned [64]
   int* d_status = nullptr;
   double* d_arn = nullptr;     // fused Arnoldi step: CTA partials
   unsigned* d_arn_bar = nullptr;  // fused Arnoldi step: arrival count, release epoch, error word
+  double* d_gm = nullptr;      // stage solves: CTA partials
+  unsigned* d_gm_bar = nullptr;   // stage solves: barrier words
+  double steps_seen = 0.0;     // Krylov steps already counted from the record in d_scalar
   double* d_gterm = nullptr;   // adjoint-sweep gradient terms, 9 per stage [3 * Nt][9]
   size_t gterm_cap = 0;        // capacity in stages
 

@@ -663,10 +663,14 @@ int pp_create(const pp_config* cfg, pp_ctx** out) {
       cudaMalloc(&ctx->d_status, sizeof(int) * 4) != cudaSuccess ||
       cudaMalloc(&ctx->d_arn, sizeof(double) * arnoldi_partial_words()) != cudaSuccess ||
       cudaMalloc(&ctx->d_arn_bar, sizeof(unsigned) * arnoldi_barrier_words()) != cudaSuccess ||
+      cudaMalloc(&ctx->d_gm, sizeof(double) * stage_gmres_partial_words()) != cudaSuccess ||
+      cudaMalloc(&ctx->d_gm_bar, sizeof(unsigned) * stage_gmres_barrier_words()) != cudaSuccess ||
       cudaMallocHost(&ctx->h_scalar, sizeof(double) * 64) != cudaSuccess)
     return fail(PP_ENOMEM);
   if (cudaMemset(ctx->d_counter, 0, sizeof(unsigned) * 4) != cudaSuccess ||
       cudaMemset(ctx->d_status, 0, sizeof(int) * 4) != cudaSuccess ||
+      cudaMemset(ctx->d_scalar, 0, sizeof(double) * 64) != cudaSuccess ||
+      cudaMemset(ctx->d_gm_bar, 0, sizeof(unsigned) * stage_gmres_barrier_words()) != cudaSuccess ||
       cudaMemset(ctx->d_arn_bar, 0, sizeof(unsigned) * arnoldi_barrier_words()) != cudaSuccess)
     return fail(PP_ECUDA);
   *out = ctx;
@@ -685,6 +689,8 @@ int pp_destroy(pp_ctx* ctx) {
   cudaFree(ctx->d_gterm);
   cudaFree(ctx->d_arn);
   cudaFree(ctx->d_arn_bar);
+  cudaFree(ctx->d_gm);
+  cudaFree(ctx->d_gm_bar);
   if (ctx->h_scalar) cudaFreeHost(ctx->h_scalar);
   cudaFree(ctx->d_J);
   cudaFree(ctx->d_Ainv);
@@ -797,6 +803,52 @@ int pp_mesh_create(pp_ctx* ctx, const double* verts, int nv, const int32_t* tris
       side[i] = (e2 < 0 || e2 > e) ? 1 : 0;
     }
   (void)p;
+  // Elimination order of the stage solves: two-colour each component breadth first; where the
+  // mesh is not two-colourable an element of the second colour that meets another one is kept.
+  // The larger class is eliminated; elements without neighbours are kept.
+  std::vector<int> colour(nt, -1), queue;
+  queue.reserve(nt);
+  for (int s = 0; s < nt; ++s) {
+    if (colour[s] >= 0) continue;
+    colour[s] = 0;
+    size_t head = queue.size();
+    queue.push_back(s);
+    for (; head < queue.size(); ++head)
+      for (int f = 0; f < 3; ++f) {
+        const int e2 = nbr[3 * queue[head] + f];
+        if (e2 >= 0 && colour[e2] < 0) {
+          colour[e2] = 1 - colour[queue[head]];
+          queue.push_back(e2);
+        }
+      }
+  }
+  const int ones = (int)std::count(colour.begin(), colour.end(), 1);
+  const int drop = 2 * ones >= nt ? 1 : 0;
+  std::vector<char> eliminated(nt, 0);
+  for (int e : queue) {
+    if (colour[e] != drop) continue;
+    bool alone = true, free = true;
+    for (int f = 0; f < 3; ++f) {
+      const int e2 = nbr[3 * e + f];
+      if (e2 < 0) continue;
+      alone = false;
+      if (eliminated[e2]) free = false;
+    }
+    eliminated[e] = !alone && free;
+  }
+  std::vector<int> order, place(nt), order_nbr(3 * (size_t)nt);
+  order.reserve(nt);
+  for (int e = 0; e < nt; ++e)
+    if (!eliminated[e]) order.push_back(e);
+  const int n_kept = (int)order.size();
+  for (int e = 0; e < nt; ++e)
+    if (eliminated[e]) order.push_back(e);
+  for (int q = 0; q < nt; ++q) place[order[q]] = q;
+  for (int q = 0; q < nt; ++q)
+    for (int f = 0; f < 3; ++f) {
+      const int e2 = nbr[3 * order[q] + f];
+      order_nbr[3 * q + f] = e2 >= 0 ? place[e2] : -1;
+    }
   pp_mesh* m = new pp_mesh();
   m->ctx = ctx;
   m->ne = nt;
@@ -813,6 +865,8 @@ int pp_mesh_create(pp_ctx* ctx, const double* verts, int nv, const int32_t* tris
   ints.insert(ints.end(), nbrface.begin(), nbrface.end());
   ints.insert(ints.end(), tag.begin(), tag.end());
   ints.insert(ints.end(), side.begin(), side.end());
+  ints.insert(ints.end(), order.begin(), order.end());
+  ints.insert(ints.end(), order_nbr.begin(), order_nbr.end());
   if (cudaSetDevice(ctx->device) != cudaSuccess ||
       cudaMalloc(&m->d_real, sizeof(double) * real.size()) != cudaSuccess ||
       cudaMalloc(&m->d_int, sizeof(int) * ints.size()) != cudaSuccess) {
@@ -840,6 +894,9 @@ int pp_mesh_create(pp_ctx* ctx, const double* verts, int nv, const int32_t* tris
   d.nbrface = m->d_int + 3 * nt;
   d.tag = m->d_int + 6 * nt;
   d.side = m->d_int + 9 * nt;
+  d.n_kept = n_kept;
+  d.order = m->d_int + 12 * nt;
+  d.order_nbr = m->d_int + 13 * nt;
   *out = m;
   return PP_OK;
 }

@@ -23,6 +23,7 @@
 // HBM-bound; the same products in FP32 are bandwidth-bound.
 #include "pp_internal.h"
 #include "prof.h"
+#include "reduce.cuh"
 #include "../../include/pp_prof.h"
 
 namespace pp {
@@ -125,39 +126,6 @@ __global__ void __launch_bounds__(INV_THREADS)
     if (outT) outT[ent] = A[col][row];
   }
 }
-
-// ------------------------------------------------------------------ warp reduce-scatter
-template <int CNT, int O, class T>
-__device__ __forceinline__ void rs_step(T* v, int lane) {
-  if constexpr (O > 0) {
-    if constexpr (CNT > 1) {
-      constexpr int half = CNT / 2;
-      const bool upper = (lane & O) != 0;
-#pragma unroll
-      for (int t = 0; t < half; ++t) {
-        const T send = upper ? v[t] : v[t + half];
-        const T keep = upper ? v[t + half] : v[t];
-        v[t] = keep + __shfl_xor_sync(0xffffffffu, send, O);
-      }
-      rs_step<half, O / 2, T>(v, lane);
-    } else {
-      v[0] += __shfl_xor_sync(0xffffffffu, v[0], O);
-      rs_step<1, O / 2, T>(v, lane);
-    }
-  }
-}
-
-// Warp reduce-scatter of KB (power of two, <= 32) per-lane values: afterwards lane l
-// holds the warp sum of value (l >> (5 - log2 KB)) in v[0] (31 shuffles for KB = 32).
-template <int KB, class T>
-__device__ __forceinline__ void warp_reduce_scatter(T* v, int lane) {
-  rs_step<KB, 16, T>(v, lane);
-}
-
-template <int KB>
-struct ILog2 {
-  static constexpr int value = KB >= 32 ? 5 : KB >= 16 ? 4 : KB >= 8 ? 3 : KB >= 4 ? 2 : KB >= 2 ? 1 : 0;
-};
 
 // ------------------------------------------------------------------ block products
 // Warp-per-block products with compile-time block size NB = 4 Np.  Normal: lanes over

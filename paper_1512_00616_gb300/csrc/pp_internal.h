@@ -116,6 +116,11 @@ struct DevMesh {
   const int* nbr;        // [ne][3]   neighbour or -1
   const int* nbrface;    // [ne][3]
   const int* tag;        // [ne][3]   0 interior, 1 wall, 2 far field
+  // elimination order of the stage solves: positions 0 .. n_kept - 1 hold the kept elements,
+  // the rest the eliminated ones, no two of which share a face
+  int n_kept;
+  const int* order;      // [ne]      element at each position
+  const int* order_nbr;  // [ne][3]   positions of its face neighbours or -1
 };
 
 // ---------------------------------------------------------------- kernel wrappers
@@ -225,6 +230,35 @@ template <class S>
 cudaError_t launch_stream_rows(const DevMesh& m, const DevTables& tb, int nb, int nblk, const S* B, double alpha,
                                double beta, const S* x, S* y, cudaStream_t st);
 cudaError_t stream_rows_error(int* flag, bool reset);  // bounded-wait expiry flag of those kernels
+// One stage solve (gmres_kernels.cu): restarted GMRES on (I + B) y = b with the folded blocks B
+// and the eliminated elements taken out, then x = D y.  Nothing is read back: failures (1 the cap
+// with need_conv set, 4 non-finite, 8 an expired barrier wait) stay in rec[0], which makes later
+// solves return at once, and rec[1] counts the Krylov steps.  V holds m + 1 vectors, z and y one
+// each; ywarm (kept elements, or null) is the initial guess when warm is set and receives y.
+template <class S>
+struct StageGmres {
+  const S* B;
+  const S* D;
+  int d_trans;       // apply the transposed D blocks
+  const S* b;
+  S* x;
+  S* ywarm;
+  int warm;
+  double rtol, atol;
+  int maxit, m, need_conv;
+  S* V;
+  S* z;
+  S* y;
+  double* partial;   // stage_gmres_partial_words()
+  unsigned* bar;     // stage_gmres_barrier_words(), zero before the first launch
+  double* rec;
+};
+constexpr int kGmresMaxRestart = 60;
+constexpr int kClusterRows = 2560;  // most kept rows solved by one cluster of 8 CTAs (one pass each)
+template <class S>
+cudaError_t launch_stage_gmres(const DevMesh& m, int nb, const StageGmres<S>& q, cudaStream_t st);
+size_t stage_gmres_partial_words();
+int stage_gmres_barrier_words();
 // BN = -c J_off Ainv_nbr and BT = (-c Ainv_nbr J_off,nbr)^T (3 blocks per element each; BT may
 // be null): the block-Jacobi preconditioner folded into the stage operator.
 template <class S>

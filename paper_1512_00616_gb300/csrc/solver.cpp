@@ -5,10 +5,11 @@
 //  - gmres():          restarted, right-preconditioned GMRES with classical
 //                      Gram-Schmidt and selective reorthogonalization (fused
 //                      update + multi-dot kernels), Givens rotations on the
-//                      device.  Used for the stage solves (on the operator with
-//                      the block-Jacobi preconditioner folded in) and, without
-//                      preconditioner, for the shooting system (Algorithm primal)
-//                      and the periodic adjoint system (Algorithm dual).
+//                      device.  Used for the shooting system (Algorithm primal), the
+//                      periodic adjoint system (Algorithm dual), the pseudo-transient
+//                      steps of the steady state, the outer level of mixed precision,
+//                      and stage solves without room for the folded operator; the
+//                      other stage solves are one launch each (gmres_kernels.cu).
 //  - primal_sweep():   Eq. dirk2: DIRK3 steps, Newton per stage on
 //                      R_i = M k_i - dt r(u_i); stores u_i, dr/du(u_i) and the
 //                      block-Jacobi inverse at the converged stage.
@@ -41,11 +42,36 @@ double now_s() {
 
 template <class S>
 int host_dot(pp_ctx* ctx, int64_t n, const S* x, const S* y, double* out) {
-  PP_CK(launch_dot<S>(n, x, y, ctx->d_scalar, ctx->d_partial, ctx->d_counter, ctx->stream));
-  PP_CK(cudaMemcpyAsync(ctx->h_scalar, ctx->d_scalar, sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
+  PP_CK(launch_dot<S>(n, x, y, ctx->d_scalar + kDot, ctx->d_partial, ctx->d_counter, ctx->stream));
+  PP_CK(cudaMemcpyAsync(ctx->h_scalar + kDot, ctx->d_scalar + kDot, 3 * sizeof(double), cudaMemcpyDeviceToHost,
+                        ctx->stream));
   PP_CK(cudaStreamSynchronize(ctx->stream));
-  *out = ctx->h_scalar[0];
+  *out = ctx->h_scalar[kDot];
   return PP_OK;
+}
+
+// The record of the stage solves as the last synchronized copy has it (host_dot, read_record):
+// adds the steps since the last call to *steps, and turns a failure into its status, clearing it
+// for the next sweep.
+int take_record(pp_ctx* ctx, int64_t* steps) {
+  const double code = ctx->h_scalar[kDot + 1], done = ctx->h_scalar[kDot + 2];
+  *steps += (int64_t)(done - ctx->steps_seen);
+  ctx->steps_seen = done;
+  if (code == 0.0) return PP_OK;
+  ctx->steps_seen = 0.0;
+  PP_CK(cudaMemsetAsync(ctx->d_scalar + kDot + 1, 0, 2 * sizeof(double), ctx->stream));
+  PP_CK(cudaMemsetAsync(ctx->d_gm_bar, 0, sizeof(unsigned) * stage_gmres_barrier_words(), ctx->stream));
+  PP_CK(cudaStreamSynchronize(ctx->stream));
+  if (code == 1.0) return set_error(ctx, PP_ENOCONV, "stage GMRES hit gmres_maxit");
+  if (code == 4.0) return set_error(ctx, PP_ENAN, "GMRES: non-finite Arnoldi quantity");
+  return set_error(ctx, PP_ECUDA, "stage GMRES: grid barrier wait expired");
+}
+
+int read_record(pp_ctx* ctx, int64_t* steps) {
+  PP_CK(cudaMemcpyAsync(ctx->h_scalar + kDot, ctx->d_scalar + kDot, 3 * sizeof(double), cudaMemcpyDeviceToHost,
+                        ctx->stream));
+  PP_CK(cudaStreamSynchronize(ctx->stream));
+  return take_record(ctx, steps);
 }
 
 int host_norm(pp_ctx* ctx, int64_t n, const double* x, double* out) {
@@ -232,20 +258,13 @@ int stage_solve32(pp_ctx* ctx, const pp_mesh* mesh, const StageView& sv, int tra
   const DevMesh& m = mesh->dev;
   const float* Bf = trans ? sv.BT32 : sv.BN32;
   if (Bf) {
-    // folded operator: GMRES on (I + B) y = b, then x = D^{-1} y (D^{-T} y)
-    float* yv = ctx->k32.t;
-    // Krylov recurrence on B (Arnoldi adds the unit shift back to H): w = B v keeps most of
-    // its norm after the projections, where w = (I + B) v cancels down to |B v|
-    OpT<float> A = [&](const float* in, float* out) {
-      ProfScope ps(PP_K_STAGE_OP32, ctx->stream);
-      PP_CK(launch_stream_rows<float>(m, ctx->tb, ctx->tb.nb, 3, Bf, 0.0, 0.0, in, out, ctx->stream));
-      return PP_OK;
-    };
-    int st = gmres<float>(ctx, ctx->k32, A, OpT<float>(), b, yv, rtol, 0.0, maxit, iters, nullptr, false, false,
-                          1.0);
-    if (st != PP_OK && st != PP_ENOCONV) return st;
-    PP_CK(launch_block_apply<float>(m, ctx->tb.nb, trans ? sv.AT32 : sv.A32, yv, x, 0, ctx->stream));
-    return PP_OK;  // an inexact inner / Newton solve is acceptable
+    // one launch; an inexact inner / Newton solve is acceptable, its steps are in the record
+    KrylovT<float>& K = ctx->k32;
+    PP_CK(launch_stage_gmres<float>(m, ctx->tb.nb,
+                                    {Bf, trans ? sv.AT32 : sv.A32, 0, b, x, nullptr, 0, rtol, 0.0, maxit, K.m, 0, K.V,
+                                     K.w, K.t, ctx->d_gm, ctx->d_gm_bar, ctx->d_scalar + kDot + 1},
+                                    ctx->stream));
+    return PP_OK;
   }
   const float* Jm = trans ? sv.JT32 : sv.J32;   // the transposed copies run through the normal kernels
   const float* Am = trans ? sv.AT32 : sv.A32;
@@ -263,10 +282,13 @@ int stage_solve32(pp_ctx* ctx, const pp_mesh* mesh, const StageView& sv, int tra
 
 // Stage solve (M - c J) x = b or its transpose.  exact = false (primal Newton steps)
 // may be inexact; exact = true (tangent / adjoint) must reach rtol on the FP64 operator.
+// *iters counts the steps of the host-driven levels; those of the one-launch solves and their
+// failures are in the record (take_record).
 int stage_solve(pp_ctx* ctx, const pp_mesh* mesh, const StageView& sv, int trans, const double* b, double* x,
                 double rtol, double atol, int* iters, bool exact, double* ywarm = nullptr, bool use_warm = false) {
   const DevMesh& m = mesh->dev;
   const int64_t n = ctx->ws_nu;
+  *iters = 0;
   if (ctx->cfg.precision == PP_PREC_MIXED) {
     float* b32 = ctx->d_vec32;
     float* x32 = ctx->d_vec32 + n;
@@ -302,23 +324,14 @@ int stage_solve(pp_ctx* ctx, const pp_mesh* mesh, const StageView& sv, int trans
   // FP64 path with the folded operator: GMRES on (I + B) y = b, then x = D^{-1} y (D^{-T} y)
   const double* Bf = trans ? sv.BT : sv.BN;
   if (Bf) {
-    double* yv = ctx->kin.t;  // unused by GMRES without a preconditioner
-    // Krylov recurrence on B, shifted back in H (see stage_solve32)
-    Op A = [&](const double* in, double* out) {
-      ProfScope ps(PP_K_STAGE_OP, ctx->stream);
-      PP_CK(launch_stream_rows<double>(m, ctx->tb, ctx->tb.nb, 3, Bf, 0.0, 0.0, in, out, ctx->stream));
-      return PP_OK;
-    };
-    // warm start (linear sweeps): the same stage's y of the previous step is the initial guess
-    if (ywarm && use_warm) PP_TRY(copy(ctx, n, yv, ywarm));
-    int st = gmres<double>(ctx, ctx->kin, A, Op(), b, yv, rtol, atol, ctx->cfg.gmres_maxit, iters, nullptr, false,
-                           ywarm && use_warm, 1.0);
-    if (st != PP_OK && st != PP_ENOCONV) return st;
-    if (ywarm) PP_TRY(copy(ctx, n, ywarm, yv));
-    if (!trans) PP_CK(launch_block_apply<double>(m, ctx->tb.nb, sv.Ainv, yv, x, 0, ctx->stream));
-    else if (sv.AinvT) PP_CK(launch_block_apply<double>(m, ctx->tb.nb, sv.AinvT, yv, x, 0, ctx->stream));
-    else PP_CK(launch_block_apply<double>(m, ctx->tb.nb, sv.Ainv, yv, x, 1, ctx->stream));
-    if (st == PP_ENOCONV && exact) return set_error(ctx, PP_ENOCONV, "stage GMRES hit gmres_maxit");
+    // one launch; a warm start (linear sweeps) takes the same stage's y of the previous step
+    Krylov& K = ctx->kin;
+    const bool at = trans && sv.AinvT;
+    PP_CK(launch_stage_gmres<double>(m, ctx->tb.nb,
+                                     {Bf, at ? sv.AinvT : sv.Ainv, trans && !at, b, x, ywarm, use_warm ? 1 : 0, rtol,
+                                      atol, ctx->cfg.gmres_maxit, K.m, exact ? 1 : 0, K.V, K.w, K.t, ctx->d_gm,
+                                      ctx->d_gm_bar, ctx->d_scalar + kDot + 1},
+                                     ctx->stream));
     return PP_OK;
   }
   // FP64 path: with stored transposes the transposed system uses the normal (row-streaming) kernels
@@ -450,6 +463,7 @@ int run_steps(pp_ctx* ctx, const pp_mesh* mesh, const double* mu, int n_mu, doub
         PP_TRY(lincomb(ctx, n, R, {1.0, -dt}, {R, r}));
         double rn2, mun;
         PP_TRY(host_dot<double>(ctx, n, R, R, &rn2));
+        PP_TRY(take_record(ctx, &ctx->last_gmres_iters));
         double rn = std::sqrt(rn2);
         // backtracking safeguard: a step that made the residual non-finite or larger is halved
         if (it > 0 && (!std::isfinite(rn) || rn > prev_res) && backtracks < 8) {
@@ -520,11 +534,13 @@ int run_steps(pp_ctx* ctx, const pp_mesh* mesh, const double* mu, int n_mu, doub
 
 // Makes the stage data of step `step` resident (checkpointed linearization: recompute
 // its segment from the stored state and predictor at the segment start).
-int ensure_segment(pp_ctx* ctx, int step) {
+// Steps of the linear solves so far go to *steps before the recomputation counts its own.
+int ensure_segment(pp_ctx* ctx, int step, int64_t* steps) {
   const int K = ctx->cfg.checkpoint_stride;
   if (K <= 0) return PP_OK;
   const int seg = step / K;
   if (seg == ctx->seg_cur) return PP_OK;
+  PP_TRY(read_record(ctx, steps));
   const int64_t n = ctx->ws_nu;
   double* u = work_vec(ctx, 0);
   double* kprev = work_vec(ctx, 8);
@@ -610,7 +626,7 @@ int tangent_sweep(pp_ctx* ctx, const double* v, double* out) {
   PP_TRY(copy(ctx, n, du, v));
   ctx->last_gmres_tangent = 0;
   for (int step = 0; step < Nt; ++step) {
-    PP_TRY(ensure_segment(ctx, step));
+    PP_TRY(ensure_segment(ctx, step, &ctx->last_gmres_tangent));
     for (int i = 0; i < 3; ++i) {
       StageView sv = stored_stage(ctx, step, i);
       const double* win = du;
@@ -629,6 +645,7 @@ int tangent_sweep(pp_ctx* ctx, const double* v, double* out) {
     }
     PP_TRY(lincomb(ctx, n, du, {1.0, ctx->b[0], ctx->b[1], ctx->b[2]}, {du, dk[0], dk[1], dk[2]}));
   }
+  PP_TRY(read_record(ctx, &ctx->last_gmres_tangent));
   PP_TRY(lincomb(ctx, n, out, {1.0, -1.0}, {v0, du}));
   PP_CK(cudaStreamSynchronize(ctx->stream));
   PP_TRY(check_stream_kernels(ctx));
@@ -671,7 +688,7 @@ int adjoint_sweep(pp_ctx* ctx, const double* lam_Nt, const double* weights, doub
   PP_TRY(copy(ctx, n, lam, lam_Nt));
   ctx->last_gmres_adjoint = 0;
   for (int step = Nt - 1; step >= 0; --step) {
-    PP_TRY(ensure_segment(ctx, step));
+    PP_TRY(ensure_segment(ctx, step, &ctx->last_gmres_adjoint));
     for (int i = 2; i >= 0; --i) {
       StageView sv = stored_stage(ctx, step, i);
       const double ti = step * dt + ctx->c[i] * dt;
@@ -737,6 +754,7 @@ int adjoint_sweep(pp_ctx* ctx, const double* lam_Nt, const double* weights, doub
     if (withF)
       PP_TRY(lincomb(ctx, n, lam, {1.0, dt * ctx->b[0], dt * ctx->b[1], dt * ctx->b[2]}, {lam, g[0], g[1], g[2]}));
   }
+  PP_TRY(read_record(ctx, &ctx->last_gmres_adjoint));
   PP_TRY(copy(ctx, n, lam0, lam));
   std::vector<double> gterm;
   if (withF && dFdmu) {
@@ -1267,7 +1285,8 @@ int stage_apply(pp_ctx* ctx, int step, int i, int kind, int trans, int prec, con
     return set_error(ctx, PP_EINVAL, "pp_stage_apply: bad arguments");
   if (prec == 1 && ctx->cfg.precision != PP_PREC_MIXED)
     return set_error(ctx, PP_EINVAL, "pp_stage_apply: FP32 copies exist in PP_PREC_MIXED only");
-  PP_TRY(ensure_segment(ctx, step));
+  int64_t steps = 0;
+  PP_TRY(ensure_segment(ctx, step, &steps));
   const pp_mesh* mesh = ctx->lin_mesh;
   const DevMesh& m = mesh->dev;
   const int64_t n = ctx->ws_nu;
