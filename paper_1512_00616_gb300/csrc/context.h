@@ -93,6 +93,7 @@ struct pp_ctx {
   double* d_vec = nullptr;      // pool of work vectors
   int n_vec = 0;
   double* d_elem = nullptr;     // [ne*8] per-element partials
+  int* d_wexp = nullptr;        // exponents of the operand and the basis of the stage solves
   pp::Krylov kin, kout;         // stage-solve and outer (shooting / periodic adjoint) GMRES levels
   pp::KrylovT<float> k32;       // inner FP32 level of the mixed-precision stage solves
   float* d_vec32 = nullptr;     // FP32 work vectors [4][nu]
@@ -108,8 +109,10 @@ struct pp_ctx {
   double* st_u = nullptr;       // [stages][nu] stage states
   double* st_JT = nullptr;      // [stages][ne*4*nb*nb] transposed block-columns (optional)
   double* st_AinvT = nullptr;   // [stages][ne*nb*nb] transposed inverses (optional; FP64 mode)
-  double* st_BN = nullptr;      // [stages][ne*3*nb*nb] folded operator blocks -c J_off D^-1 (optional; FP64 mode)
-  double* st_BT = nullptr;      // [stages][ne*3*nb*nb] folded transposed blocks (optional; FP64 mode)
+  uint64_t* st_BN = nullptr;    // [stages][ne*3*nb*nb] folded operator blocks -c J_off D^-1, fixed-point words (optional; FP64 mode)
+  uint64_t* st_BT = nullptr;    // [stages][ne*3*nb*nb] folded transposed blocks (optional; FP64 mode)
+  int* st_EN = nullptr;         // [stages][ne*3*nb] exponents of their rows
+  int* st_ET = nullptr;
   float* st_BN32 = nullptr;     // mixed mode: FP32 folded blocks from the FP32 copies (optional)
   float* st_BT32 = nullptr;
   float* st_J32 = nullptr;      // mixed mode: FP32 copies of J, J^T-columns and the inverses

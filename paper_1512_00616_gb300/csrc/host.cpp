@@ -406,14 +406,17 @@ int ensure_workspace(pp_ctx* ctx, const pp_mesh* mesh) {
   cudaFree(ctx->d_Ainv);
   cudaFree(ctx->d_vec);
   cudaFree(ctx->d_elem);
+  cudaFree(ctx->d_wexp);
   ctx->d_J = ctx->d_Ainv = ctx->d_vec = ctx->d_elem = nullptr;
+  ctx->d_wexp = nullptr;
   const size_t nb2 = (size_t)ctx->tb.nb * ctx->tb.nb;
   ctx->n_vec = 30;  // 0-8 primal, 9-15 tangent, 14-23 adjoint, 24-26 shooting / periodic adjoint,
                     // 27-29 warm starts of the linear stage solves
   if (cudaMalloc(&ctx->d_J, sizeof(double) * mesh->ne * 4 * nb2) != cudaSuccess ||
       cudaMalloc(&ctx->d_Ainv, sizeof(double) * mesh->ne * nb2) != cudaSuccess ||
       cudaMalloc(&ctx->d_vec, sizeof(double) * ctx->n_vec * nu) != cudaSuccess ||
-      cudaMalloc(&ctx->d_elem, sizeof(double) * mesh->ne * 8) != cudaSuccess) {
+      cudaMalloc(&ctx->d_elem, sizeof(double) * mesh->ne * 8) != cudaSuccess ||
+      cudaMalloc(&ctx->d_wexp, sizeof(int) * (size_t)mesh->ne * (ctx->cfg.gmres_restart + 2)) != cudaSuccess) {
     cudaGetLastError();
     ctx->ws_ne = 0;
     return set_error(ctx, PP_ENOMEM, "workspace allocation failed");
@@ -456,7 +459,15 @@ int ensure_store(pp_ctx* ctx, const pp_mesh* mesh, int Nt) {
   }
   if (ctx->store_stages >= stages && ctx->lin_mesh == mesh) return PP_OK;
   auto release = [&]() {
-    for (double** p : {&ctx->st_J, &ctx->st_Ainv, &ctx->st_u, &ctx->st_JT, &ctx->st_AinvT, &ctx->st_BN, &ctx->st_BT}) {
+    for (double** p : {&ctx->st_J, &ctx->st_Ainv, &ctx->st_u, &ctx->st_JT, &ctx->st_AinvT}) {
+      cudaFree(*p);
+      *p = nullptr;
+    }
+    for (uint64_t** p : {&ctx->st_BN, &ctx->st_BT}) {
+      cudaFree(*p);
+      *p = nullptr;
+    }
+    for (int** p : {&ctx->st_EN, &ctx->st_ET}) {
       cudaFree(*p);
       *p = nullptr;
     }
@@ -489,13 +500,16 @@ int ensure_store(pp_ctx* ctx, const pp_mesh* mesh, int Nt) {
   // path), kept while 8 GB of device memory stay free
   {
     const size_t nB = stages * mesh->ne * 3 * nb2;
-    const size_t word = mixed ? sizeof(float) : sizeof(double);
+    const size_t nE = mixed ? 0 : nB / ctx->tb.nb;
+    const size_t word = mixed ? sizeof(float) : sizeof(uint64_t);
     cudaMemGetInfo(&fr, &tot);
-    if (fr > word * 2 * nB + ((size_t)8 << 30)) {
+    if (fr > 2 * (word * nB + sizeof(int) * nE) + ((size_t)8 << 30)) {
       bool okB;
       if (!mixed)
-        okB = cudaMalloc(&ctx->st_BN, sizeof(double) * nB) == cudaSuccess &&
-              cudaMalloc(&ctx->st_BT, sizeof(double) * nB) == cudaSuccess;
+        okB = cudaMalloc(&ctx->st_BN, sizeof(uint64_t) * nB) == cudaSuccess &&
+              cudaMalloc(&ctx->st_BT, sizeof(uint64_t) * nB) == cudaSuccess &&
+              cudaMalloc(&ctx->st_EN, sizeof(int) * nE) == cudaSuccess &&
+              cudaMalloc(&ctx->st_ET, sizeof(int) * nE) == cudaSuccess;
       else
         okB = cudaMalloc(&ctx->st_BN32, sizeof(float) * nB) == cudaSuccess &&
               cudaMalloc(&ctx->st_BT32, sizeof(float) * nB) == cudaSuccess;
@@ -503,8 +517,11 @@ int ensure_store(pp_ctx* ctx, const pp_mesh* mesh, int Nt) {
         cudaGetLastError();
         cudaFree(ctx->st_BN);
         cudaFree(ctx->st_BT);
+        cudaFree(ctx->st_EN);
+        cudaFree(ctx->st_ET);
         cudaFree(ctx->st_BN32);
         cudaFree(ctx->st_BT32);
+        ctx->st_EN = ctx->st_ET = nullptr;
         ctx->st_BN = ctx->st_BT = nullptr;
         ctx->st_BN32 = ctx->st_BT32 = nullptr;
       }
@@ -697,6 +714,7 @@ int pp_destroy(pp_ctx* ctx) {
   cudaFree(ctx->d_vec);
   cudaFree(ctx->d_vec32);
   cudaFree(ctx->d_elem);
+  cudaFree(ctx->d_wexp);
   for (Krylov* k : {&ctx->kin, &ctx->kout}) {
     free_krylov(*k);
     for (int i = 0; i < kRing; ++i)
@@ -712,6 +730,8 @@ int pp_destroy(pp_ctx* ctx) {
   cudaFree(ctx->st_AinvT);
   cudaFree(ctx->st_BN);
   cudaFree(ctx->st_BT);
+  cudaFree(ctx->st_EN);
+  cudaFree(ctx->st_ET);
   cudaFree(ctx->st_J32);
   cudaFree(ctx->st_JT32);
   cudaFree(ctx->st_A32);

@@ -18,9 +18,10 @@
 //    reduction (warp, CTA, then the CTA that finishes last in a fixed order), and the
 //    GMRES Givens update fused into the norm pass.
 //
-// GB300 note: its FP64 pipe issues ~2 DFMA per clock per SM, so FP64 block products are
-// ALU-bound (~21 us for the 4 x 40 x 40 x 2048 Jacobian product) before they are
+// GB300 note: its FP64 pipe issues 1.68 DFMA per clock per SM, so FP64 block products are
+// ALU-bound (~25 us for the 4 x 40 x 40 x 2048 Jacobian product) before they are
 // HBM-bound; the same products in FP32 are bandwidth-bound.
+#include "fixed.cuh"
 #include "pp_internal.h"
 #include "prof.h"
 #include "reduce.cuh"
@@ -337,37 +338,44 @@ __global__ void __launch_bounds__(256)
 //   BT[e][f] = (-c Ainv[e2] J[e2][1+g])^T              g = nbrface(e, f)
 // so that (M - cJ) D^{-1} = I + BN and (M - cJ)^T D^{-T} = I + BT, with D = M - c J_ee the
 // block diagonal (Ainv its inverse) and BN, BT zero on boundary faces.
+// FP64 blocks are written as fixed-point words (fixed.cuh), one exponent per block row in EN / ET
+// [e][f][row]; FP32 blocks as floats (EN, ET unused).
 template <int NB, class S>
 __global__ void __launch_bounds__(256)
-    k_fold_blocks(DevMesh m, const S* __restrict__ J, const S* __restrict__ Ainv, double c, S* __restrict__ BN,
-                  S* __restrict__ BT) {
+    k_fold_blocks(DevMesh m, const S* __restrict__ J, const S* __restrict__ Ainv, double c, FoldOut<S> out) {
   extern __shared__ __align__(16) unsigned char fsm_raw[];
+  __shared__ int rmax[NB];
   S* P = reinterpret_cast<S*>(fsm_raw);
   S* Q = P + NB * NB;
   constexpr int nb2 = NB * NB;
+  constexpr int NV = (nb2 + 255) / 256;
   const int e = blockIdx.x / 3, f = blockIdx.x - 3 * (blockIdx.x / 3);
   const int e2 = m.nbr[3 * e + f];
-  S* outN = BN ? BN + ((size_t)e * 3 + f) * nb2 : nullptr;
-  S* outT = BT ? BT + ((size_t)e * 3 + f) * nb2 : nullptr;
-  if (e2 < 0) {
-    for (int i = threadIdx.x; i < nb2; i += blockDim.x) {
-      if (outN) outN[i] = S(0);
-      if (outT) outT[i] = S(0);
-    }
-    return;
-  }
+  const size_t blk = ((size_t)e * 3 + f) * nb2;
   for (int pass = 0; pass < 2; ++pass) {
-    S* out = pass == 0 ? outN : outT;
-    if (!out) continue;
+    auto* const dst = pass == 0 ? out.BN : out.BT;
+    int* const exps = pass == 0 ? out.EN : out.ET;
+    if (!dst) continue;
+    if (e2 < 0) {
+      for (int i = threadIdx.x; i < nb2; i += 256) dst[blk + i] = {};
+      if (exps)
+        for (int i = threadIdx.x; i < NB; i += 256) exps[((size_t)e * 3 + f) * NB + i] = 0;
+      continue;
+    }
     const S* Pg = pass == 0 ? J + ((size_t)e * 4 + 1 + f) * nb2 : Ainv + (size_t)e2 * nb2;
     const S* Qg = pass == 0 ? Ainv + (size_t)e2 * nb2 : J + ((size_t)e2 * 4 + 1 + m.nbrface[3 * e + f]) * nb2;
     __syncthreads();
-    for (int i = threadIdx.x; i < nb2; i += blockDim.x) {
+    for (int i = threadIdx.x; i < nb2; i += 256) {
       P[i] = Pg[i];
       Q[i] = Qg[i];
     }
+    if (threadIdx.x < NB) rmax[threadIdx.x] = 0;
     __syncthreads();
-    for (int idx = threadIdx.x; idx < nb2; idx += blockDim.x) {
+    S val[NV];
+#pragma unroll
+    for (int t = 0; t < NV; ++t) {
+      const int idx = threadIdx.x + 256 * t;
+      if (idx >= nb2) continue;
       const int cc = idx / NB, r = idx - cc * NB;  // output (r, cc), column-major
       S a0 = S(0), a1 = S(0);
       if (pass == 0) {
@@ -385,9 +393,42 @@ __global__ void __launch_bounds__(256)
           a1 += P[(k + 1) * NB + cc] * Q[r * NB + k + 1];
         }
       }
-      out[idx] = S(-c) * (a0 + a1);
+      val[t] = S(-c) * (a0 + a1);
+      if constexpr (sizeof(S) == 8) atomicMax(&rmax[r], fix_exponent(val[t]));
+      else dst[blk + idx] = val[t];
+    }
+    if constexpr (sizeof(S) == 8) {
+      __syncthreads();
+#pragma unroll
+      for (int t = 0; t < NV; ++t) {
+        const int idx = threadIdx.x + 256 * t;
+        if (idx < nb2) dst[blk + idx] = fix_encode(val[t], rmax[idx % NB]);
+      }
+      if (threadIdx.x < NB) exps[((size_t)e * 3 + f) * NB + threadIdx.x] = rmax[threadIdx.x];
     }
   }
+}
+
+// y = x + B x with the stored folded blocks (diagnostics); one CTA per element, thread = row
+template <class S>
+__global__ void __launch_bounds__(64)
+    k_folded_apply(DevMesh m, int nb, const typename FoldOut<S>::W* __restrict__ B, const int* __restrict__ E,
+                   const S* __restrict__ x, S* __restrict__ y) {
+  const int e = blockIdx.x, r = threadIdx.x;
+  if (r >= nb) return;
+  S s = x[(size_t)e * nb + r];
+  for (int f = 0; f < 3; ++f) {
+    const int e2 = m.nbr[3 * e + f];
+    if (e2 < 0) continue;
+    const size_t blk = (size_t)e * 3 + f;
+    for (int c = 0; c < nb; ++c) {
+      S b;
+      if constexpr (sizeof(S) == 8) b = fix_decode(B[blk * nb * nb + (size_t)c * nb + r], E[blk * nb + r]);
+      else b = B[blk * nb * nb + (size_t)c * nb + r];
+      s += b * x[(size_t)e2 * nb + c];
+    }
+  }
+  y[(size_t)e * nb + r] = s;
 }
 
 // ------------------------------------------------------------------ vector kernels
@@ -1179,7 +1220,7 @@ cudaError_t launch_block_apply(const DevMesh& m, int nb, const S* Ainv, const S*
 }
 
 template <class S>
-cudaError_t launch_fold_blocks(const DevMesh& m, int nb, const S* J, const S* Ainv, double c, S* BN, S* BT,
+cudaError_t launch_fold_blocks(const DevMesh& m, int nb, const S* J, const S* Ainv, double c, const FoldOut<S>& out,
                                cudaStream_t st) {
   ProfScope ps(PP_K_FOLD, st);
   const size_t smem = sizeof(S) * 2 * nb * nb;
@@ -1188,7 +1229,7 @@ cudaError_t launch_fold_blocks(const DevMesh& m, int nb, const S* J, const S* Ai
     static const cudaError_t attr =                                                                      \
         cudaFuncSetAttribute(k_fold_blocks<NBV, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
     if (attr != cudaSuccess) return attr;                                                                \
-    k_fold_blocks<NBV, S><<<m.ne * 3, 256, smem, st>>>(m, J, Ainv, c, BN, BT);                           \
+    k_fold_blocks<NBV, S><<<m.ne * 3, 256, smem, st>>>(m, J, Ainv, c, out);                              \
     break;                                                                                               \
   }
   switch (nb) {
@@ -1200,6 +1241,14 @@ cudaError_t launch_fold_blocks(const DevMesh& m, int nb, const S* J, const S* Ai
       return cudaErrorInvalidValue;
   }
 #undef PP_FOLD
+  return cudaGetLastError();
+}
+
+template <class S>
+cudaError_t launch_folded_apply(const DevMesh& m, int nb, const typename FoldOut<S>::W* B, const int* E, const S* x,
+                                S* y, cudaStream_t st) {
+  ProfScope ps(PP_K_OTHER, st);
+  k_folded_apply<S><<<m.ne, 64, 0, st>>>(m, nb, B, E, x, y);
   return cudaGetLastError();
 }
 
@@ -1449,8 +1498,10 @@ cudaError_t launch_scale(int64_t n, double* y, double a, const double* x, cudaSt
                                              unsigned*, cudaStream_t);                                              \
   template cudaError_t launch_update_norm2<S>(int64_t, const S*, int64_t, int, const double*, S*, double*, double*, \
                                               unsigned*, cudaStream_t);                                             \
-  template cudaError_t launch_fold_blocks<S>(const DevMesh&, int, const S*, const S*, double, S*, S*,         \
-                                             cudaStream_t);                                                     \
+  template cudaError_t launch_fold_blocks<S>(const DevMesh&, int, const S*, const S*, double, const FoldOut<S>&,    \
+                                             cudaStream_t);                                                         \
+  template cudaError_t launch_folded_apply<S>(const DevMesh&, int, const typename FoldOut<S>::W*, const int*,       \
+                                              const S*, S*, cudaStream_t);                                          \
   template cudaError_t launch_arnoldi_step<S>(int64_t, const S*, int64_t, int, S*, S*, double*, double*, double*,    \
                                              double*, unsigned*, double*, int, int, double*, double*, double*,      \
                                              double*, double*, double, cudaStream_t);                               \

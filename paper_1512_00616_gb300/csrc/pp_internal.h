@@ -222,22 +222,21 @@ cudaError_t launch_colsum(int ne, int k, const double* per_elem, double* out, do
                           cudaStream_t st);
 
 // TMA-staged block-row products (stream_kernels.cu): nblk = 4, the stage operator
-// y = alpha M x + beta J x; nblk = 3, the folded operator y = x + B x (beta != 0) or its
-// shifted form y = B x (beta = 0); nblk = 1, the block product y = A x.  Normal products only.
+// y = alpha M x + beta J x; nblk = 1, the block product y = A x.  Normal products only.
 template <class S>
 bool stream_rows_supported(int nb, const S* B, const S* x, const S* y);
 template <class S>
 cudaError_t launch_stream_rows(const DevMesh& m, const DevTables& tb, int nb, int nblk, const S* B, double alpha,
                                double beta, const S* x, S* y, cudaStream_t st);
 cudaError_t stream_rows_error(int* flag, bool reset);  // bounded-wait expiry flag of those kernels
-// One stage solve (gmres_kernels.cu): restarted GMRES on (I + B) y = b with the folded blocks B
+// One stage solve (gmres_kernels.cuh): restarted GMRES on (I + B) y = b with the folded blocks B
 // and the eliminated elements taken out, then x = D y.  Nothing is read back: failures (1 the cap
 // with need_conv set, 4 non-finite, 8 an expired barrier wait) stay in rec[0], which makes later
-// solves return at once, and rec[1] counts the Krylov steps.  V holds m + 1 vectors, z and y one
-// each; ywarm (kept elements, or null) is the initial guess when warm is set and receives y.
+// solves return at once, and rec[1] counts the Krylov steps.  V holds m + 1 vectors; ywarm (kept elements, or null) is the initial guess when warm is set and receives y.
 template <class S>
 struct StageGmres {
-  const S* B;
+  const void* B;     // folded blocks as launch_fold_blocks writes them, and their exponents (FP64)
+  const int* Bexp;
   const S* D;
   int d_trans;       // apply the transposed D blocks
   const S* b;
@@ -247,8 +246,9 @@ struct StageGmres {
   double rtol, atol;
   int maxit, m, need_conv;
   S* V;
-  S* z;
-  S* y;
+  S* y;              // [N_u]
+  S* wire;           // [N_u] words of the exchanged operand
+  int* wexp;         // [ne + (m + 1) ne] exponents of its slices and of the basis (FP64)
   double* partial;   // stage_gmres_partial_words()
   unsigned* bar;     // stage_gmres_barrier_words(), zero before the first launch
   double* rec;
@@ -260,10 +260,32 @@ cudaError_t launch_stage_gmres(const DevMesh& m, int nb, const StageGmres<S>& q,
 size_t stage_gmres_partial_words();
 int stage_gmres_barrier_words();
 // BN = -c J_off Ainv_nbr and BT = (-c Ainv_nbr J_off,nbr)^T (3 blocks per element each; BT may
-// be null): the block-Jacobi preconditioner folded into the stage operator.
+// be null): the block-Jacobi preconditioner folded into the stage operator.  FP64 blocks are
+// stored as fixed-point words (fixed.cuh) with one exponent per block row (EN, ET).
+struct Fix;
 template <class S>
-cudaError_t launch_fold_blocks(const DevMesh& m, int nb, const S* J, const S* Ainv, double c, S* BN, S* BT,
+struct FoldOut {
+  using W = float;
+  float* BN;
+  float* BT;
+  int* EN = nullptr;
+  int* ET = nullptr;
+};
+template <>
+struct FoldOut<double> {
+  using W = Fix;
+  Fix* BN;
+  Fix* BT;
+  int* EN;
+  int* ET;
+};
+template <class S>
+cudaError_t launch_fold_blocks(const DevMesh& m, int nb, const S* J, const S* Ainv, double c, const FoldOut<S>& out,
                                cudaStream_t st);
+// y = x + B x with those blocks
+template <class S>
+cudaError_t launch_folded_apply(const DevMesh& m, int nb, const typename FoldOut<S>::W* B, const int* E, const S* x,
+                                S* y, cudaStream_t st);
 int reduction_blocks();  // number of partial sums used by the reductions
 
 }  // namespace pp

@@ -9,7 +9,7 @@
 //                      periodic adjoint system (Algorithm dual), the pseudo-transient
 //                      steps of the steady state, the outer level of mixed precision,
 //                      and stage solves without room for the folded operator; the
-//                      other stage solves are one launch each (gmres_kernels.cu).
+//                      other stage solves are one launch each (gmres_kernels.cuh).
 //  - primal_sweep():   Eq. dirk2: DIRK3 steps, Newton per stage on
 //                      R_i = M k_i - dt r(u_i); stores u_i, dr/du(u_i) and the
 //                      block-Jacobi inverse at the converged stage.
@@ -246,8 +246,10 @@ struct StageView {
   const float* JT32 = nullptr;
   const float* A32 = nullptr;
   const float* AT32 = nullptr;
-  const double* BN = nullptr;     // folded operator I + BN = (M - cJ) D^{-1} (optional, FP64 mode)
-  const double* BT = nullptr;     // folded transposed operator I + BT = (M - cJ)^T D^{-T}
+  const uint64_t* BN = nullptr;   // folded operator I + BN = (M - cJ) D^{-1} (optional, FP64 mode): fixed-point
+  const uint64_t* BT = nullptr;   // words; folded transposed operator I + BT = (M - cJ)^T D^{-T}
+  const int* EN = nullptr;        // exponents of their rows
+  const int* ET = nullptr;
   const float* BN32 = nullptr;    // mixed mode: FP32 folded blocks of the inner solves
   const float* BT32 = nullptr;
 };
@@ -261,8 +263,8 @@ int stage_solve32(pp_ctx* ctx, const pp_mesh* mesh, const StageView& sv, int tra
     // one launch; an inexact inner / Newton solve is acceptable, its steps are in the record
     KrylovT<float>& K = ctx->k32;
     PP_CK(launch_stage_gmres<float>(m, ctx->tb.nb,
-                                    {Bf, trans ? sv.AT32 : sv.A32, 0, b, x, nullptr, 0, rtol, 0.0, maxit, K.m, 0, K.V,
-                                     K.w, K.t, ctx->d_gm, ctx->d_gm_bar, ctx->d_scalar + kDot + 1},
+                                    {Bf, nullptr, trans ? sv.AT32 : sv.A32, 0, b, x, nullptr, 0, rtol, 0.0, maxit, K.m, 0,
+                                     K.V, K.t, K.w, ctx->d_wexp, ctx->d_gm, ctx->d_gm_bar, ctx->d_scalar + kDot + 1},
                                     ctx->stream));
     return PP_OK;
   }
@@ -322,15 +324,15 @@ int stage_solve(pp_ctx* ctx, const pp_mesh* mesh, const StageView& sv, int trans
     return st;
   }
   // FP64 path with the folded operator: GMRES on (I + B) y = b, then x = D^{-1} y (D^{-T} y)
-  const double* Bf = trans ? sv.BT : sv.BN;
+  const uint64_t* Bf = trans ? sv.BT : sv.BN;
   if (Bf) {
     // one launch; a warm start (linear sweeps) takes the same stage's y of the previous step
     Krylov& K = ctx->kin;
     const bool at = trans && sv.AinvT;
     PP_CK(launch_stage_gmres<double>(m, ctx->tb.nb,
-                                     {Bf, at ? sv.AinvT : sv.Ainv, trans && !at, b, x, ywarm, use_warm ? 1 : 0, rtol,
-                                      atol, ctx->cfg.gmres_maxit, K.m, exact ? 1 : 0, K.V, K.w, K.t, ctx->d_gm,
-                                      ctx->d_gm_bar, ctx->d_scalar + kDot + 1},
+                                     {Bf, trans ? sv.ET : sv.EN, at ? sv.AinvT : sv.Ainv, trans && !at, b, x, ywarm,
+                                      use_warm ? 1 : 0, rtol, atol, ctx->cfg.gmres_maxit, K.m, exact ? 1 : 0, K.V,
+                                      K.t, K.w, ctx->d_wexp, ctx->d_gm, ctx->d_gm_bar, ctx->d_scalar + kDot + 1},
                                      ctx->stream));
     return PP_OK;
   }
@@ -364,6 +366,8 @@ StageView stage_view_slot(pp_ctx* ctx, size_t s, double c) {
   if (ctx->st_AinvT) v.AinvT = ctx->st_AinvT + s * ne * nb2(ctx);
   if (ctx->st_BN) v.BN = ctx->st_BN + s * ne * 3 * nb2(ctx);
   if (ctx->st_BT) v.BT = ctx->st_BT + s * ne * 3 * nb2(ctx);
+  if (ctx->st_EN) v.EN = ctx->st_EN + s * ne * 3 * ctx->tb.nb;
+  if (ctx->st_ET) v.ET = ctx->st_ET + s * ne * 3 * ctx->tb.nb;
   if (ctx->st_BN32) v.BN32 = ctx->st_BN32 + s * ne * 3 * nb2(ctx);
   if (ctx->st_BT32) v.BT32 = ctx->st_BT32 + s * ne * 3 * nb2(ctx);
   if (ctx->st_J32) {
@@ -398,8 +402,9 @@ int finalize_stage_slot(pp_ctx* ctx, const pp_mesh* mesh, const StageView& sv, b
       if (sv.JT) PP_CK(launch_transpose_blocks<double, double>(m, nb, sv.J, const_cast<double*>(sv.JT), ctx->stream));
     }
     if (sv.BN32)
-      PP_CK(launch_fold_blocks<float>(m, nb, sv.J32, sv.A32, sv.c, const_cast<float*>(sv.BN32),
-                                      full && sv.BT32 ? const_cast<float*>(sv.BT32) : nullptr, ctx->stream));
+      PP_CK(launch_fold_blocks<float>(
+          m, nb, sv.J32, sv.A32, sv.c,
+          {const_cast<float*>(sv.BN32), full && sv.BT32 ? const_cast<float*>(sv.BT32) : nullptr}, ctx->stream));
     return PP_OK;
   }
   PP_CK(launch_block_inverse<double>(m, ctx->tb, sv.J, sv.c, const_cast<double*>(sv.Ainv),
@@ -407,8 +412,10 @@ int finalize_stage_slot(pp_ctx* ctx, const pp_mesh* mesh, const StageView& sv, b
   if (full && sv.JT)
     PP_CK(launch_transpose_blocks<double, double>(m, nb, sv.J, const_cast<double*>(sv.JT), ctx->stream));
   if (sv.BN)
-    PP_CK(launch_fold_blocks(m, nb, sv.J, sv.Ainv, sv.c, const_cast<double*>(sv.BN),
-                             full && sv.BT ? const_cast<double*>(sv.BT) : nullptr, ctx->stream));
+    PP_CK(launch_fold_blocks<double>(m, nb, sv.J, sv.Ainv, sv.c,
+                                     {(Fix*)sv.BN, full && sv.BT ? (Fix*)sv.BT : nullptr, const_cast<int*>(sv.EN),
+                                      const_cast<int*>(sv.ET)},
+                                     ctx->stream));
   return PP_OK;
 }
 
@@ -1301,9 +1308,9 @@ int stage_apply(pp_ctx* ctx, int step, int i, int kind, int trans, int prec, con
       if (trans && sv.AinvT) PP_CK(launch_block_apply<double>(m, nb, sv.AinvT, x, y, 0, ctx->stream));
       else PP_CK(launch_block_apply<double>(m, nb, sv.Ainv, x, y, trans, ctx->stream));
     } else {
-      const double* Bf = trans ? sv.BT : sv.BN;
+      const uint64_t* Bf = trans ? sv.BT : sv.BN;
       if (!Bf) return set_error(ctx, PP_ESTATE, "pp_stage_apply: no FP64 folded operator stored");
-      PP_CK(launch_stream_rows<double>(m, ctx->tb, nb, 3, Bf, 0.0, 1.0, x, y, ctx->stream));
+      PP_CK(launch_folded_apply<double>(m, nb, (const Fix*)Bf, trans ? sv.ET : sv.EN, x, y, ctx->stream));
     }
   } else {
     if (!sv.J32) return set_error(ctx, PP_ESTATE, "pp_stage_apply: no FP32 copies stored");
@@ -1317,7 +1324,7 @@ int stage_apply(pp_ctx* ctx, int step, int i, int kind, int trans, int prec, con
     } else {
       const float* Bf = trans ? sv.BT32 : sv.BN32;
       if (!Bf) return set_error(ctx, PP_ESTATE, "pp_stage_apply: no FP32 folded operator stored");
-      PP_CK(launch_stream_rows<float>(m, ctx->tb, nb, 3, Bf, 0.0, 1.0, x32, y32, ctx->stream));
+      PP_CK(launch_folded_apply<float>(m, nb, Bf, nullptr, x32, y32, ctx->stream));
     }
     PP_CK(launch_cast<float, double>(n, y, y32, ctx->stream));
   }

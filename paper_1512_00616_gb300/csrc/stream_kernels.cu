@@ -3,16 +3,12 @@
 //
 //  y_e = alpha detB_e (Mref (x) I4) x_e + beta sum_q B_{e,q} x_{src(e,q)}     NBLK = 4
 //  y_e = A_e x_e                                                              NBLK = 1
-//  y_e = x_e + sum_f B_{e,f} x_{nbr(e,f)}                                     NBLK = 3
 //
 // NBLK = 4 is the DIRK stage operator M - a_ii dt dr/du of Eq. dirk2 (diagonal block and
 // the three face-neighbour blocks of the element row; the Jacobian J[e][q] is stored as
 // contiguous column-major nb x nb blocks).  NBLK = 1 is the block-Jacobi preconditioner
-// application (explicit inverse A_e of the diagonal block).  NBLK = 3 is the stage
-// operator with the block-Jacobi preconditioner folded in, (M - cJ) D^{-1} = I + O D^{-1}
-// (D the diagonal blocks, O the face-neighbour blocks; B_{e,f} = O_{e,f} D^{-1}_{nbr}
-// precomputed per stage).  All read every matrix entry exactly once per call, which
-// makes them the streaming (HBM / L2) core of each Krylov step of the stage solves.
+// application (explicit inverse A_e of the diagonal block).  Both read every matrix entry
+// exactly once per call.
 //
 // Design for sm_103a:
 //  - persistent CTAs, grid = resident CTAs per SM x SM count, element e of CTA b is
@@ -114,10 +110,10 @@ __device__ __forceinline__ bool consumer_all(bool v, int nthreads) {
 
 template <int NB, int NBLK, class S>
 struct StreamShape {
-  static constexpr int NG = NBLK == 3 ? 3 : 4;  // column groups per element
+  static constexpr int NG = 4;                  // column groups per element
   static constexpr int CW = (NG * NB + 31) / 32;  // consumer warps
   static constexpr int THREADS = 32 * (CW + 1);
-  static constexpr int UNIT = NB * NB + 2 * NB;  // block + input slice (+ own slice), elements of S
+  static constexpr int UNIT = NB * NB + NB;  // block + input slice, elements of S
   static constexpr int UNIT_BYTES = UNIT * (int)sizeof(S);
   static constexpr int BUDGET = 100 * 1024;  // two CTAs per SM where the units fit (measured
                                              // faster than four smaller rings at nb = 40)
@@ -168,11 +164,8 @@ __global__ void __launch_bounds__(StreamShape<NB, NBLK, S>::THREADS)
       const int e = (int)blockIdx.x + li * G;
       int src = e;
       if (NBLK == 4 && q > 0) src = m.nbr[3 * e + q - 1];
-      if (NBLK == 3) src = m.nbr[3 * e + q];
       S* dst = ring + (size_t)slot * UNIT;
-      const bool own = (NBLK == 3 && q == 0);  // the identity term needs the element's own slice
-      const uint32_t bytes = (src >= 0 ? (uint32_t)((NB * NB + NB) * sizeof(S)) : 0u) +
-                             (own ? (uint32_t)(NB * sizeof(S)) : 0u);
+      const uint32_t bytes = src >= 0 ? (uint32_t)((NB * NB + NB) * sizeof(S)) : 0u;
       pres[slot] = src >= 0 ? 1 : 0;
       if (bytes == 0) {
         mbar_arrive(&full[slot]);  // boundary face: nothing to load, the consumers skip it
@@ -182,7 +175,6 @@ __global__ void __launch_bounds__(StreamShape<NB, NBLK, S>::THREADS)
           bulk_load(dst, B + ((size_t)e * NBLK + q) * NB * NB, (uint32_t)(NB * NB * sizeof(S)), &full[slot]);
           bulk_load(dst + NB * NB, x + (size_t)src * NB, (uint32_t)(NB * sizeof(S)), &full[slot]);
         }
-        if (own) bulk_load(dst + NB * NB + NB, x + (size_t)e * NB, (uint32_t)(NB * sizeof(S)), &full[slot]);
       }
     }
     return;
@@ -216,7 +208,7 @@ __global__ void __launch_bounds__(StreamShape<NB, NBLK, S>::THREADS)
       S acc[8];
 #pragma unroll
       for (int t = 0; t < 8; ++t) acc[t] = S(0);
-      if (NBLK == 4 || NBLK == 3) {
+      if (NBLK == 4) {
         const int slot = (li * NBLK + g) % R;
         if (pres[slot]) {
           const S* Bs = ring + (size_t)slot * UNIT;
@@ -235,14 +227,7 @@ __global__ void __launch_bounds__(StreamShape<NB, NBLK, S>::THREADS)
     }
     consumer_sync(32 * CW);
     if (p < NB) {
-      S s;
-      if (NBLK == 3) {
-        // y = beta x + B x: beta = 1 gives the folded operator I + B, beta = 0 the
-        // shifted Krylov operator B
-        const S bx = red[p] + red[NB + p] + red[2 * NB + p];
-        s = beta != 0.0 ? ring[(size_t)((li * 3) % R) * UNIT + NB * NB + NB + p] + bx : bx;
-      }
-      else s = (red[p] + red[NB + p]) + (red[2 * NB + p] + red[3 * NB + p]);
+      S s = (red[p] + red[NB + p]) + (red[2 * NB + p] + red[3 * NB + p]);
       if (NBLK == 4) {
         s *= S(beta);
         if (alpha != 0.0) {
@@ -313,9 +298,8 @@ cudaError_t launch_stream_rows(const DevMesh& m, const DevTables& tb, int nb, in
                                double beta, const S* x, S* y, cudaStream_t st) {
 #define PP_ROWS(NBV)                                                                      \
   case NBV:                                                                               \
-    return nblk == 4   ? launch_rows<NBV, 4, S>(m, tb, B, alpha, beta, x, y, st)          \
-           : nblk == 3 ? launch_rows<NBV, 3, S>(m, tb, B, alpha, beta, x, y, st)          \
-                       : launch_rows<NBV, 1, S>(m, tb, B, alpha, beta, x, y, st);
+    return nblk == 4 ? launch_rows<NBV, 4, S>(m, tb, B, alpha, beta, x, y, st)            \
+                     : launch_rows<NBV, 1, S>(m, tb, B, alpha, beta, x, y, st);
   switch (nb) {
     PP_ROWS(12)
     PP_ROWS(24)
