@@ -1,8 +1,8 @@
 // Element-local quadrature kernels of the ALE DG discretization (Sec. 6):
 //  - k_residual     r(u, mu, t) of M du/dt = r (Eq. semidisc) with the CDG viscous
-//                   terms (liftings of the face jumps); with a dual-valued
-//                   frame it gives dr/ds for a motion seed s (theta, theta', h'),
-//                   the building block of dr/dmu in Eq. funcl-grad-nosens-dirk;
+//                   terms (liftings of the face jumps); with a frame that carries
+//                   derivatives it gives kappa . dr/ds for the motion seeds s (theta,
+//                   theta', h') of dr/dmu in Eq. funcl-grad-nosens-dirk;
 //  - k_jacobian     element block Jacobian dr/du (diagonal + 3 face-neighbour
 //                   blocks): exact flux derivatives at every quadrature point by
 //                   forward-mode dual numbers, contracted with the basis;
@@ -11,8 +11,7 @@
 //
 // Layouts: u[e][a][i] (nb = 4 Np doubles per element, contiguous); Jacobian
 // blocks [e][slot][col][row] (column-major nb x nb).
-#include <mutex>
-
+#include "fixed.cuh"
 #include "flux.cuh"
 #include "prof.h"
 #include "../../include/pp_prof.h"
@@ -22,9 +21,7 @@ namespace pp {
 namespace {
 
 constexpr int RES_WARPS = 4;
-constexpr int JAC_THREADS = 128;
-constexpr int NSV = 12;  // volume seeds: U (4) + grad U (8)
-constexpr int NSF = 24;  // face seeds: U-, grad U-, U+, grad U+
+constexpr int NSV = 12;  // seeds of a point: U (4) + grad U (8)
 
 template <class T>
 __device__ __forceinline__ void frame_P(const FrameT<T>& fr, const double* BinvT, T P[4]) {
@@ -114,261 +111,458 @@ __device__ __forceinline__ const double* lift_row(const DevTables& tb, int side,
   return tb.lift_f + (g * nqf + nqf - 1 - q) * nqf + nqf - 1;
 }
 
+// s + sum_t a_t b_t over N fixed-point terms, `stride` words apart in a (at most 60 per exact sum)
+template <int N>
+__device__ __forceinline__ double fix_dot(const Fix* a, const Fix* b, int ea, int eb, double s, int stride = 1) {
+  constexpr int parts = (N + 59) / 60, M = (N + parts - 1) / parts;
+  static_assert(parts == 1 || parts * M == N, "equal parts");
+#pragma unroll
+  for (int p = 0; p < parts; ++p) {
+    FixDot acc;
+    acc.clear();
+#pragma unroll(M <= 30 ? M : M % 10 == 0 ? 10 : 12)
+    for (int t = 0; t < M; ++t) acc.add(a[(p * M + t) * stride], b[p * M + t]);
+    s = acc.result(ea + eb, ea == 0x7ff || eb == 0x7ff, s);
+  }
+  return s;
+}
+
+// s - sum_t a_t b_t
+template <int N>
+__device__ __forceinline__ double fix_dot_minus(const Fix* a, const Fix* b, int ea, int eb, double s) {
+  return -fix_dot<N>(a, b, ea, eb, -s);
+}
+
+// A group's entry as a double, its exponent collected in ge; turned into fixed point after a barrier.
+__device__ __forceinline__ void fix_put(double* w, int* ge, double v) {
+  *w = v;
+  atomicMax(ge, fix_exponent(v));
+}
+__device__ __forceinline__ void fix_enc(double* w, int ge) { *reinterpret_cast<Fix*>(w) = fix_encode(*w, ge); }
+
 // ------------------------------------------------------------------------ residual
-// Warp per element.  Phase A: the jumps U_hat - U- at every face point (both traces).
-// Phase B: volume points, gradient lifted by the element's own face liftings.  Phase C:
-// face points, with the lifted gradient of the side that supplies the viscous flux.
-// Phase D: projection on the test functions.
-template <class T>
-__global__ void __launch_bounds__(RES_WARPS * 32)
+// T = double: the residual r.  T = DualV<3>: kappa . dr/ds for three motion seeds s carried by the
+// frame, summed per element (dr itself is not written).
+//
+// A CTA takes groups of elements and deals (element, point) and (element, row) tasks to its threads, so
+// that the warps are full (a warp per element leaves 44% of the lanes of the 36 + 18 points at p = 4
+// idle, and a warp instruction costs the FP64 pipe the same whatever its active lanes).  Bound:
+// FP64 issue.  The interpolations and the projection on the test functions run on the integer pipe
+// (fixed.cuh); what remains in FP64 are the fluxes.
+// Phases: A jumps U_hat - U- at the face points; B volume points with the element's own liftings;
+// C face points with the lifted gradient of the side that supplies the viscous flux; D projection.
+template <int PD, class T>
+struct Res {
+  static constexpr int NP = (PD + 1) * (PD + 2) / 2, NB = 4 * NP, NF = PD + 2, NV = NF * NF, F3 = 3 * NF;
+  static constexpr bool VAL = sizeof(T) == sizeof(double);
+  static constexpr int NC = VAL ? 1 : 3;                      // components projected
+  static constexpr int W = sizeof(T) / sizeof(double);
+  static constexpr int THREADS = VAL ? 256 : 128;
+  static constexpr int EB = THREADS / NV;                     // most elements of a group
+  static constexpr int LP = NP | 1;                           // odd table rows: no bank conflicts
+  // shared memory in 8-byte words: tables, then per element
+  static constexpr int pv = 0, dv = pv + NV * LP, pf = dv + 2 * NV * LP, df = pf + F3 * LP, elems = df + 2 * F3 * LP;
+  static constexpr int su = 0, Uf = su + 4 * NB, Js = Uf + F3 * 8, G = Js + F3 * 4 * W, H = G + NC * 4 * 2 * NV,
+                       per = (H + NC * 4 * F3) | 1;
+  static constexpr int words = elems + EB * per;
+};
+template <int PD, class T>
+struct ResExp {
+  using L = Res<PD, T>;
+  int tab[4];
+  int u[L::EB][4][4], G[L::EB][L::NC][4], H[L::EB][L::NC][4];
+};
+
+__device__ __forceinline__ double part(double a, int) { return a; }
+__device__ __forceinline__ double part(const DualV<3>& a, int k) { return a.d[k]; }
+
+template <int PD, class T>
+__global__ void __launch_bounds__(Res<PD, T>::THREADS, 2)
     k_residual(DevMesh m, DevTables tb, Phys ph, FrameT<T> fr, const double* __restrict__ u,
-               double* __restrict__ rval, double* __restrict__ rder) {
-  constexpr int W = sizeof(T) / sizeof(double);
-  __shared__ double s_u[RES_WARPS][4 * kMaxNb];
-  __shared__ double s_G[RES_WARPS][kMaxQv * 8 * W];
-  __shared__ double s_H[RES_WARPS][3 * kMaxQf * 4 * W];
-  __shared__ double s_J[RES_WARPS][3 * kMaxQf * 4 * W];
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int e = blockIdx.x * RES_WARPS + warp;
-  if (e >= m.ne) return;
-  const int Np = tb.Np, nb = tb.nb, nqv = tb.nqv, nqf = tb.nqf;
-  double* su = s_u[warp];
-  T* G = reinterpret_cast<T*>(s_G[warp]);
-  T* Hs = reinterpret_cast<T*>(s_H[warp]);
-  T* Js = reinterpret_cast<T*>(s_J[warp]);
-
-  for (int idx = lane; idx < 4 * nb; idx += 32) {
-    int slot = idx / nb, k = idx - slot * nb;
-    int src = e;
-    if (slot > 0) {
-      int nn = m.nbr[3 * e + slot - 1];
-      src = nn >= 0 ? nn : e;
+               const double* __restrict__ kappa, double* __restrict__ out, int eb) {
+  using L = Res<PD, T>;
+  constexpr int NP = L::NP, NB = L::NB, NF = L::NF, NV = L::NV, F3 = L::F3, NT = L::THREADS, NC = L::NC, LP = L::LP;
+  extern __shared__ double smem[];
+  __shared__ ResExp<PD, T> ex;
+  const int tid = threadIdx.x;
+  // tables, one exponent each
+  if (tid < 4) ex.tab[tid] = 0;
+  __syncthreads();
+  auto each_table = [&](auto&& f) {
+    for (int i = tid; i < NV * NP; i += NT) {
+      const int q = i / NP, j = i - q * NP;
+      f(smem + L::pv + q * LP + j, &ex.tab[0], tb.phi_v + i);
+      f(smem + L::dv + q * LP + j, &ex.tab[1], tb.dphi_v + 2 * i);
+      f(smem + L::dv + (NV + q) * LP + j, &ex.tab[1], tb.dphi_v + 2 * i + 1);
     }
-    su[idx] = u[(size_t)src * nb + k];
-  }
-  __syncwarp();
-
-  T P[4];
-  frame_P(fr, m.BinvT + 4 * e, P);
-  const double detB = m.detB[e];
-  T nf[3][2];
-#pragma unroll
-  for (int f = 0; f < 3; ++f) rotate_normal(fr, m.N + 6 * e + 2 * f, nf[f]);
-
-  // phase A: jumps
-  for (int idx = lane; idx < 3 * nqf; idx += 32) {
-    const int f = idx / nqf, q = idx - f * nqf;
-    const int tag = m.tag[3 * e + f];
-    double um[4], up[4];
-    interp_val(su, Np, tb.phi_f + (f * nqf + q) * Np, um);
-    if (tag == 0) {
-      const int g = m.nbrface[3 * e + f], qq = nqf - 1 - q;
-      interp_val(su + (1 + f) * nb, Np, tb.phi_f + (g * nqf + qq) * Np, up);
-    } else {
-#pragma unroll
-      for (int a = 0; a < 4; ++a) up[a] = um[a];
+    for (int i = tid; i < F3 * NP; i += NT) {
+      const int q = i / NP, j = i - q * NP;
+      f(smem + L::pf + q * LP + j, &ex.tab[2], tb.phi_f + i);
+      f(smem + L::df + q * LP + j, &ex.tab[3], tb.dphi_f + 2 * i);
+      f(smem + L::df + (F3 + q) * LP + j, &ex.tab[3], tb.dphi_f + 2 * i + 1);
     }
-    T Um[4], Up[4], vG[2], Uh[4];
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      Um[a] = T(um[a]);
-      Up[a] = T(up[a]);
-    }
-    double X, Y;
-    ref_to_X(m, e, tb.xi_f[2 * (f * nqf + q)], tb.xi_f[2 * (f * nqf + q) + 1], X, Y);
-    mesh_velocity(fr, ph, X, Y, vG);
-    face_value(tag, Um, Up, vG, ph, Uh);
-#pragma unroll
-    for (int a = 0; a < 4; ++a) Js[(f * kMaxQf + q) * 4 + a] = Uh[a] - Um[a];
-  }
-  __syncwarp();
+  };
+  each_table([](double* w, int* ge, const double* v) { fix_put(w, ge, *v); });
+  __syncthreads();
+  each_table([](double* w, int* ge, const double*) { fix_enc(w, *ge); });
+  auto fix = [&](int off) { return reinterpret_cast<const Fix*>(smem + off); };
 
-  // phase B: volume points
-  for (int q = lane; q < nqv; q += 32) {
-    T U[4], dU[4][2], vG[2], F[4][2];
-    interp(su, Np, tb.phi_v + q * Np, tb.dphi_v + 2 * q * Np, P, U, dU);
-#pragma unroll
-    for (int f = 0; f < 3; ++f)
-      if (m.side[3 * e + f])
-        lift_add(dU, nf[f], m.s_own[3 * e + f], tb.lift_v + (f * nqv + q) * nqf, 1, Js + f * kMaxQf * 4, nqf);
-    double X, Y;
-    ref_to_X(m, e, tb.xi_v[2 * q], tb.xi_v[2 * q + 1], X, Y);
-    mesh_velocity(fr, ph, X, Y, vG);
-    volume_flux(U, dU, vG, ph, F);
-    double wq = tb.w_v[q] * detB;
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      G[(q * 4 + a) * 2 + 0] = wq * (P[0] * F[a][0] + P[2] * F[a][1]);
-      G[(q * 4 + a) * 2 + 1] = wq * (P[1] * F[a][0] + P[3] * F[a][1]);
+  for (int e0 = blockIdx.x * eb; e0 < m.ne; e0 += gridDim.x * eb) {
+    const int n = min(eb, m.ne - e0);
+    __syncthreads();
+    for (int k = tid; k < (int)((sizeof(ex.u) + sizeof(ex.G) + sizeof(ex.H)) / 4); k += NT) (&ex.u[0][0][0])[k] = 0;
+    __syncthreads();
+    for (int idx = tid; idx < n * 4 * NB; idx += NT) {
+      const int el = idx / (4 * NB), r = idx - el * 4 * NB, slot = r / NB, k = r - slot * NB;
+      int src = e0 + el;
+      if (slot > 0) {
+        const int nn = m.nbr[3 * src + slot - 1];
+        src = nn >= 0 ? nn : src;
+      }
+      fix_put(smem + L::elems + el * L::per + L::su + r, &ex.u[el][slot][k / NP], u[(size_t)src * NB + k]);
     }
-  }
-  // phase C: face points
-  for (int idx = lane; idx < 3 * nqf; idx += 32) {
-    const int f = idx / nqf, q = idx - f * nqf;
-    const int tag = m.tag[3 * e + f], side = m.side[3 * e + f];
-    T Um[4], dUm[4][2], Up[4], dUp[4][2], vG[2], H[4];
-    interp(su, Np, tb.phi_f + (f * nqf + q) * Np, tb.dphi_f + 2 * (f * nqf + q) * Np, P, Um, dUm);
-    int g = 0;
-    if (tag == 0) {
-      const int e2 = m.nbr[3 * e + f], qq = nqf - 1 - q;
-      g = m.nbrface[3 * e + f];
-      T P2[4];
-      frame_P(fr, m.BinvT + 4 * e2, P2);
-      interp(su + (1 + f) * nb, Np, tb.phi_f + (g * nqf + qq) * Np, tb.dphi_f + 2 * (g * nqf + qq) * Np, P2, Up,
-             dUp);
-    } else {
+    __syncthreads();
+    for (int idx = tid; idx < n * 4 * NB; idx += NT) {
+      const int el = idx / (4 * NB), r = idx - el * 4 * NB, slot = r / NB, k = r - slot * NB;
+      fix_enc(smem + L::elems + el * L::per + L::su + r, ex.u[el][slot][k / NP]);
+    }
+    __syncthreads();
+    // phase A: both traces and the jumps
+    for (int task = tid; task < n * F3; task += NT) {
+      const int el = task / F3, fq = task - el * F3, f = fq / NF, q = fq - f * NF, e = e0 + el;
+      double* const S = smem + L::elems + el * L::per;
+      const Fix* su = reinterpret_cast<const Fix*>(S + L::su);
+      const int tag = m.tag[3 * e + f];
+      const int fn = tag == 0 ? m.nbrface[3 * e + f] * NF + NF - 1 - q : fq;
+      const int sn = tag == 0 ? 1 + f : 0;
+      T Um[4], Up[4], vG[2], Uh[4];
 #pragma unroll
       for (int a = 0; a < 4; ++a) {
-        Up[a] = Um[a];
-        dUp[a][0] = dUm[a][0];
-        dUp[a][1] = dUm[a][1];
+        const double um = fix_dot<NP>(fix(L::pf) + fq * LP, su + a * NP, ex.tab[2], ex.u[el][0][a], 0.0);
+        const double up = tag == 0 ? fix_dot<NP>(fix(L::pf) + fn * LP, su + sn * NB + a * NP, ex.tab[2], ex.u[el][sn][a], 0.0) : um;
+        S[L::Uf + fq * 8 + a] = um;
+        S[L::Uf + fq * 8 + 4 + a] = up;
+        Um[a] = T(um);
+        Up[a] = T(up);
+      }
+      double X, Y;
+      ref_to_X(m, e, tb.xi_f[2 * fq], tb.xi_f[2 * fq + 1], X, Y);
+      mesh_velocity(fr, ph, X, Y, vG);
+      face_value(tag, Um, Up, vG, ph, Uh);
+      T* Js = reinterpret_cast<T*>(S + L::Js);
+#pragma unroll
+      for (int a = 0; a < 4; ++a) Js[fq * 4 + a] = Uh[a] - Um[a];
+    }
+    __syncthreads();
+    // phases B and C: volume points, then face points from the next full warp on
+    const int nvol = (n * NV + 31) / 32 * 32;
+    for (int task = tid; task < nvol + n * F3; task += NT) {
+      if (task < nvol) {
+        if (task >= n * NV) continue;
+        const int el = task / NV, q = task - el * NV, e = e0 + el;
+        double* const S = smem + L::elems + el * L::per;
+        const Fix* su = reinterpret_cast<const Fix*>(S + L::su);
+        const T* Js = reinterpret_cast<const T*>(S + L::Js);
+        T P[4], U[4], dU[4][2], vG[2], F[4][2];
+        frame_P(fr, m.BinvT + 4 * e, P);
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+          const int eu = ex.u[el][0][a];
+          U[a] = T(fix_dot<NP>(fix(L::pv) + q * LP, su + a * NP, ex.tab[0], eu, 0.0));
+          const double s0 = fix_dot<NP>(fix(L::dv) + q * LP, su + a * NP, ex.tab[1], eu, 0.0);
+          const double s1 = fix_dot<NP>(fix(L::dv) + (NV + q) * LP, su + a * NP, ex.tab[1], eu, 0.0);
+          dU[a][0] = P[0] * s0 + P[1] * s1;
+          dU[a][1] = P[2] * s0 + P[3] * s1;
+        }
+        for (int f = 0; f < 3; ++f)
+          if (m.side[3 * e + f]) {
+            T nf[2];
+            rotate_normal(fr, m.N + 6 * e + 2 * f, nf);
+            lift_add(dU, nf, m.s_own[3 * e + f], tb.lift_v + (f * NV + q) * NF, 1, Js + f * NF * 4, NF);
+          }
+        double X, Y;
+        ref_to_X(m, e, tb.xi_v[2 * q], tb.xi_v[2 * q + 1], X, Y);
+        mesh_velocity(fr, ph, X, Y, vG);
+        volume_flux(U, dU, vG, ph, F);
+        const double wq = tb.w_v[q] * m.detB[e];
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+          const T g0 = wq * (P[0] * F[a][0] + P[2] * F[a][1]), g1 = wq * (P[1] * F[a][0] + P[3] * F[a][1]);
+#pragma unroll
+          for (int c = 0; c < NC; ++c) {
+            double* G = S + L::G + (c * 4 + a) * 2 * NV;
+            fix_put(G + q, &ex.G[el][c][a], part(g0, c));
+            fix_put(G + NV + q, &ex.G[el][c][a], part(g1, c));
+          }
+        }
+      } else {
+        const int t2 = task - nvol, el = t2 / F3, fq = t2 - el * F3, f = fq / NF, q = fq - f * NF, e = e0 + el;
+        double* const S = smem + L::elems + el * L::per;
+        const Fix* su = reinterpret_cast<const Fix*>(S + L::su);
+        const T* Js = reinterpret_cast<const T*>(S + L::Js);
+        const int tag = m.tag[3 * e + f], side = m.side[3 * e + f];
+        // the gradient of the side that supplies the viscous flux
+        const int g = tag == 0 ? m.nbrface[3 * e + f] : 0;
+        const int slot = side ? 0 : 1 + f, fs = side ? fq : g * NF + NF - 1 - q, es = side ? e : m.nbr[3 * e + f];
+        T P[4], Um[4], Up[4], QS[4][2], n2[2], vG[2], H[4];
+        frame_P(fr, m.BinvT + 4 * es, P);
+#pragma unroll
+        for (int a = 0; a < 4; ++a) {
+          const Fix* ua = su + slot * NB + a * NP;
+          const double s0 = fix_dot<NP>(fix(L::df) + fs * LP, ua, ex.tab[3], ex.u[el][slot][a], 0.0);
+          const double s1 = fix_dot<NP>(fix(L::df) + (F3 + fs) * LP, ua, ex.tab[3], ex.u[el][slot][a], 0.0);
+          QS[a][0] = P[0] * s0 + P[1] * s1;
+          QS[a][1] = P[2] * s0 + P[3] * s1;
+          Um[a] = T(S[L::Uf + fq * 8 + a]);
+          Up[a] = T(S[L::Uf + fq * 8 + 4 + a]);
+        }
+        rotate_normal(fr, m.N + 6 * e + 2 * f, n2);
+        int step;
+        const double* A = lift_row(tb, side, f, g, q, step);
+        lift_add(QS, n2, side ? m.s_own[3 * e + f] : m.s_nbr[3 * e + f], A, step, Js + f * NF * 4, NF);
+        double X, Y;
+        ref_to_X(m, e, tb.xi_f[2 * fq], tb.xi_f[2 * fq + 1], X, Y);
+        mesh_velocity(fr, ph, X, Y, vG);
+        face_flux(tag, side, Um, Up, QS, n2, vG, m.c11[3 * e + f], ph, H);
+        const double wl = tb.w_f[q] * m.L[3 * e + f];
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+          for (int c = 0; c < NC; ++c)
+            fix_put(S + L::H + (c * 4 + a) * F3 + fq, &ex.H[el][c][a], wl * part(H[a], c));
       }
     }
-    T QS[4][2];
-#pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      QS[a][0] = side ? dUm[a][0] : dUp[a][0];
-      QS[a][1] = side ? dUm[a][1] : dUp[a][1];
+    __syncthreads();
+    for (int idx = tid; idx < n * NC * 4 * (2 * NV + F3); idx += NT) {
+      const int el = idx / (NC * 4 * (2 * NV + F3)), r = idx - el * NC * 4 * (2 * NV + F3), ca = r / (2 * NV + F3),
+                t = r - ca * (2 * NV + F3);
+      double* const S = smem + L::elems + el * L::per;
+      if (t < 2 * NV) fix_enc(S + L::G + ca * 2 * NV + t, (&ex.G[el][0][0])[ca]);
+      else fix_enc(S + L::H + ca * F3 + t - 2 * NV, (&ex.H[el][0][0])[ca]);
     }
-    int step;
-    const double* A = lift_row(tb, side, f, g, q, step);
-    lift_add(QS, nf[f], side ? m.s_own[3 * e + f] : m.s_nbr[3 * e + f], A, step, Js + f * kMaxQf * 4, nqf);
-    double X, Y;
-    ref_to_X(m, e, tb.xi_f[2 * (f * nqf + q)], tb.xi_f[2 * (f * nqf + q) + 1], X, Y);
-    mesh_velocity(fr, ph, X, Y, vG);
-    face_flux(tag, side, Um, Up, QS, nf[f], vG, m.c11[3 * e + f], ph, H);
-    double wl = tb.w_f[q] * m.L[3 * e + f];
+    __syncthreads();
+    // phase D
+    for (int idx = tid; idx < n * NB; idx += NT) {
+      const int el = idx / NB, o = idx - el * NB, a = o / NP, i = o - a * NP;
+      double* const S = smem + L::elems + el * L::per;
+      double acc[NC];
 #pragma unroll
-    for (int a = 0; a < 4; ++a) Hs[(f * kMaxQf + q) * 4 + a] = wl * H[a];
-  }
-  __syncwarp();
-  for (int o = lane; o < nb; o += 32) {
-    int a = o / Np, i = o - a * Np;
-    T acc(0.0);
-    for (int q = 0; q < nqv; ++q) {
-      const double* d = tb.dphi_v + 2 * (q * Np + i);
-      acc += d[0] * G[(q * 4 + a) * 2] + d[1] * G[(q * 4 + a) * 2 + 1];
+      for (int c = 0; c < NC; ++c) {
+        const Fix* G = reinterpret_cast<const Fix*>(S + L::G) + (c * 4 + a) * 2 * NV;
+        const Fix* H = reinterpret_cast<const Fix*>(S + L::H) + (c * 4 + a) * F3;
+        acc[c] = -fix_dot<F3>(fix(L::pf) + i, H, ex.tab[2], ex.H[el][c][a], 0.0, LP);
+        acc[c] = fix_dot<2 * NV>(fix(L::dv) + i, G, ex.tab[1], ex.G[el][c][a], acc[c], LP);
+      }
+      if constexpr (L::VAL) {
+        out[(size_t)(e0 + el) * NB + o] = acc[0];
+      } else {
+        // kappa times the rows, in place of the states
+        const double kp = kappa[(size_t)(e0 + el) * NB + o];
+#pragma unroll
+        for (int c = 0; c < NC; ++c) S[L::su + c * NB + o] = kp * acc[c];
+      }
     }
-    for (int f = 0; f < 3; ++f)
-      for (int q = 0; q < nqf; ++q) acc -= tb.phi_f[(f * nqf + q) * Np + i] * Hs[(f * kMaxQf + q) * 4 + a];
-    if (rval) rval[(size_t)e * nb + o] = val(acc);
-    if (rder) rder[(size_t)e * nb + o] = der(acc);
+    if constexpr (!L::VAL) {
+      __syncthreads();
+      // eight lanes per (element, seed), then a butterfly over them
+      const int l = tid & 7;
+      for (int g8 = tid >> 3; g8 < (n * NC + 3) / 4 * 4; g8 += NT / 8) {
+        const int el = g8 / NC, c = g8 - el * NC;
+        double s = 0.0;
+        if (el < n)
+          for (int o = l; o < NB; o += 8) s += smem[L::elems + el * L::per + L::su + c * NB + o];
+#pragma unroll
+        for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if (l == 0 && el < n) out[(size_t)(e0 + el) * NC + c] = s;
+      }
+    }
   }
 }
 
 // ------------------------------------------------------------------------ Jacobian
-// Shared-memory carve-up of k_jacobian (doubles), sized from the runtime degree.
-struct JacSmem {
-  int su, SV, SF, Cv, Cf, Tv, Tf, Tn, Wv, Wf, Wn, Js, Gb, cv, cf, Y, Lam, LamW, total;
-  __host__ __device__ JacSmem(int nb, int Np, int nqv) {
-    su = 0;
-    SV = su + 4 * nb;                 // [q][12]: U, lifted grad U at the volume points
-    SF = SV + nqv * 12;               // [side][f][q][12]: both traces (flux side: lifted gradient)
-    Cv = SF + 2 * 3 * kMaxQf * 12;
-    Cf = Cv + nqv * 4 * 2 * NSV;
-    Tv = Cf + 3 * kMaxQf * 4 * NSF;
-    Tf = Tv + nqv * 3 * Np;
-    Tn = Tf + 3 * kMaxQf * 3 * Np;
-    Wv = Tn + 3 * kMaxQf * 3 * Np;
-    Wf = Wv + nqv * 2 * Np;
-    Wn = Wf + 3 * kMaxQf * Np;
-    Js = Wn + 3 * kMaxQf * Np;        // [f][q][4] jumps U_hat - U-
-    Gb = Js + 3 * kMaxQf * 4;         // [f][q][4][4] d U_wall / d U- at wall points
-    cv = Gb + 3 * kMaxQf * 16;        // [f][q][k] per pair: volume gradient coefficients along n_f
-    cf = cv + 3 * nqv * 2;            // [f][q]    per pair: face gradient coefficients along n_f
-    Y = cf + 3 * kMaxQf;              // [f][i][q] per pair: cv contracted with the test gradients
-    Lam = Y + 3 * Np * nqv;           // [f][i][p] per pair: d r_(a,i) / d jump_(f,b)(p)
-    LamW = Lam + 3 * Np * kMaxQf;     // [f][b][i][p] Lam of wall faces for every b of the row a
-    total = LamW + 3 * 4 * Np * kMaxQf;
-  }
+// Element block Jacobian dr/du, one CTA per element, templated on the degree.
+//
+// Phase 0: U and grad U at every point (both traces on faces), the face jumps U_hat - U- and, at
+// wall points, d U_wall / d U-; then the CDG liftings: the volume gradients and the flux side's
+// face gradients become the lifted ones.
+// Phase 1: exact derivatives of the quadrature-point fluxes with respect to (U, lifted grad U),
+// weighted and projected on the reference gradients of test and trial functions: state seeds by
+// forward-mode derivatives (one thread carries 4 seeds of a volume point, 2 of a face point, so
+// that the value part with its divisions and roots is shared), gradient seeds in closed form (the
+// viscous flux is linear in the gradient at fixed U).
+// Phase 2, per row variable a and column variables b: W = C T over the trial functions,
+// J_ab = D W, plus the liftings' chain: Lam = d r_a / d jump_b at the face points (through the
+// volume and the face gradients), contracted with d jump / d u (-phi of this element, +phi of the
+// neighbour; at wall points d U_wall / d U- couples b to every variable, added per row a).  The
+// mass equation has no viscous flux and the momentum equations none from grad(rho E): those pairs
+// have no gradient part and no liftings.
+//
+// Bound: FP64 issue (one warp instruction per 19 clocks and SM).  The contractions (D W, Lam, the
+// lifting chain: 260,000 multiply-adds per element at p = 3) run on the integer pipe (fixed.cuh):
+// factors are written as doubles with the largest exponent of their group, encoded in place, and a
+// sum costs two FP64 instructions instead of one per term.
+template <int PD>
+struct Jac {
+  static constexpr int NP = (PD + 1) * (PD + 2) / 2, NB = 4 * NP, NF = PD + 2, NV = NF * NF, F3 = 3 * NF;
+  static constexpr int T = 256;              // threads
+  static constexpr int NBV = PD <= 3 ? 2 : 1;  // column variables at a time
+  // term strides, odd: lanes over rows read different banks
+  static constexpr int LV = 2 * NV + 1, LF = F3 | 1, LY = NV | 1;
+  // shared memory in 8-byte words
+  static constexpr int su = 0;
+  static constexpr int SV = su + 4 * NB;               // [q][12]: U, lifted grad U at the volume points
+  static constexpr int SF = SV + NV * 12;              // [side][f][q][12]: both traces (flux side: lifted gradient)
+  static constexpr int Cv = SF + 2 * F3 * 12;          // [q][a][k][12]
+  static constexpr int Cf = Cv + NV * 8 * 12;          // [f][q][a][16]: U- | U+ | gradient of the flux side
+  static constexpr int Js = Cf + F3 * 4 * 16;          // [f][q][4] jumps
+  static constexpr int Gb = Js + F3 * 4;               // [f][q][4][4] d U_wall / d U- at wall points
+  static constexpr int dV = Gb + F3 * 16;              // [i][LV] test gradients (k, q)
+  static constexpr int pF = dV + NP * LV;              // [i][LF] own face basis values
+  static constexpr int pN = pF + NP * LF;              // [j][LF] the neighbours' at the matched points
+  static constexpr int lv = pN + NP * LF;              // [f][p][LY] lifting at the volume points
+  static constexpr int Wv = lv + F3 * LY;              // [b][j][LV]
+  static constexpr int Wf = Wv + NBV * NP * LV;        // [b][j][LF]
+  static constexpr int Wn = Wf + NBV * NP * LF;        // [b][j][LF]
+  static constexpr int cv = Wn + NBV * NP * LF;        // [b][f][q][2] gradient coefficients along n_f
+  static constexpr int cf = cv + NBV * 3 * NV * 2;     // [b][f][q]
+  static constexpr int Y = cf + NBV * F3;              // [b][f][i][LY] cv contracted with the test gradients
+  static constexpr int Lam = Y + NBV * 3 * NP * LY;    // [b][i][LF] d r_(a,i) / d jump_(f,b)(p)
+  static constexpr int LamW = Lam + NBV * NP * LF;     // [f][b][i][NF] of the wall faces, doubles
+  static constexpr int words = LamW + 3 * 4 * NP * NF;
+};
+// exponents of the groups
+template <int PD>
+struct JacExp {
+  using L = Jac<PD>;
+  int dV[L::NP], pF[L::NP], pN[L::NP], lv[L::F3];
+  int Wv[L::NBV][L::NP], Wf[L::NBV][L::NP], Wn[L::NBV][3][L::NP], Y[L::NBV][3][L::NP], Lam[L::NBV][L::NP];
 };
 
-// Element block Jacobian.  Phase 0: U and grad U at every point (both traces on faces), the
-// face jumps U_hat - U- and, at wall points, d U_wall / d U-; then the CDG liftings: the
-// volume gradients and the flux side's face gradients become the lifted ones.  Phase 1:
-// exact derivatives of the quadrature-point fluxes with respect to (U, lifted grad U) by
-// dual numbers (state seeds) and by linearity (gradient seeds: the viscous flux is linear
-// in the gradient at fixed U), weighted and projected on the reference test gradients (C).
-// Phase 2, per variable pair (a, b): W = C T over the trial tables, J_ab = D W, plus the
-// liftings' chain: Lam = d r_a / d jump_b at the face points (through the volume and the
-// face gradients), contracted with d jump / d u (-phi of this element, +phi of the
-// neighbour; at wall points d U_wall / d U- couples b to every variable, added per row a).
-__global__ void __launch_bounds__(JAC_THREADS)
+// per-face data of one element
+struct JacFaces {
+  double P[4], nf[3][2], Pn[3][4], s_lift[3];
+  double nuo[3][2], nus[3][2];  // P^-1 n of this element and of the flux side
+  int side[3], tag[3], g[3];
+};
+
+// viscous flux derivative for the unit gradient of variable b along d: F[a - 1][dir], a = 1 .. 3
+__device__ __forceinline__ void viscous_seed(int b, int d, double u, double v, double E, double ir, double mu, double kq,
+                                             double F[3][2]) {
+  const double du = b == 0 ? -u * ir : b == 1 ? ir : 0.0;
+  const double dv = b == 0 ? -v * ir : b == 2 ? ir : 0.0;
+  const double dE = b == 0 ? -E * ir : b == 3 ? ir : 0.0;
+  const double q = kq * (dE - u * du - v * dv);
+  // along x: div = du, shear = dv; along y: div = dv, shear = du
+  const double nrm = mu * (d == 0 ? du : dv), sh = mu * (d == 0 ? dv : du);
+  const double txx = d == 0 ? (4.0 / 3.0) * nrm : (-2.0 / 3.0) * nrm;
+  const double tyy = d == 0 ? (-2.0 / 3.0) * nrm : (4.0 / 3.0) * nrm;
+  F[0][0] = txx;
+  F[0][1] = sh;
+  F[1][0] = sh;
+  F[1][1] = tyy;
+  F[2][0] = u * txx + v * sh + (d == 0 ? q : 0.0);
+  F[2][1] = u * sh + v * tyy + (d == 1 ? q : 0.0);
+}
+
+template <int PD>
+__global__ void __launch_bounds__(Jac<PD>::T, 2)
     k_jacobian(DevMesh m, DevTables tb, Phys ph, FrameT<double> fr, const double* __restrict__ u,
                double* __restrict__ J) {
+  using L = Jac<PD>;
+  constexpr int NP = L::NP, NB = L::NB, NF = L::NF, NV = L::NV, F3 = L::F3, T = L::T, NBV = L::NBV;
+  constexpr int LV = L::LV, LF = L::LF, LY = L::LY;
   extern __shared__ double smem[];
-  const int e = blockIdx.x;
-  const int tid = threadIdx.x;
-  const int Np = tb.Np, nb = tb.nb, nqv = tb.nqv, nqf = tb.nqf;
-  const JacSmem L(nb, Np, nqv);
-  double* su = smem + L.su;
-  double* Cv = smem + L.Cv;
-  double* Cf = smem + L.Cf;
-  double* Tv = smem + L.Tv;  // [q][t][j]
-  double* Tf = smem + L.Tf;  // [f][q][t][j] (own trace)
-  double* Tn = smem + L.Tn;  // [f][q][t][j] (neighbour trace at the matched point)
-  double* Wv = smem + L.Wv;  // [q][k][j]
-  double* Wf = smem + L.Wf;  // [f][q][j]
-  double* Wn = smem + L.Wn;  // [f][q][j]
-  double* Js = smem + L.Js;
-  double* Gb = smem + L.Gb;
-  double* cvv = smem + L.cv;
-  double* cff = smem + L.cf;
-  double* Yv = smem + L.Y;
-  double* Lam = smem + L.Lam;
-  double* LamW = smem + L.LamW;
-  for (int idx = tid; idx < 4 * nb; idx += JAC_THREADS) {
-    int slot = idx / nb, k = idx - slot * nb;
+  __shared__ JacExp<PD> ex;
+  const int e = blockIdx.x, tid = threadIdx.x;
+  double* const su = smem + L::su;
+  double* const SV = smem + L::SV;
+  double* const SF = smem + L::SF;
+  double* const Cv = smem + L::Cv;
+  double* const Cf = smem + L::Cf;
+  double* const Js = smem + L::Js;
+  double* const Gb = smem + L::Gb;
+  double* const cvv = smem + L::cv;
+  double* const cff = smem + L::cf;
+  double* const LamW = smem + L::LamW;
+  auto put = [](double* w, int* ge, double v) { fix_put(w, ge, v); };
+  auto enc = [](double* w, int ge) { fix_enc(w, ge); };
+  auto fix = [&](int off) { return reinterpret_cast<const Fix*>(smem + off); };
+
+  for (int k = tid; k < (int)(sizeof(ex) / sizeof(int)); k += T) reinterpret_cast<int*>(&ex)[k] = 0;
+  for (int idx = tid; idx < 4 * NB; idx += T) {
+    int slot = idx / NB, k = idx - slot * NB;
     int src = e;
     if (slot > 0) {
       int nn = m.nbr[3 * e + slot - 1];
       src = nn >= 0 ? nn : e;
     }
-    su[idx] = u[(size_t)src * nb + k];
+    su[idx] = u[(size_t)src * NB + k];
   }
-  __syncthreads();
-  double P[4];
-  frame_P(fr, m.BinvT + 4 * e, P);
+  __shared__ JacFaces fc;
+  double(&P)[4] = fc.P;
+  double(&nf)[3][2] = fc.nf;
+  double(&Pn)[3][4] = fc.Pn;
+  double(&nuo)[3][2] = fc.nuo;
+  double(&nus)[3][2] = fc.nus;
+  double(&s_lift)[3] = fc.s_lift;
+  int(&sidef)[3] = fc.side;
+  int(&tagf)[3] = fc.tag;
+  int(&gf)[3] = fc.g;
+  if (tid < 3) {
+    const int f = tid;
+    double Po[4], Pf[4], n[2];
+    frame_P(fr, m.BinvT + 4 * e, Po);
+    rotate_normal(fr, m.N + 6 * e + 2 * f, n);
+    const int side = m.side[3 * e + f], tag = m.tag[3 * e + f];
+    frame_P(fr, m.BinvT + 4 * (tag == 0 ? m.nbr[3 * e + f] : e), Pf);
+    sidef[f] = side;
+    tagf[f] = tag;
+    gf[f] = tag == 0 ? m.nbrface[3 * e + f] : 0;
+    s_lift[f] = side ? m.s_own[3 * e + f] : m.s_nbr[3 * e + f];
+    const double io = 1.0 / (Po[0] * Po[3] - Po[1] * Po[2]), in = 1.0 / (Pf[0] * Pf[3] - Pf[1] * Pf[2]);
+    nuo[f][0] = (Po[3] * n[0] - Po[1] * n[1]) * io;
+    nuo[f][1] = (Po[0] * n[1] - Po[2] * n[0]) * io;
+    nus[f][0] = side ? nuo[f][0] : (Pf[3] * n[0] - Pf[1] * n[1]) * in;
+    nus[f][1] = side ? nuo[f][1] : (Pf[0] * n[1] - Pf[2] * n[0]) * in;
+    for (int k = 0; k < 2; ++k) nf[f][k] = n[k];
+    for (int k = 0; k < 4; ++k) {
+      Pn[f][k] = Pf[k];
+      if (f == 0) P[k] = Po[k];
+    }
+  }
   const double detB = m.detB[e];
-  FrameT<Dual> frd;
-#pragma unroll
-  for (int k = 0; k < 4; ++k) {
-    frd.Q[k] = Dual(fr.Q[k]);
-    frd.Qd[k] = Dual(fr.Qd[k]);
-  }
-  frd.hd = Dual(fr.hd);
-  double nf[3][2];
-  int sidef[3], tagf[3], gf[3];
-  double s_lift[3];
-#pragma unroll
-  for (int f = 0; f < 3; ++f) {
-    rotate_normal(fr, m.N + 6 * e + 2 * f, nf[f]);
-    sidef[f] = m.side[3 * e + f];
-    tagf[f] = m.tag[3 * e + f];
-    gf[f] = tagf[f] == 0 ? m.nbrface[3 * e + f] : 0;
-    s_lift[f] = sidef[f] ? m.s_own[3 * e + f] : m.s_nbr[3 * e + f];
-  }
+  __syncthreads();
   const bool has_wall = tagf[0] == 1 || tagf[1] == 1 || tagf[2] == 1;
 
-  double* SV = smem + L.SV;
-  double* SF = smem + L.SF;
+  // reference tables, as doubles
+  for (int idx = tid; idx < NP * 2 * NV; idx += T) {
+    const int i = idx / (2 * NV), r = idx - i * 2 * NV, k = r / NV, q = r - k * NV;
+    put(smem + L::dV + i * LV + r, &ex.dV[i], tb.dphi_v[2 * (q * NP + i) + k]);
+  }
+  for (int idx = tid; idx < NP * F3; idx += T) {
+    const int i = idx / F3, fq = idx - i * F3, f = fq / NF, q = fq - f * NF;
+    put(smem + L::pF + i * LF + fq, &ex.pF[i], tb.phi_f[fq * NP + i]);
+    put(smem + L::pN + i * LF + fq, &ex.pN[i], tagf[f] == 0 ? tb.phi_f[(gf[f] * NF + NF - 1 - q) * NP + i] : 0.0);
+  }
+  for (int idx = tid; idx < F3 * NV; idx += T) {
+    const int fp = idx / NV, q = idx - fp * NV, f = fp / NF, p = fp - f * NF;
+    put(smem + L::lv + fp * LY + q, &ex.lv[fp], tb.lift_v[(f * NV + q) * NF + p]);
+  }
   // phase 0a: U and grad U at every quadrature point, once (both traces on faces)
-  for (int task = tid; task < nqv + 6 * nqf; task += JAC_THREADS) {
+  for (int task = tid; task < NV + 2 * F3; task += T) {
     double U0[4], dU0[4][2];
     double* dst;
-    if (task < nqv) {
-      interp(su, Np, tb.phi_v + task * Np, tb.dphi_v + 2 * task * Np, P, U0, dU0);
+    if (task < NV) {
+      interp(su, NP, tb.phi_v + task * NP, tb.dphi_v + 2 * task * NP, P, U0, dU0);
       dst = SV + task * 12;
     } else {
-      const int t2 = task - nqv, side = t2 / (3 * nqf), r2 = t2 - side * 3 * nqf, f = r2 / nqf, q = r2 - f * nqf;
-      dst = SF + ((side * 3 + f) * kMaxQf + q) * 12;
+      const int t2 = task - NV, side = t2 / F3, fq = t2 - side * F3, f = fq / NF, q = fq - f * NF;
+      dst = SF + (side * F3 + fq) * 12;
       if (side == 0 || tagf[f] != 0) {
-        interp(su, Np, tb.phi_f + (f * nqf + q) * Np, tb.dphi_f + 2 * (f * nqf + q) * Np, P, U0, dU0);
+        interp(su, NP, tb.phi_f + fq * NP, tb.dphi_f + 2 * fq * NP, P, U0, dU0);
       } else {
-        const int e2 = m.nbr[3 * e + f], g = gf[f], qq = nqf - 1 - q;
-        double P2[4];
-        frame_P(fr, m.BinvT + 4 * e2, P2);
-        interp(su + (1 + f) * nb, Np, tb.phi_f + (g * nqf + qq) * Np, tb.dphi_f + 2 * (g * nqf + qq) * Np, P2, U0,
+        const int g = gf[f], qq = NF - 1 - q;
+        interp(su + (1 + f) * NB, NP, tb.phi_f + (g * NF + qq) * NP, tb.dphi_f + 2 * (g * NF + qq) * NP, Pn[f], U0,
                dU0);
       }
     }
@@ -380,54 +574,57 @@ __global__ void __launch_bounds__(JAC_THREADS)
     }
   }
   __syncthreads();
-  // phase 0b: jumps, and d U_wall / d U- at wall points (4 dual seeds)
-  for (int idx = tid; idx < 3 * nqf; idx += JAC_THREADS) {
-    const int f = idx / nqf, q = idx - f * nqf;
-    const double* Sm = SF + ((0 * 3 + f) * kMaxQf + q) * 12;
-    const double* Sp = SF + ((1 * 3 + f) * kMaxQf + q) * 12;
-    double X, Y, vG[2], Uh[4];
-    ref_to_X(m, e, tb.xi_f[2 * (f * nqf + q)], tb.xi_f[2 * (f * nqf + q) + 1], X, Y);
-    mesh_velocity(fr, ph, X, Y, vG);
+  for (int idx = tid; idx < NP * 2 * NV; idx += T) enc(smem + L::dV + idx / (2 * NV) * LV + idx % (2 * NV), ex.dV[idx / (2 * NV)]);
+  for (int idx = tid; idx < NP * F3; idx += T) {
+    enc(smem + L::pF + idx / F3 * LF + idx % F3, ex.pF[idx / F3]);
+    enc(smem + L::pN + idx / F3 * LF + idx % F3, ex.pN[idx / F3]);
+  }
+  for (int idx = tid; idx < F3 * NV; idx += T) enc(smem + L::lv + idx / NV * LY + idx % NV, ex.lv[idx / NV]);
+  // phase 0b: jumps, and d U_wall / d U- at wall points
+  for (int fq = tid; fq < F3; fq += T) {
+    const int f = fq / NF;
+    const double* Sm = SF + fq * 12;
+    const double* Sp = SF + (F3 + fq) * 12;
+    double X, Yc, vG[2], Uh[4];
+    ref_to_X(m, e, tb.xi_f[2 * fq], tb.xi_f[2 * fq + 1], X, Yc);
+    mesh_velocity(fr, ph, X, Yc, vG);
     face_value(tagf[f], Sm, Sp, vG, ph, Uh);
 #pragma unroll
-    for (int a = 0; a < 4; ++a) Js[(f * kMaxQf + q) * 4 + a] = Uh[a] - Sm[a];
+    for (int a = 0; a < 4; ++a) Js[fq * 4 + a] = Uh[a] - Sm[a];
     if (tagf[f] == 1) {
-      Dual vd[2] = {Dual(vG[0]), Dual(vG[1])};
-      for (int c = 0; c < 4; ++c) {
-        Dual Ud[4], Ub[4];
+      DualV<4> Ud[4], vd[2] = {DualV<4>(vG[0]), DualV<4>(vG[1])}, Ub[4];
 #pragma unroll
-        for (int a = 0; a < 4; ++a) Ud[a] = Dual(Sm[a], a == c ? 1.0 : 0.0);
-        wall_state(Ud, vd, Ub);
-#pragma unroll
-        for (int b = 0; b < 4; ++b) Gb[((f * kMaxQf + q) * 4 + b) * 4 + c] = Ub[b].d;
+      for (int a = 0; a < 4; ++a) {
+        Ud[a] = DualV<4>(Sm[a]);
+        Ud[a].d[a] = 1.0;
       }
+      wall_state(Ud, vd, Ub);
+#pragma unroll
+      for (int b = 0; b < 4; ++b)
+#pragma unroll
+        for (int c = 0; c < 4; ++c) Gb[(fq * 4 + b) * 4 + c] = Ub[b].d[c];
     }
   }
   __syncthreads();
   // phase 0c: lifted gradients (volume points; the flux side's trace on each face)
-  for (int task = tid; task < nqv + 3 * nqf; task += JAC_THREADS) {
+  for (int task = tid; task < NV + F3; task += T) {
     double dU[4][2];
     double* dst;
-    if (task < nqv) {
+#pragma unroll
+    for (int a = 0; a < 4; ++a) {
+      dU[a][0] = 0.0;
+      dU[a][1] = 0.0;
+    }
+    if (task < NV) {
       dst = SV + task * 12;
-#pragma unroll
-      for (int a = 0; a < 4; ++a) {
-        dU[a][0] = 0.0;
-        dU[a][1] = 0.0;
-      }
       for (int f = 0; f < 3; ++f)
-        if (sidef[f]) lift_add(dU, nf[f], s_lift[f], tb.lift_v + (f * nqv + task) * nqf, 1, Js + f * kMaxQf * 4, nqf);
+        if (sidef[f]) lift_add(dU, nf[f], s_lift[f], tb.lift_v + (f * NV + task) * NF, 1, Js + f * NF * 4, NF);
     } else {
-      const int t2 = task - nqv, f = t2 / nqf, q = t2 - f * nqf;
-      dst = SF + (((sidef[f] ? 0 : 1) * 3 + f) * kMaxQf + q) * 12;
-#pragma unroll
-      for (int a = 0; a < 4; ++a) {
-        dU[a][0] = 0.0;
-        dU[a][1] = 0.0;
-      }
+      const int fq = task - NV, f = fq / NF, q = fq - f * NF;
+      dst = SF + ((sidef[f] ? 0 : F3) + fq) * 12;
       int step;
       const double* A = lift_row(tb, sidef[f], f, gf[f], q, step);
-      lift_add(dU, nf[f], s_lift[f], A, step, Js + f * kMaxQf * 4, nqf);
+      lift_add(dU, nf[f], s_lift[f], A, step, Js + f * NF * 4, NF);
     }
 #pragma unroll
     for (int a = 0; a < 4; ++a) {
@@ -437,277 +634,288 @@ __global__ void __launch_bounds__(JAC_THREADS)
   }
   __syncthreads();
 
-  // phase 1a: volume seeds.  The state seeds (4 per point) run the flux in dual numbers;
-  // the viscous flux is linear in grad U at fixed U, so the derivative for gradient seed
-  // (b, d) is the viscous flux of the unit gradient (8 per point, plain FP64).
-  for (int task = tid; task < nqv * NSV; task += JAC_THREADS) {
-    const bool dual = task < 4 * nqv;
-    const int q = dual ? task >> 2 : (task - 4 * nqv) >> 3;
-    const int s = dual ? (task & 3) : 4 + ((task - 4 * nqv) & 7);
-    const double* Sq = SV + q * 12;
-    double Fd[4][2];
-    if (dual) {
-      Dual U[4], dU[4][2], vG[2], F[4][2];
+  // phase 1.  The heavy tasks go to warps of their own: the volume points to warp 0, the face points'
+  // state seeds (two per thread) to warps 1 .. 3 and the gradient seeds to the others; which warps
+  // these are turns with the block, so that co-resident CTAs load the SM's four partitions evenly.
+  const double kq0 = ph.mu * ph.gam / ph.Pr;
+  const int warp = ((tid >> 5) + blockIdx.x) & 7, lane = tid & 31;
+  if (warp == 0) {
+    for (int q = lane; q < NV; q += 32) {
+      const double* Sq = SV + q * 12;
+      DualV<4> U[4], dU[4][2], vG[2], F[4][2];
 #pragma unroll
       for (int a = 0; a < 4; ++a) {
-        U[a] = Dual(Sq[a], s == a ? 1.0 : 0.0);
-        dU[a][0] = Dual(Sq[4 + 2 * a]);
-        dU[a][1] = Dual(Sq[5 + 2 * a]);
+        U[a] = DualV<4>(Sq[a]);
+        U[a].d[a] = 1.0;
+        dU[a][0] = DualV<4>(Sq[4 + 2 * a]);
+        dU[a][1] = DualV<4>(Sq[5 + 2 * a]);
       }
-      double X, Y;
-      ref_to_X(m, e, tb.xi_v[2 * q], tb.xi_v[2 * q + 1], X, Y);
-      mesh_velocity(frd, ph, X, Y, vG);
+      double X, Yc, vg[2];
+      ref_to_X(m, e, tb.xi_v[2 * q], tb.xi_v[2 * q + 1], X, Yc);
+      mesh_velocity(fr, ph, X, Yc, vg);
+      vG[0] = DualV<4>(vg[0]);
+      vG[1] = DualV<4>(vg[1]);
       volume_flux(U, dU, vG, ph, F);
+      const double wq = tb.w_v[q] * detB;
 #pragma unroll
-      for (int a = 0; a < 4; ++a) {
-        Fd[a][0] = F[a][0].d;
-        Fd[a][1] = F[a][1].d;
+      for (int a = 0; a < 4; ++a)
+#pragma unroll
+        for (int s = 0; s < 4; ++s) {
+          Cv[((q * 4 + a) * 2 + 0) * 12 + s] = wq * (P[0] * F[a][0].d[s] + P[2] * F[a][1].d[s]);
+          Cv[((q * 4 + a) * 2 + 1) * 12 + s] = wq * (P[1] * F[a][0].d[s] + P[3] * F[a][1].d[s]);
+        }
+    }
+  } else if (warp <= 3) {
+    // state seeds of the face points: U- (s0 = 0, 2) and U+ (s0 = 4, 6)
+    for (int task = (warp - 1) * 32 + lane; task < F3 * 4; task += 96) {
+      const int fq = task >> 2, s0 = (task & 3) * 2, f = fq / NF;
+      const int tag = tagf[f], side = sidef[f];
+      const bool plus = s0 >= 4;
+      double* out = Cf + fq * 64 + s0;
+      if (tag != 0 && plus) {
+#pragma unroll
+        for (int a = 0; a < 4; ++a) out[a * 16] = out[a * 16 + 1] = 0.0;
+        continue;
       }
-    } else {
-      double U[4], E[4][2], Fv[4][2];
+      const double* Sm = SF + fq * 12;
+      const double* Sp = SF + (F3 + fq) * 12;
+      const double* SS = side ? Sm : Sp;
+      DualV<2> Um[4], Up[4], QS[4][2], n[2], vG[2], H[4];
 #pragma unroll
       for (int a = 0; a < 4; ++a) {
-        U[a] = Sq[a];
-        E[a][0] = (s == 4 + 2 * a) ? 1.0 : 0.0;
-        E[a][1] = (s == 5 + 2 * a) ? 1.0 : 0.0;
+        Um[a] = DualV<2>(Sm[a]);
+        Up[a] = DualV<2>(Sp[a]);
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+          Um[a].d[k] = s0 + k == a ? 1.0 : 0.0;
+          Up[a].d[k] = s0 + k == 4 + a ? 1.0 : 0.0;
+        }
+        QS[a][0] = DualV<2>(SS[4 + 2 * a]);
+        QS[a][1] = DualV<2>(SS[5 + 2 * a]);
       }
-      viscous_flux(U, E, ph, false, Fv);
+      double X, Yc, vg[2];
+      ref_to_X(m, e, tb.xi_f[2 * fq], tb.xi_f[2 * fq + 1], X, Yc);
+      mesh_velocity(fr, ph, X, Yc, vg);
+#pragma unroll
+      for (int d = 0; d < 2; ++d) {
+        n[d] = DualV<2>(nf[f][d]);
+        vG[d] = DualV<2>(vg[d]);
+      }
+      face_flux(tag, side, Um, Up, QS, n, vG, m.c11[3 * e + f], ph, H);
+      const double wl = tb.w_f[fq - f * NF] * m.L[3 * e + f];
 #pragma unroll
       for (int a = 0; a < 4; ++a) {
-        Fd[a][0] = -Fv[a][0];
-        Fd[a][1] = -Fv[a][1];
+        out[a * 16] = wl * H[a].d[0];
+        out[a * 16 + 1] = wl * H[a].d[1];
       }
     }
-    const double wq = tb.w_v[q] * detB;
+  } else {
+    // gradient seeds, as coefficients of the reference gradient of the trial function
+    for (int task = (warp - 4) * 32 + lane; task < 4 * (NV + F3); task += 128) {
+      const bool vol = task < 4 * NV;
+      const int q = vol ? task >> 2 : (task - 4 * NV) >> 2, b = task & 3;
+      if (vol) {
+        const double* Sq = SV + q * 12;
+        const double ir = 1.0 / Sq[0], wq = tb.w_v[q] * detB;
+        double F[2][3][2];
 #pragma unroll
-    for (int a = 0; a < 4; ++a) {
-      Cv[((q * 4 + a) * 2 + 0) * NSV + s] = wq * (P[0] * Fd[a][0] + P[2] * Fd[a][1]);
-      Cv[((q * 4 + a) * 2 + 1) * NSV + s] = wq * (P[1] * Fd[a][0] + P[3] * Fd[a][1]);
-    }
-  }
-  // phase 1b: face seeds: both traces' states in dual numbers (U- 0..3, U+ 12..15) with the
-  // lifted gradient held fixed; the flux side's gradient by linearity (grad U- 4..11 when
-  // this element supplies the viscous flux, grad U+ 16..23 when the neighbour does)
-  for (int task = tid; task < 3 * nqf * NSF; task += JAC_THREADS) {
-    const bool dual = task < 3 * nqf * 8;
-    int f, q, s;
-    if (dual) {
-      f = task / (nqf * 8);
-      const int rem = task - f * nqf * 8;
-      q = rem >> 3;
-      const int j = rem & 7;
-      s = j < 4 ? j : 8 + j;  // 0..3 (U-), 12..15 (U+)
-    } else {
-      const int t2 = task - 3 * nqf * 8;
-      f = t2 / (nqf * 16);
-      const int rem = t2 - f * nqf * 16;
-      q = rem >> 4;
-      const int j = rem & 15;
-      s = j < 8 ? 4 + j : 8 + j;  // 4..11 (grad U-), 16..23 (grad U+)
-    }
-    const int tag = tagf[f], side = sidef[f];
-    double* out = Cf + ((f * kMaxQf + q) * 4) * NSF + s;
-    const bool grad_seed = !dual;
-    const bool plus = s >= 12;
-    if ((tag != 0 && plus) || (grad_seed && (plus ? side == 1 : side == 0))) {
+        for (int d = 0; d < 2; ++d) viscous_seed(b, d, Sq[1] * ir, Sq[2] * ir, Sq[3] * ir, ir, ph.mu, kq0, F[d]);
 #pragma unroll
-      for (int a = 0; a < 4; ++a) out[a * NSF] = 0.0;
-      continue;
-    }
-    const double* Sm = SF + ((0 * 3 + f) * kMaxQf + q) * 12;
-    const double* Sp = SF + ((1 * 3 + f) * kMaxQf + q) * 12;
-    const double* SS = side ? Sm : Sp;
-    const double wl = tb.w_f[q] * m.L[3 * e + f];
-    const double c11 = m.c11[3 * e + f];
-    if (dual) {
-      Dual Um[4], Up[4], QS[4][2], n[2], vG[2], H[4];
+        for (int a = 0; a < 4; ++a)
 #pragma unroll
-      for (int a = 0; a < 4; ++a) {
-        Um[a] = Dual(Sm[a], s == a ? 1.0 : 0.0);
-        Up[a] = Dual(Sp[a], s == 12 + a ? 1.0 : 0.0);
-        QS[a][0] = Dual(SS[4 + 2 * a]);
-        QS[a][1] = Dual(SS[5 + 2 * a]);
-      }
-      rotate_normal(frd, m.N + 6 * e + 2 * f, n);
-      double X, Y;
-      ref_to_X(m, e, tb.xi_f[2 * (f * nqf + q)], tb.xi_f[2 * (f * nqf + q) + 1], X, Y);
-      mesh_velocity(frd, ph, X, Y, vG);
-      face_flux(tag, side, Um, Up, QS, n, vG, c11, ph, H);
+          for (int k = 0; k < 2; ++k)
 #pragma unroll
-      for (int a = 0; a < 4; ++a) out[a * NSF] = wl * H[a].d;
-    } else {
-      const int sg = plus ? s - 16 : s - 4;
-      const int b = sg >> 1, d = sg & 1;
-      double U[4], E[4][2], Fv[4][2];
-#pragma unroll
-      for (int a = 0; a < 4; ++a) {
-        U[a] = SS[a];
-        E[a][0] = (a == b && d == 0) ? 1.0 : 0.0;
-        E[a][1] = (a == b && d == 1) ? 1.0 : 0.0;
-      }
-      if (tag == 1) {
-        // wall: the viscous flux is evaluated at the wall state (interior density and
-        // internal energy, wall velocity), adiabatic
-        double X, Y, vG[2], Ub[4];
-        ref_to_X(m, e, tb.xi_f[2 * (f * nqf + q)], tb.xi_f[2 * (f * nqf + q) + 1], X, Y);
-        mesh_velocity(fr, ph, X, Y, vG);
-        wall_state(U, vG, Ub);
-        viscous_flux(Ub, E, ph, true, Fv);
+            for (int l = 0; l < 2; ++l) {
+              double s = 0.0;
+              if (a > 0)
+                s = P[k] * (F[0][a - 1][0] * P[l] + F[1][a - 1][0] * P[2 + l]) +
+                    P[2 + k] * (F[0][a - 1][1] * P[l] + F[1][a - 1][1] * P[2 + l]);
+              Cv[((q * 4 + a) * 2 + k) * 12 + 4 + 2 * b + l] = -wq * s;
+            }
       } else {
-        viscous_flux(U, E, ph, false, Fv);
-      }
+        const int f = q / NF, tag = tagf[f];
+        const double* SS = SF + ((sidef[f] ? 0 : F3) + q) * 12;
+        const double* PS = sidef[f] ? P : Pn[f];
+        double U[4] = {SS[0], SS[1], SS[2], SS[3]};
+        if (tag == 1) {
+          // wall: the viscous flux is evaluated at the wall state, adiabatic
+          double X, Yc, vG[2], Ub[4];
+          ref_to_X(m, e, tb.xi_f[2 * q], tb.xi_f[2 * q + 1], X, Yc);
+          mesh_velocity(fr, ph, X, Yc, vG);
+          wall_state(U, vG, Ub);
 #pragma unroll
-      for (int a = 0; a < 4; ++a) out[a * NSF] = -wl * (Fv[a][0] * nf[f][0] + Fv[a][1] * nf[f][1]);
+          for (int a = 0; a < 4; ++a) U[a] = Ub[a];
+        }
+        const double ir = 1.0 / U[0], wl = tb.w_f[q - f * NF] * m.L[3 * e + f];
+        double F[2][3][2];
+#pragma unroll
+        for (int d = 0; d < 2; ++d)
+          viscous_seed(b, d, U[1] * ir, U[2] * ir, U[3] * ir, ir, ph.mu, tag == 1 ? 0.0 : kq0, F[d]);
+#pragma unroll
+        for (int a = 0; a < 4; ++a)
+#pragma unroll
+          for (int l = 0; l < 2; ++l) {
+            double s = 0.0;
+            if (a > 0)
+              s = (F[0][a - 1][0] * nf[f][0] + F[0][a - 1][1] * nf[f][1]) * PS[l] +
+                  (F[1][a - 1][0] * nf[f][0] + F[1][a - 1][1] * nf[f][1]) * PS[2 + l];
+            Cf[q * 64 + a * 16 + 8 + 2 * b + l] = -wl * s;
+          }
+      }
     }
   }
-  // trial tables: basis values and physical gradients at the volume / face points
-  for (int idx = tid; idx < nqv * Np; idx += JAC_THREADS) {
-    const int q = idx / Np, j = idx - q * Np;
-    const double* dj = tb.dphi_v + 2 * (q * Np + j);
-    Tv[(q * 3 + 0) * Np + j] = tb.phi_v[q * Np + j];
-    Tv[(q * 3 + 1) * Np + j] = P[0] * dj[0] + P[1] * dj[1];
-    Tv[(q * 3 + 2) * Np + j] = P[2] * dj[0] + P[3] * dj[1];
-  }
-  for (int idx = tid; idx < 3 * nqf * Np; idx += JAC_THREADS) {
-    const int f = idx / (nqf * Np), rem = idx - f * nqf * Np, q = rem / Np, j = rem - q * Np;
-    const double* dj = tb.dphi_f + 2 * ((f * nqf + q) * Np + j);
-    double* to = Tf + ((f * kMaxQf + q) * 3) * Np + j;
-    to[0] = tb.phi_f[(f * nqf + q) * Np + j];
-    to[Np] = P[0] * dj[0] + P[1] * dj[1];
-    to[2 * Np] = P[2] * dj[0] + P[3] * dj[1];
-    double* tn = Tn + ((f * kMaxQf + q) * 3) * Np + j;
-    if (tagf[f] == 0) {
-      const int e2 = m.nbr[3 * e + f], g = gf[f], qq = nqf - 1 - q;
-      double P2[4];
-      frame_P(fr, m.BinvT + 4 * e2, P2);
-      const double* dn = tb.dphi_f + 2 * ((g * nqf + qq) * Np + j);
-      tn[0] = tb.phi_f[(g * nqf + qq) * Np + j];
-      tn[Np] = P2[0] * dn[0] + P2[1] * dn[1];
-      tn[2 * Np] = P2[2] * dn[0] + P2[3] * dn[1];
-    } else {
-      tn[0] = tn[Np] = tn[2 * Np] = 0.0;
-    }
-  }
-  __syncthreads();
 
-  // phase 2: per variable pair (a, b)
-  const size_t nb2 = (size_t)nb * nb;
+  // phase 2: per row variable a and NBV column variables
+  const size_t nb2 = (size_t)NB * NB;
   double* Jd = J + (size_t)e * 4 * nb2;
-  const int nW = nqv * 2 * Np, nWf = 3 * nqf * Np;
-  for (int ab = 0; ab < 16; ++ab) {
-    const int a = ab >> 2, b = ab & 3;
-    const int sb[3] = {b, 4 + 2 * b, 5 + 2 * b};
+  auto has_grad = [](int a, int b) { return a > 0 && (a == 3 || b < 3); };
+  for (int ab = 0; ab < 16; ab += NBV) {
+    const int a = ab >> 2, b0 = ab & 3;
+    __syncthreads();
+    for (int k = tid; k < (int)(sizeof(ex.Wv) + sizeof(ex.Wf) + sizeof(ex.Wn) + sizeof(ex.Y) + sizeof(ex.Lam)) / 4; k += T)
+      (&ex.Wv[0][0])[k] = 0;
+    __syncthreads();
     // W = C T, and the gradient coefficients along each face normal for the liftings
-    for (int idx = tid; idx < nW + 2 * nWf + 3 * nqv * 2 + 3 * nqf; idx += JAC_THREADS) {
-      if (idx < nW) {
-        const int q = idx / (2 * Np), rem = idx - q * 2 * Np, k = rem / Np, j = rem - k * Np;
-        const double* C = Cv + ((q * 4 + a) * 2 + k) * NSV;
-        const double* T = Tv + (q * 3) * Np + j;
-        Wv[idx] = C[sb[0]] * T[0] + C[sb[1]] * T[Np] + C[sb[2]] * T[2 * Np];
-      } else if (idx < nW + 2 * nWf) {
-        const int id2 = idx - nW;
-        const int side = id2 >= nWf;  // 0 own trace, 1 neighbour trace
-        const int id3 = side ? id2 - nWf : id2;
-        const int f = id3 / (nqf * Np), rem = id3 - f * nqf * Np, q = rem / Np, j = rem - q * Np;
-        const double* C = Cf + ((f * kMaxQf + q) * 4 + a) * NSF + (side ? 12 : 0);
-        const double* T = (side ? Tn : Tf) + ((f * kMaxQf + q) * 3) * Np + j;
-        const double w = C[sb[0]] * T[0] + C[sb[1]] * T[Np] + C[sb[2]] * T[2 * Np];
-        (side ? Wn : Wf)[(f * kMaxQf + q) * Np + j] = w;
-      } else if (idx < nW + 2 * nWf + 3 * nqv * 2) {
-        // cv[f][q][k] = s_f sum_d C_v(q, a, k; grad_d U_b) n_f[d] (faces this element lifts)
-        const int id2 = idx - nW - 2 * nWf, f = id2 / (nqv * 2), rem = id2 - f * nqv * 2, q = rem >> 1, k = rem & 1;
-        const double* C = Cv + ((q * 4 + a) * 2 + k) * NSV;
-        cvv[id2] = sidef[f] ? s_lift[f] * (C[sb[1]] * nf[f][0] + C[sb[2]] * nf[f][1]) : 0.0;
-      } else {
-        // cf[f][q] = s_S sum_d C_f(f, q, a; grad_d U_b of the flux side) n_f[d]
-        const int id2 = idx - nW - 2 * nWf - 3 * nqv * 2, f = id2 / nqf, q = id2 - f * nqf;
-        const double* C = Cf + ((f * kMaxQf + q) * 4 + a) * NSF + (sidef[f] ? 0 : 12);
-        cff[f * kMaxQf + q] = s_lift[f] * (C[sb[1]] * nf[f][0] + C[sb[2]] * nf[f][1]);
+    for (int idx = tid; idx < NBV * NP * 2 * NV; idx += T) {
+      const int jj = idx % NP, r = idx / NP, kq = r % (2 * NV), bb = r / (2 * NV), k = kq / NV, q = kq - k * NV, b = b0 + bb;
+      const double* C = Cv + ((q * 4 + a) * 2 + k) * 12;
+      double w = C[b] * tb.phi_v[q * NP + jj];
+      if (has_grad(a, b)) {
+        const double* dj = tb.dphi_v + 2 * (q * NP + jj);
+        w += C[4 + 2 * b] * dj[0] + C[5 + 2 * b] * dj[1];
+      }
+      put(smem + L::Wv + (bb * NP + jj) * LV + kq, &ex.Wv[bb][jj], w);
+    }
+    for (int idx = tid; idx < NBV * NP * F3; idx += T) {
+      const int jj = idx % NP, r = idx / NP, fq = r % F3, bb = r / F3, f = fq / NF, q = fq - f * NF, b = b0 + bb;
+      const double* C = Cf + fq * 64 + a * 16;
+      const int fn = gf[f] * NF + NF - 1 - q;
+      double wo = C[b] * tb.phi_f[fq * NP + jj];
+      double wn = tagf[f] == 0 ? C[4 + b] * tb.phi_f[fn * NP + jj] : 0.0;
+      if (has_grad(a, b)) {
+        const double* dj = tb.dphi_f + 2 * ((sidef[f] ? fq : fn) * NP + jj);
+        const double g = C[8 + 2 * b] * dj[0] + C[9 + 2 * b] * dj[1];
+        if (sidef[f]) wo += g;
+        else wn += g;
+      }
+      put(smem + L::Wf + (bb * NP + jj) * LF + fq, &ex.Wf[bb][jj], wo);
+      put(smem + L::Wn + (bb * NP + jj) * LF + fq, &ex.Wn[bb][f][jj], wn);
+    }
+    if (a > 0) {
+      // cv[f][q][k] = s_f sum_d C_v(q, a, k; grad_d U_b) n_f[d] (faces this element lifts)
+      for (int idx = tid; idx < NBV * 3 * NV * 2; idx += T) {
+        const int k = idx & 1, r = idx >> 1, q = r % NV, fb = r / NV, f = fb % 3, b = b0 + fb / 3;
+        const double* C = Cv + ((q * 4 + a) * 2 + k) * 12;
+        cvv[idx] = sidef[f] ? s_lift[f] * (C[4 + 2 * b] * nuo[f][0] + C[5 + 2 * b] * nuo[f][1]) : 0.0;
+      }
+      // cf[f][q] = s_S sum_d C_f(f, q, a; grad_d U_b of the flux side) n_f[d]
+      for (int idx = tid; idx < NBV * F3; idx += T) {
+        const int fq = idx % F3, f = fq / NF, b = b0 + idx / F3;
+        const double* C = Cf + fq * 64 + a * 16 + 8 + 2 * b;
+        cff[idx] = s_lift[f] * (C[0] * nus[f][0] + C[1] * nus[f][1]);
       }
     }
     __syncthreads();
-    // Y[f][i][q] = sum_k dphi_k,i(q) cv[f][q][k]
-    for (int idx = tid; idx < 3 * Np * nqv; idx += JAC_THREADS) {
-      const int f = idx / (Np * nqv), rem = idx - f * Np * nqv, i = rem / nqv, q = rem - i * nqv;
-      const double* di = tb.dphi_v + 2 * (q * Np + i);
-      const double* c = cvv + (f * nqv + q) * 2;
-      Yv[idx] = di[0] * c[0] + di[1] * c[1];
+    for (int idx = tid; idx < NBV * NP * 2 * NV; idx += T) {
+      const int jj = idx % NP, r = idx / NP, kq = r % (2 * NV), bb = r / (2 * NV);
+      enc(smem + L::Wv + (bb * NP + jj) * LV + kq, ex.Wv[bb][jj]);
+    }
+    for (int idx = tid; idx < NBV * NP * F3; idx += T) {
+      const int jj = idx % NP, r = idx / NP, fq = r % F3, bb = r / F3;
+      enc(smem + L::Wf + (bb * NP + jj) * LF + fq, ex.Wf[bb][jj]);
+      enc(smem + L::Wn + (bb * NP + jj) * LF + fq, ex.Wn[bb][fq / NF][jj]);
+    }
+    if (a > 0) {
+      // Y[f][i][q] = sum_k dphi_k,i(q) cv[f][q][k]
+      for (int idx = tid; idx < NBV * 3 * NP * NV; idx += T) {
+        const int i = idx % NP, r = idx / NP, q = r % NV, fb = r / NV, f = fb % 3, bb = fb / 3;
+        if (!sidef[f]) continue;
+        const double* di = tb.dphi_v + 2 * (q * NP + i);
+        const double* c = cvv + ((size_t)fb * NV + q) * 2;
+        put(smem + L::Y + (fb * NP + i) * LY + q, &ex.Y[bb][f][i], di[0] * c[0] + di[1] * c[1]);
+      }
+      __syncthreads();
+      for (int idx = tid; idx < NBV * 3 * NP * NV; idx += T) {
+        const int i = idx % NP, r = idx / NP, q = r % NV, fb = r / NV, f = fb % 3, bb = fb / 3;
+        if (sidef[f]) enc(smem + L::Y + (fb * NP + i) * LY + q, ex.Y[bb][f][i]);
+      }
+      __syncthreads();
+      // Lam[f][i][p] = d r_(a,i) / d jump_(f,b)(p): volume part (faces this element lifts)
+      // minus the face part (test function phi_i on face f, the flux side's lifting row)
+      for (int idx = tid; idx < NBV * NP * F3; idx += T) {
+        const int i = idx % NP, r = idx / NP, fp = r % F3, bb = r / F3, f = fp / NF, p = fp - f * NF;
+        double acc = 0.0;
+        if (has_grad(a, b0 + bb)) {
+          for (int q = 0; q < NF; ++q) {
+            int step;
+            const double* A = lift_row(tb, sidef[f], f, gf[f], q, step);
+            acc -= tb.phi_f[(f * NF + q) * NP + i] * (cff[bb * F3 + f * NF + q] * A[p * step]);
+          }
+          if (sidef[f])
+            acc = fix_dot<NV>(fix(L::Y) + ((bb * 3 + f) * NP + i) * LY, fix(L::lv) + fp * LY, ex.Y[bb][f][i], ex.lv[fp], acc);
+        }
+        put(smem + L::Lam + (bb * NP + i) * LF + fp, &ex.Lam[bb][i], acc);
+        if (tagf[f] == 1) LamW[((f * 4 + b0 + bb) * NP + i) * NF + p] = acc;
+      }
+      __syncthreads();
+      for (int idx = tid; idx < NBV * NP * F3; idx += T) {
+        const int i = idx % NP, r = idx / NP, fp = r % F3, bb = r / F3;
+        enc(smem + L::Lam + (bb * NP + i) * LF + fp, ex.Lam[bb][i]);
+      }
     }
     __syncthreads();
-    // Lam[f][i][p] = d r_(a,i) / d jump_(f,b)(p): volume part (faces this element lifts)
-    // minus the face part (test function phi_i on face f, the flux side's lifting row)
-    for (int idx = tid; idx < 3 * Np * nqf; idx += JAC_THREADS) {
-      const int f = idx / (Np * nqf), rem = idx - f * Np * nqf, i = rem / nqf, p = rem - i * nqf;
-      double acc = 0.0;
-      if (sidef[f]) {
-        const double* y = Yv + (f * Np + i) * nqv;
-        const double* lv = tb.lift_v + f * nqv * nqf + p;
-        for (int q = 0; q < nqv; ++q) acc += y[q] * lv[q * nqf];
-      }
-      for (int q = 0; q < nqf; ++q) {
-        int step;
-        const double* A = lift_row(tb, sidef[f], f, gf[f], q, step);
-        acc -= tb.phi_f[(f * nqf + q) * Np + i] * cff[f * kMaxQf + q] * A[p * step];
-      }
-      Lam[(f * Np + i) * kMaxQf + p] = acc;
-      if (tagf[f] == 1) LamW[((f * 4 + b) * Np + i) * kMaxQf + p] = acc;
-    }
-    __syncthreads();
-    for (int idx = tid; idx < 4 * Np * Np; idx += JAC_THREADS) {
-      const int slot = idx / (Np * Np), rem = idx - slot * Np * Np, j = rem / Np, i = rem - j * Np;
+    for (int idx = tid; idx < NBV * 4 * NP * NP; idx += T) {
+      const int i = idx % NP, r = idx / NP, jj = r % NP, sb = r / NP, slot = sb & 3, bb = sb >> 2, b = b0 + bb;
+      const bool grad = has_grad(a, b);
+      const Fix* lam = fix(L::Lam) + (bb * NP + i) * LF;
       double acc = 0.0;
       if (slot == 0) {
-        for (int q = 0; q < nqv; ++q) {
-          const double* di = tb.dphi_v + 2 * (q * Np + i);
-          acc += di[0] * Wv[(q * 2 + 0) * Np + j] + di[1] * Wv[(q * 2 + 1) * Np + j];
-        }
-        for (int f = 0; f < 3; ++f) {
-          for (int q = 0; q < nqf; ++q)
-            acc -= tb.phi_f[(f * nqf + q) * Np + i] * Wf[(f * kMaxQf + q) * Np + j];
-          // d jump / d u_e = -phi_j (the wall state's own dependence is added below)
-          for (int p = 0; p < nqf; ++p)
-            acc -= Lam[(f * Np + i) * kMaxQf + p] * Tf[((f * kMaxQf + p) * 3) * Np + j];
-        }
+        acc = fix_dot<2 * NV>(fix(L::dV) + i * LV, fix(L::Wv) + (bb * NP + jj) * LV, ex.dV[i], ex.Wv[bb][jj], acc);
+        acc = fix_dot_minus<F3>(fix(L::pF) + i * LF, fix(L::Wf) + (bb * NP + jj) * LF, ex.pF[i], ex.Wf[bb][jj], acc);
+        // d jump / d u_e = -phi_j (the wall state's own dependence is added below)
+        if (grad) acc = fix_dot_minus<F3>(lam, fix(L::pF) + jj * LF, ex.Lam[bb][i], ex.pF[jj], acc);
       } else {
-        const int f = slot - 1;
-        for (int q = 0; q < nqf; ++q) acc -= tb.phi_f[(f * nqf + q) * Np + i] * Wn[(f * kMaxQf + q) * Np + j];
-        // d jump / d u_nbr = +phi_j of the neighbour at the matched point (zero off interior faces)
-        for (int p = 0; p < nqf; ++p) acc += Lam[(f * Np + i) * kMaxQf + p] * Tn[((f * kMaxQf + p) * 3) * Np + j];
+        const int f = slot - 1, o = f * NF;
+        if (tagf[f] == 0) {
+          acc = fix_dot_minus<NF>(fix(L::pF) + i * LF + o, fix(L::Wn) + (bb * NP + jj) * LF + o, ex.pF[i],
+                                  ex.Wn[bb][f][jj], acc);
+          // d jump / d u_nbr = +phi_j of the neighbour at the matched point
+          if (grad) acc = fix_dot<NF>(lam + o, fix(L::pN) + jj * LF + o, ex.Lam[bb][i], ex.pN[jj], acc);
+        }
       }
-      Jd[(size_t)slot * nb2 + (size_t)(b * Np + j) * nb + a * Np + i] = acc;
+      Jd[(size_t)slot * nb2 + (size_t)(b * NP + jj) * NB + a * NP + i] = acc;
     }
-    __syncthreads();
-    if (has_wall && b == 3) {
+    if (has_wall && a > 0 && b0 + NBV == 4) {
+      __syncthreads();
       // wall points: the jump U_wall(U-) - U- also depends on U- through the wall state:
       // J_(a,c) += sum_b sum_p Lam_(a,b)[i][p] dU_wall,b/dU-_c phi_j(p)
-      for (int idx = tid; idx < 4 * Np * Np; idx += JAC_THREADS) {
-        const int c = idx / (Np * Np), rem = idx - c * Np * Np, j = rem / Np, i = rem - j * Np;
+      for (int idx = tid; idx < 4 * NP * NP; idx += T) {
+        const int c = idx / (NP * NP), rem = idx - c * NP * NP, jj = rem / NP, i = rem - jj * NP;
         double acc = 0.0;
         for (int f = 0; f < 3; ++f) {
           if (tagf[f] != 1) continue;
-          for (int p = 0; p < nqf; ++p) {
-            const double phij = Tf[((f * kMaxQf + p) * 3) * Np + j];
-            const double* G = Gb + (f * kMaxQf + p) * 16;
+          for (int p = 0; p < NF; ++p) {
+            const double phij = tb.phi_f[(f * NF + p) * NP + jj];
+            const double* G = Gb + (f * NF + p) * 16;
             double s = 0.0;
 #pragma unroll
-            for (int bb = 0; bb < 4; ++bb) s += LamW[((f * 4 + bb) * Np + i) * kMaxQf + p] * G[bb * 4 + c];
+            for (int bb = 0; bb < 4; ++bb) s += LamW[((f * 4 + bb) * NP + i) * NF + p] * G[bb * 4 + c];
             acc += s * phij;
           }
         }
-        Jd[(size_t)(c * Np + j) * nb + a * Np + i] += acc;
+        Jd[(size_t)(c * NP + jj) * NB + a * NP + i] += acc;
       }
-      __syncthreads();
     }
   }
 }
 
 // ------------------------------------------------------------------------ QoI
 // Per element: sum over its wall faces of w L (f . v_G, f_x), f = momentum part of the wall
-// flux (with the CDG lifting of the wall jump; the wall faces are always lifted by the element).
+// flux (with the CDG lifting of the wall jump; the wall faces are always lifted by the element);
+// T = DualV<3>: their derivatives for the three motion seeds of the frame, (power, force) by seed.
 template <class T>
 __global__ void __launch_bounds__(RES_WARPS * 32)
-    k_qoi(DevMesh m, DevTables tb, Phys ph, FrameT<T> fr, const double* __restrict__ u, double* __restrict__ out,
-          int want_der) {
+    k_qoi(DevMesh m, DevTables tb, Phys ph, FrameT<T> fr, const double* __restrict__ u, double* __restrict__ out) {
   constexpr int W = sizeof(T) / sizeof(double);
   __shared__ double s_J[RES_WARPS][3 * kMaxQf * 4 * W];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -750,16 +958,19 @@ __global__ void __launch_bounds__(RES_WARPS * 32)
     pw += wl * (H[1] * vG[0] + H[2] * vG[1]);
     fx += wl * H[1];
   }
-  double a0 = want_der ? der(pw) : val(pw);
-  double a1 = want_der ? der(fx) : val(fx);
+  constexpr int NC = sizeof(T) == sizeof(double) ? 1 : 3;
 #pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    a0 += __shfl_xor_sync(0xffffffffu, a0, o);
-    a1 += __shfl_xor_sync(0xffffffffu, a1, o);
-  }
-  if (lane == 0) {
-    out[2 * e] = a0;
-    out[2 * e + 1] = a1;
+  for (int c = 0; c < NC; ++c) {
+    double a0 = part(pw, c), a1 = part(fx, c);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      a0 += __shfl_xor_sync(0xffffffffu, a0, o);
+      a1 += __shfl_xor_sync(0xffffffffu, a1, o);
+    }
+    if (lane == 0) {
+      out[(size_t)2 * NC * e + 2 * c] = a0;
+      out[(size_t)2 * NC * e + 2 * c + 1] = a1;
+    }
   }
 }
 
@@ -895,51 +1106,95 @@ __global__ void __launch_bounds__(RES_WARPS * 32)
 
 static int res_blocks(int ne) { return (ne + RES_WARPS - 1) / RES_WARPS; }
 
-cudaError_t launch_residual(const DevMesh& m, const DevTables& tb, const Phys& ph, const FrameT<double>& fr,
-                            const double* u, double* r, cudaStream_t st) {
-  ProfScope ps(PP_K_RESIDUAL, st);
-  k_residual<double><<<res_blocks(m.ne), RES_WARPS * 32, 0, st>>>(m, tb, ph, fr, u, r, nullptr);
+template <int PD, class T>
+static cudaError_t run_residual(const DevMesh& m, const DevTables& tb, const Phys& ph, const FrameT<T>& fr,
+                                const double* u, const double* kappa, double* out, cudaStream_t st) {
+  using L = Res<PD, T>;
+  struct Setup {
+    cudaError_t err;
+    int resident;
+  };
+  // one device per process (see pp_create)
+  static const Setup setup = [] {
+    Setup r{cudaSuccess, 0};
+    r.err = cudaFuncSetAttribute(k_residual<PD, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * L::words);
+    if (r.err != cudaSuccess) return r;
+    int per_sm = 0, dev = 0, sms = 0;
+    r.err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_residual<PD, T>, L::THREADS, 8 * L::words);
+    if (r.err == cudaSuccess) r.err = cudaGetDevice(&dev);
+    if (r.err == cudaSuccess) r.err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    if (r.err == cudaSuccess && per_sm < 1) r.err = cudaErrorInvalidConfiguration;
+    r.resident = per_sm * sms;
+    return r;
+  }();
+  if (setup.err != cudaSuccess) return setup.err;
+  // groups as large as fill the warps, smaller on meshes that would leave SMs without one
+  int eb = (m.ne + setup.resident - 1) / setup.resident;
+  eb = eb < 1 ? 1 : eb > L::EB ? L::EB : eb;
+  const int groups = (m.ne + eb - 1) / eb, grid = groups < setup.resident ? groups : setup.resident;
+  k_residual<PD, T><<<grid, L::THREADS, 8 * L::words, st>>>(m, tb, ph, fr, u, kappa, out, eb);
   return cudaGetLastError();
 }
 
-cudaError_t launch_residual_dframe(const DevMesh& m, const DevTables& tb, const Phys& ph, const FrameT<Dual>& fr,
-                                   const double* u, double* dr, cudaStream_t st) {
+cudaError_t launch_residual(const DevMesh& m, const DevTables& tb, const Phys& ph, const FrameT<double>& fr,
+                            const double* u, double* r, cudaStream_t st) {
+  ProfScope ps(PP_K_RESIDUAL, st);
+  switch (tb.p) {
+    case 1: return run_residual<1, double>(m, tb, ph, fr, u, nullptr, r, st);
+    case 2: return run_residual<2, double>(m, tb, ph, fr, u, nullptr, r, st);
+    case 3: return run_residual<3, double>(m, tb, ph, fr, u, nullptr, r, st);
+    case 4: return run_residual<4, double>(m, tb, ph, fr, u, nullptr, r, st);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+cudaError_t launch_residual_dframe(const DevMesh& m, const DevTables& tb, const Phys& ph, const FrameT<DualV<3>>& fr,
+                                   const double* u, const double* kappa, double* per_elem, cudaStream_t st) {
   ProfScope ps(PP_K_OTHER, st);
-  k_residual<Dual><<<res_blocks(m.ne), RES_WARPS * 32, 0, st>>>(m, tb, ph, fr, u, nullptr, dr);
-  return cudaGetLastError();
+  switch (tb.p) {
+    case 1: return run_residual<1, DualV<3>>(m, tb, ph, fr, u, kappa, per_elem, st);
+    case 2: return run_residual<2, DualV<3>>(m, tb, ph, fr, u, kappa, per_elem, st);
+    case 3: return run_residual<3, DualV<3>>(m, tb, ph, fr, u, kappa, per_elem, st);
+    case 4: return run_residual<4, DualV<3>>(m, tb, ph, fr, u, kappa, per_elem, st);
+    default: return cudaErrorInvalidValue;
+  }
 }
 
 cudaError_t launch_jacobian(const DevMesh& m, const DevTables& tb, const Phys& ph, const FrameT<double>& fr,
                             const double* u, double* J, cudaStream_t st) {
   ProfScope ps(PP_K_JACOBIAN, st);
-  const size_t bytes = sizeof(double) * JacSmem(tb.nb, tb.Np, tb.nqv).total;
-  {
-    // largest dynamic shared memory requested so far (contexts of several degrees may share
-    // the process; one device per process, see pp_create)
-    static std::mutex mu;
-    static size_t configured = 0;
-    std::lock_guard<std::mutex> lock(mu);
-    if (bytes > configured) {
-      cudaError_t e = cudaFuncSetAttribute(k_jacobian, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-      if (e != cudaSuccess) return e;
-      configured = bytes;
-    }
+  switch (tb.p) {
+#define PP_JAC(PD)                                                                                       \
+  case PD: {                                                                                             \
+    constexpr int bytes = 8 * Jac<PD>::words;                                                            \
+    static const cudaError_t attr =                                                                      \
+        cudaFuncSetAttribute(k_jacobian<PD>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);        \
+    if (attr != cudaSuccess) return attr;                                                                \
+    k_jacobian<PD><<<m.ne, Jac<PD>::T, bytes, st>>>(m, tb, ph, fr, u, J);                                \
+    break;                                                                                               \
   }
-  k_jacobian<<<m.ne, JAC_THREADS, bytes, st>>>(m, tb, ph, fr, u, J);
+    PP_JAC(1)
+    PP_JAC(2)
+    PP_JAC(3)
+    PP_JAC(4)
+#undef PP_JAC
+    default:
+      return cudaErrorInvalidValue;
+  }
   return cudaGetLastError();
 }
 
 cudaError_t launch_qoi(const DevMesh& m, const DevTables& tb, const Phys& ph, const FrameT<double>& fr,
                        const double* u, double* per_elem, cudaStream_t st) {
   ProfScope ps(PP_K_OTHER, st);
-  k_qoi<double><<<res_blocks(m.ne), RES_WARPS * 32, 0, st>>>(m, tb, ph, fr, u, per_elem, 0);
+  k_qoi<double><<<res_blocks(m.ne), RES_WARPS * 32, 0, st>>>(m, tb, ph, fr, u, per_elem);
   return cudaGetLastError();
 }
 
-cudaError_t launch_qoi_dframe(const DevMesh& m, const DevTables& tb, const Phys& ph, const FrameT<Dual>& fr,
+cudaError_t launch_qoi_dframe(const DevMesh& m, const DevTables& tb, const Phys& ph, const FrameT<DualV<3>>& fr,
                               const double* u, double* per_elem, cudaStream_t st) {
   ProfScope ps(PP_K_OTHER, st);
-  k_qoi<Dual><<<res_blocks(m.ne), RES_WARPS * 32, 0, st>>>(m, tb, ph, fr, u, per_elem, 1);
+  k_qoi<DualV<3>><<<res_blocks(m.ne), RES_WARPS * 32, 0, st>>>(m, tb, ph, fr, u, per_elem);
   return cudaGetLastError();
 }
 

@@ -23,17 +23,18 @@
 
 namespace pp {
 
+// An FP64 division costs about ten instructions of a pipe that issues one per 19 clocks and SM, so
+// every function takes one reciprocal per state (ir = 1 / rho) and multiplies.
 template <class T>
-__device__ __forceinline__ T pressure(const T U[4], double gam) {
-  return (gam - 1.0) * (U[3] - 0.5 * (U[1] * U[1] + U[2] * U[2]) / U[0]);
+__device__ __forceinline__ T pressure(const T U[4], const T& ir, double gam) {
+  return (gam - 1.0) * (U[3] - 0.5 * (U[1] * U[1] + U[2] * U[2]) * ir);
 }
 
 // F[a][d]: inviscid flux of variable a in direction d
 template <class T>
-__device__ __forceinline__ void inviscid_flux(const T U[4], double gam, T F[4][2]) {
-  T r = U[0];
-  T u = U[1] / r, v = U[2] / r;
-  T p = pressure(U, gam);
+__device__ __forceinline__ void inviscid_flux(const T U[4], const T& ir, double gam, T F[4][2]) {
+  T u = U[1] * ir, v = U[2] * ir;
+  T p = pressure(U, ir, gam);
   F[0][0] = U[1];
   F[1][0] = U[1] * u + p;
   F[2][0] = U[2] * u;
@@ -47,10 +48,8 @@ __device__ __forceinline__ void inviscid_flux(const T U[4], double gam, T F[4][2
 // viscous flux from the state and its physical gradient dU[a][d];
 // q = -(mu/Pr) grad(E + p/rho - |u|^2/2) = -(mu gamma/Pr) grad(e)
 template <class T>
-__device__ __forceinline__ void viscous_flux(const T U[4], const T dU[4][2], const Phys& ph, bool adiabatic,
-                                             T F[4][2]) {
-  T r = U[0];
-  T ir = 1.0 / r;
+__device__ __forceinline__ void viscous_flux(const T U[4], const T& ir, const T dU[4][2], const Phys& ph,
+                                             bool adiabatic, T F[4][2]) {
   T u = U[1] * ir, v = U[2] * ir, E = U[3] * ir;
   T du[2], dv[2], dE[2];
 #pragma unroll
@@ -81,8 +80,9 @@ template <class T>
 __device__ __forceinline__ void volume_flux(const T U[4], const T dU[4][2], const T vG[2], const Phys& ph,
                                             T F[4][2]) {
   T Fi[4][2], Fv[4][2];
-  inviscid_flux(U, ph.gam, Fi);
-  viscous_flux(U, dU, ph, false, Fv);
+  const T ir = 1.0 / U[0];
+  inviscid_flux(U, ir, ph.gam, Fi);
+  viscous_flux(U, ir, dU, ph, false, Fv);
 #pragma unroll
   for (int a = 0; a < 4; ++a)
 #pragma unroll
@@ -90,70 +90,73 @@ __device__ __forceinline__ void volume_flux(const T U[4], const T dU[4][2], cons
 }
 
 template <class T>
-__device__ __forceinline__ void normal_flux(const T U[4], const T n[2], const T& vn, double gam, T out[4]) {
-  T F[4][2];
-  inviscid_flux(U, gam, F);
-#pragma unroll
-  for (int a = 0; a < 4; ++a) out[a] = F[a][0] * n[0] + F[a][1] * n[1] - vn * U[a];
+__device__ __forceinline__ void normal_flux(const T U[4], const T& ir, const T& p, const T n[2], const T& vn, T out[4]) {
+  const T un = (U[1] * n[0] + U[2] * n[1]) * ir;
+  const T w = un - vn;
+  out[0] = U[0] * w;
+  out[1] = U[1] * w + p * n[0];
+  out[2] = U[2] * w + p * n[1];
+  out[3] = U[3] * w + p * un;
 }
 
+// Harten's fix with delta = 0.1 c; h = 1 / (2 delta)
 template <class T>
-__device__ __forceinline__ T entropy_fix(T l, T delta) {
+__device__ __forceinline__ T entropy_fix(const T& l, const T& delta, const T& h) {
   T al = absT(l);
-  if (val(al) < val(delta)) return (l * l + delta * delta) / (2.0 * delta);
+  if (val(al) < val(delta)) return (l * l + delta * delta) * h;
   return al;
 }
 
 // Roe flux of the ALE normal flux; |A - vn I| (UR - UL) written with the two
-// wave-strength scalars of the acoustic pair.
+// wave-strength scalars of the acoustic pair.  iL, iR: 1 / rho of the two states.
 template <class T>
-__device__ __forceinline__ void roe_flux(const T UL[4], const T UR[4], const T n[2], const T& vn, double gam,
-                                         T out[4]) {
-  T rL = UL[0], rR = UR[0];
-  T uL = UL[1] / rL, vL = UL[2] / rL, uR = UR[1] / rR, vR = UR[2] / rR;
-  T pL = pressure(UL, gam), pR = pressure(UR, gam);
-  T HL = (UL[3] + pL) / rL, HR = (UR[3] + pR) / rR;
-  T sL = sqrtT(rL), sR = sqrtT(rR);
-  T isum = 1.0 / (sL + sR);
-  T ut = (sL * uL + sR * uR) * isum;
-  T vt = (sL * vL + sR * vR) * isum;
-  T Ht = (sL * HL + sR * HR) * isum;
-  T q2 = ut * ut + vt * vt;
-  T c2 = (gam - 1.0) * (Ht - 0.5 * q2);
-  T c = sqrtT(c2);
-  T un = ut * n[0] + vt * n[1];
-  T lu = un - vn;
-  T delta = 0.1 * c;
-  T l1 = entropy_fix(lu + c, delta);
-  T l2 = entropy_fix(lu - c, delta);
-  T l3 = entropy_fix(lu, delta);
+__device__ __forceinline__ void roe_flux(const T UL[4], const T& iL, const T UR[4], const T& iR, const T n[2],
+                                         const T& vn, double gam, T out[4]) {
+  const T pL = pressure(UL, iL, gam), pR = pressure(UR, iR, gam);
+  const T sL = sqrtT(UL[0]), sR = sqrtT(UR[0]);
+  const T isum = 1.0 / (sL + sR);
+  // sqrt(rho) / rho weights: s u = (s / rho) (rho u)
+  const T wL = sL * iL * isum, wR = sR * iR * isum;
+  const T ut = wL * UL[1] + wR * UR[1];
+  const T vt = wL * UL[2] + wR * UR[2];
+  const T Ht = wL * (UL[3] + pL) + wR * (UR[3] + pR);
+  const T hq2 = 0.5 * (ut * ut + vt * vt);
+  const T c2 = (gam - 1.0) * (Ht - hq2);
+  const T c = sqrtT(c2);
+  const T ic = 1.0 / c;
+  const T un = ut * n[0] + vt * n[1];
+  const T lu = un - vn;
+  const T delta = 0.1 * c, h = 5.0 * ic;
+  const T l1 = entropy_fix(lu + c, delta, h);
+  const T l2 = entropy_fix(lu - c, delta, h);
+  const T l3 = entropy_fix(lu, delta, h);
   T D[4];
 #pragma unroll
   for (int a = 0; a < 4; ++a) D[a] = UR[a] - UL[a];
-  T dp = (gam - 1.0) * (0.5 * q2 * D[0] - ut * D[1] - vt * D[2] + D[3]);
-  T dUn = D[1] * n[0] + D[2] * n[1] - un * D[0];
-  T s1 = 0.5 * (l1 + l2) - l3;
-  T s2 = (l1 - l2) / (2.0 * c);
-  T G1 = s1 * dp / c2 + s2 * dUn;
-  T G2 = s2 * dp + s1 * dUn;
+  const T dp = (gam - 1.0) * (hq2 * D[0] - ut * D[1] - vt * D[2] + D[3]);
+  const T dUn = D[1] * n[0] + D[2] * n[1] - un * D[0];
+  const T s1 = 0.5 * (l1 + l2) - l3;
+  const T s2 = 0.5 * (l1 - l2) * ic;
+  const T G1 = s1 * dp * (ic * ic) + s2 * dUn;
+  const T G2 = s2 * dp + s1 * dUn;
   T FL[4], FR[4];
-  normal_flux(UL, n, vn, gam, FL);
-  normal_flux(UR, n, vn, gam, FR);
-  T ev1[4] = {T(1.0), ut, vt, Ht};
-  T ev2[4] = {T(0.0), n[0], n[1], un};
-#pragma unroll
-  for (int a = 0; a < 4; ++a) out[a] = 0.5 * (FL[a] + FR[a]) - 0.5 * (l3 * D[a] + G1 * ev1[a] + G2 * ev2[a]);
+  normal_flux(UL, iL, pL, n, vn, FL);
+  normal_flux(UR, iR, pR, n, vn, FR);
+  out[0] = 0.5 * (FL[0] + FR[0] - (l3 * D[0] + G1));
+  out[1] = 0.5 * (FL[1] + FR[1] - (l3 * D[1] + G1 * ut + G2 * n[0]));
+  out[2] = 0.5 * (FL[2] + FR[2] - (l3 * D[2] + G1 * vt + G2 * n[1]));
+  out[3] = 0.5 * (FL[3] + FR[3] - (l3 * D[3] + G1 * Ht + G2 * un));
 }
 
 // No-slip wall state: the interior density and internal energy, moving with the wall.
 template <class T>
 __device__ __forceinline__ void wall_state(const T Um[4], const T vG[2], T Ub[4]) {
-  T r = Um[0];
-  T eint = Um[3] / r - 0.5 * (Um[1] * Um[1] + Um[2] * Um[2]) / (r * r);
+  const T r = Um[0];
   Ub[0] = r;
   Ub[1] = r * vG[0];
   Ub[2] = r * vG[1];
-  Ub[3] = r * (eint + 0.5 * (vG[0] * vG[0] + vG[1] * vG[1]));
+  // rho (E - |u|^2 / 2) + rho |v_G|^2 / 2
+  Ub[3] = Um[3] - 0.5 * (Um[1] * Um[1] + Um[2] * Um[2]) / r + 0.5 * (r * (vG[0] * vG[0] + vG[1] * vG[1]));
 }
 
 // Face value U_hat of U at one face point: the neighbour trace (tag 0), the wall state
@@ -184,12 +187,18 @@ __device__ __forceinline__ void face_flux(int tag, int side, const T Um[4], cons
   T vn = vG[0] * n[0] + vG[1] * n[1];
   T Hi[4], Uh[4], Fv[4][2];
   face_value(tag, Um, Up, vG, ph, Uh);
+  const T iL = 1.0 / Um[0];
   if (tag == 1) {
-    normal_flux(Uh, n, vn, ph.gam, Hi);
-    viscous_flux(Uh, QS, ph, true, Fv);
+    // the wall state shares the density
+    normal_flux(Uh, iL, pressure(Uh, iL, ph.gam), n, vn, Hi);
+    viscous_flux(Uh, iL, QS, ph, true, Fv);
   } else {
-    roe_flux(Um, Uh, n, vn, ph.gam, Hi);
-    viscous_flux(side ? Um : Up, QS, ph, false, Fv);
+    const T iR = 1.0 / Uh[0];
+    roe_flux(Um, iL, Uh, iR, n, vn, ph.gam, Hi);
+    T Us[4];
+#pragma unroll
+    for (int a = 0; a < 4; ++a) Us[a] = pick(side, Um[a], Up[a]);
+    viscous_flux(Us, pick(side, iL, iR), QS, ph, false, Fv);
   }
 #pragma unroll
   for (int a = 0; a < 4; ++a) H[a] = Hi[a] - (Fv[a][0] * n[0] + Fv[a][1] * n[1] + c11 * (Uh[a] - Um[a]));

@@ -62,9 +62,98 @@ __device__ __forceinline__ Dual sqrtT(Dual a) {
   double s = sqrt(a.v);
   return Dual(s, 0.5 * a.d / s);
 }
+// c ? a : b by components (a choice between array elements would put the arrays into local memory)
+PP_HD double pick(bool c, double a, double b) { return c ? a : b; }
+PP_HD Dual pick(bool c, const Dual& a, const Dual& b) { return Dual(c ? a.v : b.v, c ? a.d : b.d); }
 // |a| with the branch taken on the value (exact derivative away from a = 0)
 PP_HD double absT(double a) { return a >= 0.0 ? a : -a; }
 PP_HD Dual absT(Dual a) { return a.v >= 0.0 ? a : -a; }
+
+// N directional derivatives carried by one value: the value part (with its divisions and square
+// roots, the expensive FP64 operations) is formed once for all of them.
+template <int N>
+struct DualV {
+  double v, d[N];
+  PP_HD DualV() : v(0.0) {
+#pragma unroll
+    for (int k = 0; k < N; ++k) d[k] = 0.0;
+  }
+  PP_HD DualV(double a) : v(a) {
+#pragma unroll
+    for (int k = 0; k < N; ++k) d[k] = 0.0;
+  }
+};
+#define PP_DUALV(body_v, body_d)                     \
+  {                                                  \
+    DualV<N> r;                                      \
+    r.v = body_v;                                    \
+    _Pragma("unroll") for (int k = 0; k < N; ++k) r.d[k] = body_d; \
+    return r;                                        \
+  }
+template <int N>
+PP_HD DualV<N> operator+(const DualV<N>& a, const DualV<N>& b) PP_DUALV(a.v + b.v, a.d[k] + b.d[k])
+template <int N>
+PP_HD DualV<N> operator-(const DualV<N>& a, const DualV<N>& b) PP_DUALV(a.v - b.v, a.d[k] - b.d[k])
+template <int N>
+PP_HD DualV<N> operator-(const DualV<N>& a) PP_DUALV(-a.v, -a.d[k])
+template <int N>
+PP_HD DualV<N> operator*(const DualV<N>& a, const DualV<N>& b) PP_DUALV(a.v * b.v, a.d[k] * b.v + a.v * b.d[k])
+template <int N>
+PP_HD DualV<N> operator+(const DualV<N>& a, double b) PP_DUALV(a.v + b, a.d[k])
+template <int N>
+PP_HD DualV<N> operator+(double a, const DualV<N>& b) PP_DUALV(a + b.v, b.d[k])
+template <int N>
+PP_HD DualV<N> operator-(const DualV<N>& a, double b) PP_DUALV(a.v - b, a.d[k])
+template <int N>
+PP_HD DualV<N> operator-(double a, const DualV<N>& b) PP_DUALV(a - b.v, -b.d[k])
+template <int N>
+PP_HD DualV<N> operator*(const DualV<N>& a, double b) PP_DUALV(a.v * b, a.d[k] * b)
+template <int N>
+PP_HD DualV<N> operator*(double a, const DualV<N>& b) PP_DUALV(a * b.v, a * b.d[k])
+template <int N>
+PP_HD DualV<N> operator/(const DualV<N>& a, const DualV<N>& b) {
+  const double i = 1.0 / b.v, q = a.v * i;
+  DualV<N> r;
+  r.v = q;
+#pragma unroll
+  for (int k = 0; k < N; ++k) r.d[k] = (a.d[k] - q * b.d[k]) * i;
+  return r;
+}
+template <int N>
+PP_HD DualV<N> operator/(double a, const DualV<N>& b) {
+  const double i = 1.0 / b.v, q = a * i;
+  DualV<N> r;
+  r.v = q;
+#pragma unroll
+  for (int k = 0; k < N; ++k) r.d[k] = -q * i * b.d[k];
+  return r;
+}
+#undef PP_DUALV
+template <int N>
+PP_HD DualV<N>& operator+=(DualV<N>& a, const DualV<N>& b) { a = a + b; return a; }
+template <int N>
+PP_HD DualV<N>& operator-=(DualV<N>& a, const DualV<N>& b) { a = a - b; return a; }
+template <int N>
+PP_HD double val(const DualV<N>& a) { return a.v; }
+template <int N>
+__device__ __forceinline__ DualV<N> sqrtT(const DualV<N>& a) {
+  DualV<N> r;
+  r.v = sqrt(a.v);
+  const double h = 0.5 / r.v;
+#pragma unroll
+  for (int k = 0; k < N; ++k) r.d[k] = a.d[k] * h;
+  return r;
+}
+template <int N>
+PP_HD DualV<N> pick(bool c, const DualV<N>& a, const DualV<N>& b) {
+  DualV<N> r;
+  r.v = c ? a.v : b.v;
+#pragma unroll
+  for (int k = 0; k < N; ++k) r.d[k] = c ? a.d[k] : b.d[k];
+  return r;
+}
+template <int N>
+PP_HD DualV<N> absT(const DualV<N>& a) { return a.v >= 0.0 ? a : -a; }
 
 // ---------------------------------------------------------------- physics and motion
 struct Phys {
@@ -127,15 +216,16 @@ struct DevMesh {
 // All take the stream explicitly and return the launch error (cudaSuccess on success).
 cudaError_t launch_residual(const DevMesh& m, const DevTables& tb, const Phys& ph, const FrameT<double>& fr,
                             const double* u, double* r, cudaStream_t st);
-// derivative of r with respect to a frame seed (the frame carries the derivative)
-cudaError_t launch_residual_dframe(const DevMesh& m, const DevTables& tb, const Phys& ph, const FrameT<Dual>& fr,
-                                   const double* u, double* dr, cudaStream_t st);
+// per element kappa . dr/ds [ne][3] for three seeds s (the frame carries the derivatives)
+cudaError_t launch_residual_dframe(const DevMesh& m, const DevTables& tb, const Phys& ph, const FrameT<DualV<3>>& fr,
+                                   const double* u, const double* kappa, double* per_elem, cudaStream_t st);
 cudaError_t launch_jacobian(const DevMesh& m, const DevTables& tb, const Phys& ph, const FrameT<double>& fr,
                             const double* u, double* J, cudaStream_t st);
 // per-element (P^h, F_x^h) contributions [ne][2]
 cudaError_t launch_qoi(const DevMesh& m, const DevTables& tb, const Phys& ph, const FrameT<double>& fr,
                        const double* u, double* per_elem, cudaStream_t st);
-cudaError_t launch_qoi_dframe(const DevMesh& m, const DevTables& tb, const Phys& ph, const FrameT<Dual>& fr,
+// their derivatives for three seeds [ne][seed][2]
+cudaError_t launch_qoi_dframe(const DevMesh& m, const DevTables& tb, const Phys& ph, const FrameT<DualV<3>>& fr,
                               const double* u, double* per_elem, cudaStream_t st);
 // g = d(w0 P^h + w1 F_x^h)/du  (DEVICE [N_u], zero away from the wall)
 cudaError_t launch_qoi_du(const DevMesh& m, const DevTables& tb, const Phys& ph, const FrameT<double>& fr,

@@ -673,7 +673,6 @@ int adjoint_sweep(pp_ctx* ctx, const double* lam_Nt, const double* weights, doub
   double* y[3] = {work_vec(ctx, 18), work_vec(ctx, 19), work_vec(ctx, 20)};
   double* g[3] = {work_vec(ctx, 21), work_vec(ctx, 22), work_vec(ctx, 23)};
   double* rhs = work_vec(ctx, 14);
-  double* dr = work_vec(ctx, 15);
   const bool withF = weights != nullptr;
   const double w0 = withF ? weights[0] : 0.0, w1 = withF ? weights[1] : 0.0;
   std::vector<double> grad(n_mu, 0.0);
@@ -732,22 +731,23 @@ int adjoint_sweep(pp_ctx* ctx, const double* lam_Nt, const double* weights, doub
         // kappa_i . dr/ds and dQ/ds for the motion seeds s = theta, theta', h'
         const size_t st = (size_t)step * 3 + i;
         double* gt = ctx->d_gterm + 9 * st;
-        for (int s = 0; s < 3; ++s) {
-          FrameT<Dual> fd;
-          double cth = std::cos(mo.th), sth = std::sin(mo.th);
-          double dQ[4] = {-sth, cth, -cth, -sth};        // dQ/dtheta
-          double d2Q[4] = {-cth, -sth, sth, -cth};        // d2Q/dtheta2
-          for (int k2 = 0; k2 < 4; ++k2) {
-            fd.Q[k2] = Dual(fr.Q[k2], s == 0 ? dQ[k2] : 0.0);
-            fd.Qd[k2] = Dual(fr.Qd[k2], s == 0 ? mo.thd * d2Q[k2] : (s == 1 ? dQ[k2] : 0.0));
-          }
-          fd.hd = Dual(fr.hd, s == 2 ? 1.0 : 0.0);
-          PP_CK(launch_residual_dframe(m, ctx->tb, ctx->ph, fd, ui, dr, ctx->stream));
-          PP_CK(launch_dot<double>(n, kap, dr, gt + s, ctx->d_partial, ctx->d_counter, ctx->stream));
-          PP_CK(launch_qoi_dframe(m, ctx->tb, ctx->ph, fd, ui, ctx->d_elem, ctx->stream));
-          PP_CK(launch_colsum(mesh->ne, 2, ctx->d_elem, gt + 3 + 2 * s, ctx->d_partial, ctx->d_counter,
-                              ctx->stream));
+        const double cth = std::cos(mo.th), sth = std::sin(mo.th);
+        const double dQ[4] = {-sth, cth, -cth, -sth};    // dQ/dtheta
+        const double d2Q[4] = {-cth, -sth, sth, -cth};   // d2Q/dtheta2
+        FrameT<DualV<3>> fd;
+        for (int k2 = 0; k2 < 4; ++k2) {
+          fd.Q[k2] = DualV<3>(fr.Q[k2]);
+          fd.Q[k2].d[0] = dQ[k2];
+          fd.Qd[k2] = DualV<3>(fr.Qd[k2]);
+          fd.Qd[k2].d[0] = mo.thd * d2Q[k2];
+          fd.Qd[k2].d[1] = dQ[k2];
         }
+        fd.hd = DualV<3>(fr.hd);
+        fd.hd.d[2] = 1.0;
+        PP_CK(launch_residual_dframe(m, ctx->tb, ctx->ph, fd, ui, kap, ctx->d_elem, ctx->stream));
+        PP_CK(launch_colsum(mesh->ne, 3, ctx->d_elem, gt, ctx->d_partial, ctx->d_counter, ctx->stream));
+        PP_CK(launch_qoi_dframe(m, ctx->tb, ctx->ph, fd, ui, ctx->d_elem, ctx->stream));
+        PP_CK(launch_colsum(mesh->ne, 6, ctx->d_elem, gt + 3, ctx->d_partial, ctx->d_counter, ctx->stream));
         for (int j = 0; j < n_mu; ++j) {
           double* d = &ds_host[(st * n_mu + j) * 3];
           d[0] = mo.dth[j];
