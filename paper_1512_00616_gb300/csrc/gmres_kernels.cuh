@@ -63,10 +63,12 @@ constexpr int GM = kGmresMaxRestart;   // most basis vectors per cycle
 constexpr int GCTAS = 152;             // partial columns
 constexpr int GLD = GM + 2;            // partial rows
 constexpr int kCluster = 8;
+// how the CTAs of a solve exchange data
+enum Mode { kGrid, kClusters, kSingle };
 constexpr unsigned long long kBarrierNs = 1000000000ull;
 // barrier words, on their own 128-byte lines
 constexpr int BAR_COUNT = 0, BAR_EXIT = 32, BAR_ERROR = 64, BAR_WORDS = 96;
-constexpr int kDynSmemMax = 180 * 1024;
+constexpr int kSmemMax = 227 * 1024;   // shared memory of a CTA
 
 // Blocks and exchanged vectors: FP64 ones travel as 58-bit fixed-point words with one exponent
 // per block row / element slice (fixed.cuh), FP32 ones as they are.
@@ -113,26 +115,29 @@ __device__ __forceinline__ unsigned long long now_ns() {
 }
 
 // Barrier over all CTAs of the launch, split into arrive and wait so that loads that do not
-// depend on it go between.  Whole grid: a monotonic count (arrivals add with release, waiters
+// depend on it go between.  One CTA: a block barrier.  Whole grid: a monotonic count (arrivals add with release, waiters
 // poll it with acquire), reset by the CTA that leaves the kernel last.  Cluster: the hardware
 // barrier, which orders global memory at cluster scope.
-template <bool CL>
+template <int MODE>
 struct Barrier {
   unsigned* bar;
   unsigned target;
   int* s_ok;
   __device__ void arrive() {
-    if constexpr (CL) {
+    if constexpr (MODE == kClusters) {
       asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    } else {
+    } else if constexpr (MODE == kGrid) {
       __syncthreads();
       target += gridDim.x;
       if (threadIdx.x == 0) asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar + BAR_COUNT) : "memory");
     }
   }
   __device__ bool wait() {
-    if constexpr (CL) {
+    if constexpr (MODE == kClusters) {
       asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
+      return true;
+    } else if constexpr (MODE == kSingle) {
+      __syncthreads();
       return true;
     } else {
       if (threadIdx.x == 0) {
@@ -159,7 +164,7 @@ struct Barrier {
   }
   // after the last barrier of the launch
   __device__ void leave() {
-    if constexpr (!CL) {
+    if constexpr (MODE == kGrid) {
       if (threadIdx.x == 0 && atomicAdd(bar + BAR_EXIT, 1u) == gridDim.x - 1u) {
         bar[BAR_COUNT] = 0u;
         bar[BAR_EXIT] = 0u;
@@ -171,6 +176,7 @@ struct Barrier {
 template <int NB, class S>
 struct Rows {
   static constexpr int E = GT / NB;  // most elements per pass, one thread per row
+  static constexpr int CE = E >= 13 ? E : 24 / E * E;  // elements whose coefficients are held at a time
   static constexpr int C = 3 * NB;   // columns of a row of B
   static constexpr int U = (NB <= 24 ? 6 : 10) * (sizeof(S) == 8 ? 1 : 2);  // columns per ring chunk
   static constexpr int NCH = C / U;  // chunks per row, a multiple of 3; 6 with the deep ring
@@ -181,22 +187,37 @@ struct Rows {
 // Ring of a thread's next columns of B in shared memory, filled by cp.async: a thread copies and
 // reads only its own words, so no barrier is involved, and the ring runs on over passes, products
 // and grid barriers.  ST chunks of U columns: 3 (77 KB) beside a basis in shared memory, 6 without.
+// The blocks interleave VW columns (fold_index), so a copy is 16 bytes per thread and 512
+// contiguous bytes per warp: with one word per copy the SM's outstanding requests, not the bytes,
+// were the limit (8192 triangles: 5.1 TB/s in FP64 words, 3.0 TB/s in FP32 words).
 template <int NB, class S, int ST>
 struct Ring {
   using R = Rows<NB, S>;
   using W = typename Wire<S>::T;
+  static constexpr int VW = FoldOut<S>::VW, UV = R::U / VW;
   static constexpr int WORDS = ST * R::U * GT;
-  W* mine;  // this thread's words, GT apart
-  __device__ explicit Ring(W* base) : mine(base + threadIdx.x) {}
-  __device__ __forceinline__ W get(int slot, int u) const { return mine[(slot * R::U + u) * GT]; }
+  int4* mine;  // this thread's vectors, GT apart
+  __device__ explicit Ring(void* base) : mine(reinterpret_cast<int4*>(base) + threadIdx.x) {}
+  // vector v of chunk `slot`
+  __device__ __forceinline__ void get(int slot, int v, W (&w)[VW]) const {
+    const int4 x = mine[(slot * UV + v) * GT];
+    if constexpr (sizeof(S) == 8) {
+      w[0] = Fix{x.x, x.y};
+      w[1] = Fix{x.z, x.w};
+    } else {
+      w[0] = __int_as_float(x.x);
+      w[1] = __int_as_float(x.y);
+      w[2] = __int_as_float(x.z);
+      w[3] = __int_as_float(x.w);
+    }
+  }
   // chunk c of the row into `slot`, as one group (an empty one without a row)
   __device__ __forceinline__ void put(int slot, const W* row, bool on, int c) const {
     if (on) {
 #pragma unroll
-      for (int u = 0; u < R::U; ++u) {
-        const unsigned dst = static_cast<unsigned>(__cvta_generic_to_shared(mine + (slot * R::U + u) * GT));
-        asm volatile("cp.async.ca.shared.global [%0], [%1], %2;" ::"r"(dst), "l"(row + (size_t)(c * R::U + u) * NB),
-                     "n"((int)sizeof(W))
+      for (int v = 0; v < UV; ++v) {
+        const unsigned dst = static_cast<unsigned>(__cvta_generic_to_shared(mine + (slot * UV + v) * GT));
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(row + (size_t)(c * UV + v) * (NB * VW))
                      : "memory");
       }
     }
@@ -217,8 +238,9 @@ struct GShared {
   typename Wire<S>::T xs[2][Rows<NB, S>::XS];
   int xe[2][3 * Rows<NB, S>::E];
   int emax[3][Rows<NB, S>::E];  // exponents of the slices being published
-  typename Wire<S>::T cq[sizeof(S) == 8 ? Rows<NB, S>::E * GM : 1];  // coefficients against an element's slices
-  int ce[sizeof(S) == 8 ? Rows<NB, S>::E : 1];
+  typename Wire<S>::T cq[sizeof(S) == 8 ? Rows<NB, S>::CE * GM : 1];  // coefficients against the elements' slices
+  int ce[sizeof(S) == 8 ? Rows<NB, S>::CE : 1];
+  double dpart[3][GLD], single[2][GLD];
   double nrm2, inv, tol;
   int need, ok, stop;
 };
@@ -264,7 +286,7 @@ __device__ __forceinline__ void publish(const GArgs<S>& a, GShared<NB, S>& sh, i
 }
 
 // operand entry idx of the pass at `pos`
-template <int NB, class S>
+template <int NB, class S, int MODE>
 __device__ __forceinline__ typename Wire<S>::T operand(const GArgs<S>& a, int pos, int end, int idx) {
   using W = typename Wire<S>::T;
   const int el = idx / (3 * NB), rem = idx - el * 3 * NB, f = rem / NB, c = rem - f * NB;
@@ -272,18 +294,20 @@ __device__ __forceinline__ typename Wire<S>::T operand(const GArgs<S>& a, int po
   const int s = a.src[3 * (pos + el) + f];
   if (s < 0) return W{};
   if constexpr (sizeof(S) == 8) {
-    const int2 v = __ldcg(reinterpret_cast<const int2*>(a.wire) + (size_t)s * NB + c);
+    const int2* p = reinterpret_cast<const int2*>(a.wire) + (size_t)s * NB + c;
+    const int2 v = MODE == kSingle ? *p : __ldcg(p);
     return Fix{v.x, v.y};
   } else {
-    return __ldcg(a.wire + (size_t)s * NB + c);
+    const W* p = a.wire + (size_t)s * NB + c;
+    return MODE == kSingle ? *p : __ldcg(p);
   }
 }
 
-template <class S>
+template <class S, int MODE>
 __device__ __forceinline__ int operand_exp(const GArgs<S>& a, int pos, int end, int idx) {
   if (sizeof(S) != 8 || pos + idx / 3 >= end) return 0;
   const int s = a.src[3 * pos + idx];
-  return s < 0 ? 0 : __ldcg(a.wexp + s);
+  return s < 0 ? 0 : MODE == kSingle ? a.wexp[s] : __ldcg(a.wexp + s);
 }
 
 // this thread's row of B in the first of the equal passes over [p0, p1), or null
@@ -292,7 +316,7 @@ __device__ __forceinline__ const typename Wire<S>::T* first_row_of(const GArgs<S
   using R = Rows<NB, S>;
   const Lane<NB> ln;
   const int np = (p1 - p0 + R::E - 1) / R::E, per = np > 0 ? (p1 - p0 + np - 1) / np : 0;
-  return ln.el < per && p0 + ln.el < p1 ? a.B + (size_t)a.list[p0 + ln.el] * (3 * NB * NB) + ln.row : nullptr;
+  return ln.el < per && p0 + ln.el < p1 ? a.B + (size_t)a.list[p0 + ln.el] * (3 * NB * NB) + ln.row * FoldOut<S>::VW : nullptr;
 }
 
 // Rows at positions [p0, p1) of B times the exchanged operand: epi(on, element of the pass, row,
@@ -300,13 +324,13 @@ __device__ __forceinline__ const typename Wire<S>::T* first_row_of(const GArgs<S
 // `row` (first_row_of the range), on return those of `after`.  `ready` is called before the first
 // operand loads (the barrier wait); when it returns false nothing is done.  The scalar warp calls
 // `side` while the others do the first pass.
-template <int NB, class S, int ST, class Ready, class Side, class Epi>
+template <int NB, class S, int ST, int MODE, class Ready, class Side, class Epi>
 __device__ __forceinline__ bool rows_product(const GArgs<S>& a, GShared<NB, S>& sh, const Ring<NB, S, ST>& ring,
                                              int p0, int p1, const typename Wire<S>::T* row,
                                              const typename Wire<S>::T* after, Ready ready, Side side, Epi epi) {
   using R = Rows<NB, S>;
   using W = typename Wire<S>::T;
-  constexpr int NBB = 3 * NB * NB;
+  constexpr int NBB = 3 * NB * NB, VW = FoldOut<S>::VW;
   const Lane<NB> ln;
   // passes of equal size
   const int np = (p1 - p0 + R::E - 1) / R::E, per = np > 0 ? (p1 - p0 + np - 1) / np : 0;
@@ -319,9 +343,9 @@ __device__ __forceinline__ bool rows_product(const GArgs<S>& a, GShared<NB, S>& 
 #pragma unroll
     for (int q = 0; q < R::XP; ++q) {
       const int idx = threadIdx.x + q * GT;
-      if (idx < R::XS) sh.xs[0][idx] = operand<NB, S>(a, p0, p1, idx);
+      if (idx < R::XS) sh.xs[0][idx] = operand<NB, S, MODE>(a, p0, p1, idx);
     }
-    if (threadIdx.x < 3 * R::E) sh.xe[0][threadIdx.x] = operand_exp<S>(a, p0, p1, threadIdx.x);
+    if (threadIdx.x < 3 * R::E) sh.xe[0][threadIdx.x] = operand_exp<S, MODE>(a, p0, p1, threadIdx.x);
   }
   __syncthreads();
   if (threadIdx.x >= GT) side();
@@ -333,18 +357,18 @@ __device__ __forceinline__ bool rows_product(const GArgs<S>& a, GShared<NB, S>& 
     int er = 0;
     if (more && threadIdx.x < GT) {
 #pragma unroll
-      for (int q = 0; q < R::XP; ++q) xr[q] = operand<NB, S>(a, nx, p1, threadIdx.x + q * GT);
-      if (threadIdx.x < 3 * R::E) er = operand_exp<S>(a, nx, p1, threadIdx.x);
+      for (int q = 0; q < R::XP; ++q) xr[q] = operand<NB, S, MODE>(a, nx, p1, threadIdx.x + q * GT);
+      if (threadIdx.x < 3 * R::E) er = operand_exp<S, MODE>(a, nx, p1, threadIdx.x);
     }
     const W* const row2 = !more ? after
-                          : ln.el < per && nx + ln.el < p1 ? a.B + (size_t)a.list[nx + ln.el] * NBB + ln.row : nullptr;
+                          : ln.el < per && nx + ln.el < p1 ? a.B + (size_t)a.list[nx + ln.el] * NBB + ln.row * VW : nullptr;
     const W* xe = sh.xs[buf] + ln.el * R::C;
     S sum = S(0);
     if constexpr (sizeof(S) == 8) {
       int eb[3] = {0, 0, 0};
       if (on) {
         // the row's exponents lie as its block does
-        const int* be = a.Bexp + ((size_t)(row - a.B) - ln.row) / NB + ln.row;
+        const int* be = a.Bexp + ((size_t)(row - a.B) - ln.row * VW) / NB + ln.row;
 #pragma unroll
         for (int f = 0; f < 3; ++f) eb[f] = __ldg(be + f * NB);
       }
@@ -354,11 +378,14 @@ __device__ __forceinline__ bool rows_product(const GArgs<S>& a, GShared<NB, S>& 
         ring.wait();
         if (on) {
 #pragma unroll
-          for (int u = 0; u < R::U; ++u) {
+          for (int u = 0; u < R::U; u += VW) {
             const int col = c * R::U + u;
+            W w[VW];
+            ring.get(c % ST, u / VW, w);
             if (col % NB == 0) acc.clear();
-            acc.add(ring.get(c % ST, u), xe[col]);
-            if (col % NB == NB - 1) {
+            acc.add(w[0], xe[col]);
+            acc.add(w[1], xe[col + 1]);
+            if ((col + VW) % NB == 0) {
               const int f = col / NB, ex = sh.xe[buf][3 * ln.el + f];
               sum = acc.result(eb[f] + ex, eb[f] == 0x7ff || ex == 0x7ff, sum);
             }
@@ -374,7 +401,12 @@ __device__ __forceinline__ bool rows_product(const GArgs<S>& a, GShared<NB, S>& 
         ring.wait();
         if (on) {
 #pragma unroll
-          for (int u = 0; u < R::U; ++u) acc[u & 3] += ring.get(c % ST, u) * xe[c * R::U + u];
+          for (int u = 0; u < R::U; u += VW) {
+            W w[VW];
+            ring.get(c % ST, u / VW, w);
+#pragma unroll
+            for (int v = 0; v < VW; ++v) acc[v] += w[v] * xe[c * R::U + u + v];
+          }
         }
         if (c + ST < R::NCH) ring.put(c % ST, row, on, c + ST);
         else ring.put(c % ST, row2, row2 != nullptr, c + ST - R::NCH);
@@ -400,7 +432,8 @@ __device__ __forceinline__ bool rows_product(const GArgs<S>& a, GShared<NB, S>& 
 // CTA partials of (V_0 .. V_{k-1}, w) . w over the own rows -> region[t][cta], w in slot k.
 // FP32: a warp takes Q vectors at a time over all own rows.
 template <int Q>
-__device__ __forceinline__ void own_dots(const float* V, size_t ldv, int k, int from, int n, double* region) {
+__device__ __forceinline__ void own_dots(const float* V, size_t ldv, int k, int from, int n, double* region,
+                                         int rs) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   if (warp >= GW) return;
   const float* w = V + (size_t)k * ldv;
@@ -431,7 +464,7 @@ __device__ __forceinline__ void own_dots(const float* V, size_t ldv, int k, int 
     constexpr int sh = 5 - ILog2<Q>::value;
     if ((lane & ((1 << sh) - 1)) == 0) {
       const int t = t0 + (lane >> sh);
-      if (t <= k) region[(size_t)(t - from) * GCTAS + blockIdx.x] = (double)a[0];
+      if (t <= k) region[(size_t)(t - from) * rs + blockIdx.x] = (double)a[0];
     }
   }
 }
@@ -439,31 +472,32 @@ __device__ __forceinline__ void own_dots(const float* V, size_t ldv, int k, int 
 // `from`: first vector (0, or k for |w|^2 alone), written from region row 0 on.
 template <int NB>
 __device__ __forceinline__ void cta_dots(const float* V, const int*, size_t ldv, size_t, int k, int from, int nel,
-                                         double* region) {
+                                         double* region, int rs, double (*)[GLD]) {
   const int nk = k - from, n = nel * NB;
-  if (nk < GW) own_dots<1>(V, ldv, k, from, n, region);
-  else if (nk < 2 * GW) own_dots<2>(V, ldv, k, from, n, region);
-  else own_dots<4>(V, ldv, k, from, n, region);
+  if (nk < GW) own_dots<1>(V, ldv, k, from, n, region, rs);
+  else if (nk < 2 * GW) own_dots<2>(V, ldv, k, from, n, region, rs);
+  else own_dots<4>(V, ldv, k, from, n, region, rs);
 }
 
 // FP64: eight lanes per vector; they share the entries of a slice (coalesced), and each lane turns
 // its exact integer sum over them into a double, so the FP64 pipe sees two instructions per slice.
+// A warp takes four vectors; with few vectors up to three warps share the elements of four.
 template <int NB>
 __device__ __forceinline__ void cta_dots(const Fix* V, const int* Vexp, size_t ldv, size_t lde, int k, int from,
-                                         int nel, double* region) {
+                                         int nel, double* region, int rs, double (*dpart)[GLD]) {
   constexpr int P = (NB + 7) / 8;
-  const int lane = threadIdx.x & 31, l = lane & 7;
-  if (threadIdx.x >= GT) return;
+  const int lane = threadIdx.x & 31, l = lane & 7, warp = threadIdx.x >> 5;
+  const int groups = (k - from) / 4 + 1, share = min(3, max(1, GW / groups));
   const Fix* w = V + (size_t)k * ldv;
   const int* we = Vexp + (size_t)k * lde;
-  for (int t0 = from + (threadIdx.x >> 5) * 4; t0 <= k; t0 += GT / 8) {
-    const int t = t0 + (lane >> 3);
+  for (int g = warp; g < groups * share && warp < GW; g += GW) {
+    const int sp = g / groups, t = from + (g - sp * groups) * 4 + (lane >> 3);
     double s = 0.0;
     if (t <= k) {
       const Fix* v = V + (size_t)t * ldv;
       const int* ve = Vexp + (size_t)t * lde;
-#pragma unroll 2
-      for (int el = 0; el < nel; ++el) {
+#pragma unroll 3
+      for (int el = sp; el < nel; el += share) {
         FixDot acc;
         acc.clear();
 #pragma unroll
@@ -477,46 +511,71 @@ __device__ __forceinline__ void cta_dots(const Fix* V, const int* Vexp, size_t l
     }
 #pragma unroll
     for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (l == 0 && t <= k) region[(size_t)(t - from) * GCTAS + blockIdx.x] = s;
+    if (l == 0 && t <= k) dpart[sp][t - from] = s;
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t <= k - from; t += GALL) {
+    double s = dpart[0][t];
+    for (int sp = 1; sp < share; ++sp) s += dpart[sp][t];
+    region[(size_t)t * rs + blockIdx.x] = s;
   }
 }
 
 // out[t] = sum over the CTAs of region[t][.], t < nk, the same in every CTA: a warp per output, the
 // partials as integers against their largest exponent (exact sums, no FP64 additions).
+template <int MODE>
 __device__ __forceinline__ void sum_partials(int nk, const double* region, double* out) {
-  constexpr int R = (GCTAS + 31) / 32;
+  if constexpr (MODE == kSingle) {
+    for (int t = threadIdx.x; t < nk; t += GALL) out[t] = region[t];
+    __syncthreads();
+    return;
+  }
+  constexpr int R = (GCTAS + 31) / 32, Q = 3;  // Q outputs of a warp at a time: their loads overlap
   const int lane = threadIdx.x & 31, G = gridDim.x;
-  for (int t = threadIdx.x >> 5; t < nk && threadIdx.x < GT; t += GW) {
-    double v[R];
-    int e = 0;
+  for (int t0 = threadIdx.x >> 5; t0 < nk && threadIdx.x < GT; t0 += Q * GW) {
+    double v[Q][R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) {
-      const int c = lane + 32 * r;
-      v[r] = c < G ? __ldcg(region + (size_t)t * GCTAS + c) : 0.0;
+    for (int p = 0; p < Q; ++p)
+#pragma unroll
+      for (int r = 0; r < R; ++r) {
+        const int c = lane + 32 * r, t = t0 + p * GW;
+        v[p][r] = c < G && t < nk ? __ldcg(region + (size_t)t * GCTAS + c) : 0.0;
+      }
+    long long q[Q];
+    int e[Q];
+#pragma unroll
+    for (int p = 0; p < Q; ++p) {
+      e[p] = 0;
+#pragma unroll
+      for (int r = 0; r < R; ++r) e[p] = max(e[p], fix_exponent(v[p][r]));
+      e[p] = __reduce_max_sync(0xffffffffu, e[p]);
+      // |q| < 2^54 each, at most 160 of them
+      q[p] = 0;
+#pragma unroll
+      for (int r = 0; r < R; ++r) q[p] += fix_word(v[p][r], e[p] + 3);
     }
 #pragma unroll
-    for (int r = 0; r < R; ++r) e = max(e, fix_exponent(v[r]));
-    e = __reduce_max_sync(0xffffffffu, e);
-    // |q| < 2^54 each, at most 160 of them
-    long long q = 0;
+    for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-    for (int r = 0; r < R; ++r) q += fix_word(v[r], e + 3);
+      for (int p = 0; p < Q; ++p) q[p] += __shfl_xor_sync(0xffffffffu, q[p], o);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) q += __shfl_xor_sync(0xffffffffu, q, o);
-    if (lane == 0) out[t] = e == 0x7ff ? __longlong_as_double(0x7ff8000000000000LL) : (double)q * fix_pow2(e - 1076);
+    for (int p = 0; p < Q; ++p)
+      if (lane == p && t0 + p * GW < nk)
+        out[t0 + p * GW] = e[p] == 0x7ff ? __longlong_as_double(0x7ff8000000000000LL) : (double)q[p] * fix_pow2(e[p] - 1076);
   }
   __syncthreads();
 }
 
-// Coefficients c_t, t < k, of a pass's rows against the own slices of the basis (FP64): per element
-// one exponent for all c_t 2^(exponent of its slice of V_t).
+// Coefficients c_t, t < k, against the own slices of the basis (FP64), for up to CE own elements from
+// q0 on: per element one exponent for all c_t 2^(exponent of its slice of V_t).
 template <int NB>
 __device__ __forceinline__ void set_coefficients(GShared<NB, double>& sh, const double* c, int k, const int* Vexp,
                                                  size_t lde, int q0, int nel) {
-  constexpr int E = Rows<NB, double>::E;
-  const int n = min(E, nel - q0);
+  constexpr int CE = Rows<NB, double>::CE;
+  if (q0 % CE != 0) return;
+  const int n = min(CE, nel - q0);
   __syncthreads();
-  if (threadIdx.x < E) sh.ce[threadIdx.x] = 0;
+  if (threadIdx.x < CE) sh.ce[threadIdx.x] = 0;
   __syncthreads();
   for (int p = threadIdx.x; p < n * k; p += GALL) {
     const int el = p / k, t = p - el * k;
@@ -535,15 +594,16 @@ template <int NB>
 __device__ __forceinline__ void set_coefficients(GShared<NB, float>&, const double*, int, const int*, size_t, int,
                                                  int) {}
 
-// sum_t c_t V_t at one own row (of element el of the pass, own row i)
+// sum_t c_t V_t at one own row (of own element el, own row i)
 template <int NB>
 __device__ __forceinline__ double combine(const GShared<NB, double>& sh, const double*, int k, const Fix* V,
                                           size_t ldv, int el, int i) {
   FixDot acc;
   acc.clear();
+  el %= Rows<NB, double>::CE;
   const Fix* c = sh.cq + el * GM;
   const Fix* p = V + i;
-#pragma unroll 8
+#pragma unroll 16
   for (int t = 0; t < k; ++t) acc.add(c[t], p[(size_t)t * ldv]);
   return acc.result(sh.ce[el], sh.ce[el] >= (1 << 20), 0.0);
 }
@@ -628,10 +688,21 @@ __device__ __forceinline__ void givens(GShared<NB, S>& sh, int j, bool last) {
   }
 }
 
-template <int NB, class S, bool CL, int ST>
-__global__ void __launch_bounds__(GALL, 1) k_stage_gmres(const GArgs<S> a) {
+// the kernel's arguments: as they are, or a copy whose exchange buffers are replaced
+template <class S, int MODE>
+struct ArgsOf {
+  using T = const GArgs<S>&;
+};
+template <class S>
+struct ArgsOf<S, kSingle> {
+  using T = GArgs<S>;
+};
+
+template <int NB, class S, int MODE, int ST>
+__global__ void __launch_bounds__(GALL, 1) k_stage_gmres(const __grid_constant__ GArgs<S> args) {
   __shared__ GShared<NB, S> sh;
   extern __shared__ __align__(16) unsigned char dyn[];
+  typename ArgsOf<S, MODE>::T a = args;
   if (__ldcg(a.rec) != 0.0) return;  // an earlier solve of the sweep failed
   const int tid = threadIdx.x, G = gridDim.x, bi = blockIdx.x;
   const int wt = tid < GT ? tid : (1 << 30);  // first index of a worker's loop
@@ -643,15 +714,23 @@ __global__ void __launch_bounds__(GALL, 1) k_stage_gmres(const GArgs<S> a) {
   constexpr int E = Rows<NB, S>::E;
   using W = typename Wire<S>::T;
   // own slices of the basis and their exponents: shared memory, or the slices of V itself
-  const Ring<NB, S, ST> ring(reinterpret_cast<W*>(dyn));
+  const Ring<NB, S, ST> ring(dyn);
   constexpr bool VS = ST == 3;
   W* const Vo = VS ? reinterpret_cast<W*>(dyn) + Ring<NB, S, ST>::WORDS : a.V + (size_t)r0 * NB;
   const size_t ldv = VS ? (size_t)a.own_max * NB : nv;
   int* const Ve = VS ? reinterpret_cast<int*>(Vo + (a.m + 1) * ldv) : a.Vexp + r0;
   const size_t lde = VS ? (size_t)a.own_max : (size_t)nR;
-  Barrier<CL> bar{a.bar, 0u, &sh.ok};
-  double* const region0 = a.partial;
-  double* const region1 = a.partial + (size_t)GLD * GCTAS;
+  if constexpr (MODE == kSingle) {
+    // one CTA: the exchanged operand and the partials stay in shared memory behind the basis
+    const size_t ve_words = sizeof(S) == 8 ? (a.m + 1) * lde + ((a.m + 1) * lde & 1) : 0;
+    a.wire = reinterpret_cast<W*>(Ve + ve_words);
+    a.wexp = reinterpret_cast<int*>(a.wire + (size_t)a.ne * NB);
+  }
+  Barrier<MODE> bar{a.bar, 0u, &sh.ok};
+  // CTA partials, rs words from one output to the next
+  constexpr int rs = MODE == kSingle ? 1 : GCTAS;
+  double* const region0 = MODE == kSingle ? sh.single[0] : a.partial;
+  double* const region1 = MODE == kSingle ? sh.single[1] : a.partial + (size_t)GLD * GCTAS;
   S* const yo = a.y + (size_t)r0 * NB;
   const Lane<NB> ln;
   const W* const rowI = first_row_of<NB, S>(a, i0, i1);
@@ -690,7 +769,7 @@ __global__ void __launch_bounds__(GALL, 1) k_stage_gmres(const GArgs<S> a) {
   for (bool first = true; alive; first = false) {
     // ---- residual of the reduced system: z = b_I - B_IR y, r = b_R - y - B_RR y - B_RI z
     if (guess) {
-      alive = rows_product<NB, S, ST>(a, sh, ring, i0, i1, rowI, rowR, wait, idle, [&](bool on, int el, int row, int pos, S s) {
+      alive = rows_product<NB, S, ST, MODE>(a, sh, ring, i0, i1, rowI, rowR, wait, idle, [&](bool on, int el, int row, int pos, S s) {
         publish<NB, S>(a, sh, turn, on, el, row, pos, on ? rhs(pos, row) - s : S(0), true);
       });
     } else {
@@ -715,7 +794,7 @@ __global__ void __launch_bounds__(GALL, 1) k_stage_gmres(const GArgs<S> a) {
       bb = (double)t[0];
     }
     bar.arrive();
-    alive = rows_product<NB, S, ST>(a, sh, ring, r0, r1, rowR, rowI, wait, idle, [&](bool on, int el, int row, int pos, S s) {
+    alive = rows_product<NB, S, ST, MODE>(a, sh, ring, r0, r1, rowR, rowI, wait, idle, [&](bool on, int el, int row, int pos, S s) {
       publish<NB, S>(a, sh, turn, on, el, row, pos, on ? rhs(pos, row) - yo[(pos - r0) * NB + row] - s : S(0), false,
                      Vo, Ve, pos - r0);
     });
@@ -725,12 +804,12 @@ __global__ void __launch_bounds__(GALL, 1) k_stage_gmres(const GArgs<S> a) {
     if (first && tid == 0) {
       double s = 0.0;
       for (int w = 0; w < GW; ++w) s += sh.coef[w];
-      region0[GCTAS + bi] = s;
+      region0[rs + bi] = s;
     }
-    cta_dots<NB>(Vo, Ve, ldv, lde, 0, 0, nel, region0);
+    cta_dots<NB>(Vo, Ve, ldv, lde, 0, 0, nel, region0, rs, sh.dpart);
     bar.arrive();
     if (!(alive = bar.wait())) break;
-    sum_partials(first ? 2 : 1, region0, sh.red);
+    sum_partials<MODE>(first ? 2 : 1, region0, sh.red);
     if (tid == 0) {
       const double beta = sqrt(fmax(sh.red[0], 0.0));
       if (first) sh.tol = fmax(a.rtol * sqrt(fmax(sh.red[1], 0.0)), a.atol);
@@ -753,7 +832,7 @@ __global__ void __launch_bounds__(GALL, 1) k_stage_gmres(const GArgs<S> a) {
         W* const slot = Vo + (size_t)(j + 1) * ldv;   // w, then v_{j+1}
         int* const slot_e = Ve + (size_t)(j + 1) * lde;
         // ---- z = -B_IR v_j; the Givens update of the step before on the scalar warp meanwhile
-        alive = rows_product<NB, S, ST>(
+        alive = rows_product<NB, S, ST, MODE>(
             a, sh, ring, i0, i1, rowI, rowR, wait,
             [&] {
               if (j > 0) givens<NB, S>(sh, j - 1, total + j >= a.maxit);
@@ -763,11 +842,11 @@ __global__ void __launch_bounds__(GALL, 1) k_stage_gmres(const GArgs<S> a) {
         bar.arrive();
         // ---- w = B_RR v_j + B_RI z, unless the step before was the last
         bool stopped = false;
-        alive = rows_product<NB, S, ST>(
+        alive = rows_product<NB, S, ST, MODE>(
             a, sh, ring, r0, r1, rowR, rowI,
             [&] {
               if (!bar.wait()) return false;
-              if constexpr (CL) __syncthreads();
+              if constexpr (MODE == kClusters) __syncthreads();
               stopped = j > 0 && sh.stop != 0;
               return !stopped;
             },
@@ -786,10 +865,10 @@ __global__ void __launch_bounds__(GALL, 1) k_stage_gmres(const GArgs<S> a) {
         k = j + 1;
         __syncthreads();
         // ---- projections and |w|^2
-        cta_dots<NB>(Vo, Ve, ldv, lde, k, 0, nel, region1);
+        cta_dots<NB>(Vo, Ve, ldv, lde, k, 0, nel, region1, rs, sh.dpart);
         bar.arrive();
         if (!(alive = bar.wait())) break;
-        sum_partials(k + 1, region1, sh.red);
+        sum_partials<MODE>(k + 1, region1, sh.red);
         bool again = false;
         for (int pass = 0;; ++pass) {
           // coefficients so far, |h|^2 of this pass, and the norm it leaves
@@ -816,21 +895,21 @@ __global__ void __launch_bounds__(GALL, 1) k_stage_gmres(const GArgs<S> a) {
           if (!again) break;
           passes([&](int q) { set_coefficients<NB>(sh, sh.red, k, Ve, lde, q, nel); },
                  [&](bool on, int oe, int i) {
-                   const S s = on && pass < 2 ? entry(slot, slot_e, oe, i) - combine<NB>(sh, sh.red, k, Vo, ldv, ln.el, i)
+                   const S s = on && pass < 2 ? entry(slot, slot_e, oe, i) - combine<NB>(sh, sh.red, k, Vo, ldv, oe, i)
                                               : S(0);
                    publish<NB, S>(a, sh, turn, on, ln.el, ln.row, r0 + oe, s, false, slot, slot_e, oe);
                  });
           __syncthreads();
           double* region = pass == 0 ? region0 : region1;
-          if (pass == 0) cta_dots<NB>(Vo, Ve, ldv, lde, k, 0, nel, region);
-          else cta_dots<NB>(Vo, Ve, ldv, lde, k, k, nel, region + (size_t)k * GCTAS);
+          if (pass == 0) cta_dots<NB>(Vo, Ve, ldv, lde, k, 0, nel, region, rs, sh.dpart);
+          else cta_dots<NB>(Vo, Ve, ldv, lde, k, k, nel, region + (size_t)k * rs, rs, sh.dpart);
           bar.arrive();
           if (!(alive = bar.wait())) break;
           if (pass == 0) {
-            sum_partials(k + 1, region, sh.red);
+            sum_partials<MODE>(k + 1, region, sh.red);
           } else {
             for (int t = wt; t < k; t += GT) sh.red[t] = 0.0;
-            sum_partials(1, region + (size_t)k * GCTAS, sh.red + k);
+            sum_partials<MODE>(1, region + (size_t)k * rs, sh.red + k);
           }
         }
         if (!alive) break;
@@ -838,7 +917,7 @@ __global__ void __launch_bounds__(GALL, 1) k_stage_gmres(const GArgs<S> a) {
         const S inv = S(sh.inv);
         passes([&](int q) { set_coefficients<NB>(sh, sh.red, k, Ve, lde, q, nel); },
                [&](bool on, int oe, int i) {
-                 const S s = on ? (entry(slot, slot_e, oe, i) - combine<NB>(sh, sh.red, k, Vo, ldv, ln.el, i)) * inv
+                 const S s = on ? (entry(slot, slot_e, oe, i) - combine<NB>(sh, sh.red, k, Vo, ldv, oe, i)) * inv
                                 : S(0);
                  publish<NB, S>(a, sh, turn, on, ln.el, ln.row, r0 + oe, s, true, slot, slot_e, oe);
                });
@@ -874,7 +953,7 @@ __global__ void __launch_bounds__(GALL, 1) k_stage_gmres(const GArgs<S> a) {
            [&](bool on, int oe, int i) {
              S s = S(0);
              if (on) {
-               s = yo[i] + combine<NB>(sh, sh.coef, k, Vo, ldv, ln.el, i);
+               s = yo[i] + combine<NB>(sh, sh.coef, k, Vo, ldv, oe, i);
                yo[i] = s;
                if (a.ywarm) a.ywarm[(size_t)r0 * NB + i] = s;
              }
@@ -886,7 +965,7 @@ __global__ void __launch_bounds__(GALL, 1) k_stage_gmres(const GArgs<S> a) {
   }
   if (alive && flag != 4) {
     // ---- y_I = b_I - B_IR y_R, then x = D y element by element
-    alive = rows_product<NB, S, ST>(a, sh, ring, i0, i1, rowI, nullptr, wait, idle, [&](bool on, int, int row, int pos, S s) {
+    alive = rows_product<NB, S, ST, MODE>(a, sh, ring, i0, i1, rowI, nullptr, wait, idle, [&](bool on, int, int row, int pos, S s) {
       if (on) a.y[(size_t)pos * NB + row] = rhs(pos, row) - s;
     });
   }
@@ -924,56 +1003,70 @@ __global__ void __launch_bounds__(GALL, 1) k_stage_gmres(const GArgs<S> a) {
 struct GSetup {
   cudaError_t err = cudaSuccess;
   int sms = 0;
+  int dyn[4] = {0, 0, 0, 0};  // dynamic shared memory of the four variants
 };
 
 template <int NB, class S>
 cudaError_t launch_gmres(GArgs<S>& a, cudaStream_t st) {
+  const void* const kernels[4] = {(const void*)k_stage_gmres<NB, S, kGrid, 3>, (const void*)k_stage_gmres<NB, S, kGrid, 6>,
+                                  (const void*)k_stage_gmres<NB, S, kClusters, 3>,
+                                  (const void*)k_stage_gmres<NB, S, kSingle, 3>};
   // one device per process (see pp_create); thread-safe static initialization
-  static const GSetup setup = [] {
+  static const GSetup setup = [&] {
     GSetup s;
     int dev = 0;
     s.err = cudaGetDevice(&dev);
     if (s.err == cudaSuccess) s.err = cudaDeviceGetAttribute(&s.sms, cudaDevAttrMultiProcessorCount, dev);
-    auto room = [&](auto* kernel) {
-      if (s.err == cudaSuccess)
-        s.err = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kDynSmemMax);
-    };
-    room(k_stage_gmres<NB, S, false, 3>);
-    room(k_stage_gmres<NB, S, false, 6>);
-    room(k_stage_gmres<NB, S, true, 3>);
+    for (int k = 0; k < 4; ++k) {
+      cudaFuncAttributes at;
+      if (s.err == cudaSuccess) s.err = cudaFuncGetAttributes(&at, kernels[k]);
+      if (s.err != cudaSuccess) break;
+      s.dyn[k] = kSmemMax - (int)at.sharedSizeBytes;
+      s.err = cudaFuncSetAttribute(kernels[k], cudaFuncAttributeMaxDynamicSharedMemorySize, s.dyn[k]);
+    }
     return s;
   }();
   if (setup.err != cudaSuccess) return setup.err;
-  // the basis beside the short ring when both fit, else the deep ring
   const size_t short_bytes = sizeof(S) * Ring<NB, S, 3>::WORDS, deep_bytes = sizeof(S) * Ring<NB, S, 6>::WORDS;
+  // the short ring and the basis slices of `own` elements
   auto basis_bytes = [&](int own) {
-    return (size_t)(a.m + 1) * own * (sizeof(S) * NB + (sizeof(S) == 8 ? sizeof(int) : 0));
+    return short_bytes + (size_t)(a.m + 1) * own * (sizeof(S) * NB + (sizeof(S) == 8 ? sizeof(int) : 0)) + 8;
   };
-  auto fits = [&](int own) { return short_bytes + basis_bytes(own) <= (size_t)kDynSmemMax; };
-  const bool cluster = (int64_t)a.nR * NB <= kClusterRows && fits((a.nR + kCluster - 1) / kCluster);
-  const int G = cluster ? kCluster : std::min(std::min(setup.sms, GCTAS), a.nR);
+  // One CTA while the kept rows are one pass and everything fits its shared memory: a step then has no
+  // barrier but the CTA's own (32 triangles, p = 1: 11.6 us a step against 13.0 us with the cluster; 64
+  // triangles would take two passes, 15.1 us against 11.9 us).  A cluster of 8 up to kClusterRows, one
+  // pass each.  Otherwise all SMs, the basis beside the short ring when both fit, else the deep ring.
+  const size_t single_bytes = basis_bytes(a.nR) + (size_t)a.ne * (sizeof(S) * NB + sizeof(int));
+  const int cl_own = (a.nR + kCluster - 1) / kCluster;
+  int k, G;
+  if (a.nR <= Rows<NB, S>::E && single_bytes <= (size_t)setup.dyn[3]) {
+    k = 3;
+    G = 1;
+  } else if ((int64_t)a.nR * NB <= kClusterRows && basis_bytes(cl_own) <= (size_t)setup.dyn[2]) {
+    k = 2;
+    G = kCluster;
+  } else {
+    G = std::min(std::min(setup.sms, GCTAS), a.nR);
+    k = basis_bytes((a.nR + G - 1) / G) <= (size_t)setup.dyn[0] ? 0 : 1;
+  }
   a.own_max = (a.nR + G - 1) / G;
-  const bool v_smem = fits(a.own_max);
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3(G);
   cfg.blockDim = dim3(GALL);
-  cfg.dynamicSmemBytes = v_smem ? short_bytes + basis_bytes(a.own_max) : deep_bytes;
+  cfg.dynamicSmemBytes = k == 3 ? single_bytes : k == 1 ? deep_bytes : basis_bytes(a.own_max);
   cfg.stream = st;
   cudaLaunchAttribute at{};
-  if (cluster) {
-    at.id = cudaLaunchAttributeClusterDimension;
+  at.id = k == 2 ? cudaLaunchAttributeClusterDimension : cudaLaunchAttributeCooperative;
+  if (k == 2) {
     at.val.clusterDim.x = kCluster;
     at.val.clusterDim.y = at.val.clusterDim.z = 1;
   } else {
-    at.id = cudaLaunchAttributeCooperative;
     at.val.cooperative = 1;
   }
   cfg.attrs = &at;
-  cfg.numAttrs = 1;
-  const GArgs<S> args = a;
-  if (cluster) return cudaLaunchKernelEx(&cfg, k_stage_gmres<NB, S, true, 3>, args);
-  return v_smem ? cudaLaunchKernelEx(&cfg, k_stage_gmres<NB, S, false, 3>, args)
-                : cudaLaunchKernelEx(&cfg, k_stage_gmres<NB, S, false, 6>, args);
+  cfg.numAttrs = k == 3 ? 0 : 1;
+  void* params[] = {&a};
+  return cudaLaunchKernelExC(&cfg, kernels[k], params);
 }
 
 }  // namespace

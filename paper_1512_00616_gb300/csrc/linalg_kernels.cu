@@ -340,15 +340,19 @@ __global__ void __launch_bounds__(256)
 // block diagonal (Ainv its inverse) and BN, BT zero on boundary faces.
 // FP64 blocks are written as fixed-point words (fixed.cuh), one exponent per block row in EN / ET
 // [e][f][row]; FP32 blocks as floats (EN, ET unused).
+// FP64: both factors go to fixed point as well (one exponent per row of P and column of Q) and an
+// entry is one exact integer sum, two FP64 instructions instead of nb: with FP64 FMAs the kernel sat
+// at the FP64 pipe's floor (2048 triangles, p = 3: 1.06 ms a stage, normal and transposed blocks).
+// Rows are padded to an odd number of words, so that lanes over rows read different banks.
 template <int NB, class S>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, 2)
     k_fold_blocks(DevMesh m, const S* __restrict__ J, const S* __restrict__ Ainv, double c, FoldOut<S> out) {
   extern __shared__ __align__(16) unsigned char fsm_raw[];
-  __shared__ int rmax[NB];
-  S* P = reinterpret_cast<S*>(fsm_raw);
-  S* Q = P + NB * NB;
-  constexpr int nb2 = NB * NB;
+  __shared__ int emax[3][NB];  // rows of P, columns of Q, rows of the product
+  constexpr int nb2 = NB * NB, LD = NB + 1;
   constexpr int NV = (nb2 + 255) / 256;
+  S* P = reinterpret_cast<S*>(fsm_raw);  // [row][k]
+  S* Q = P + NB * LD;                    // [column][k]
   const int e = blockIdx.x / 3, f = blockIdx.x - 3 * (blockIdx.x / 3);
   const int e2 = m.nbr[3 * e + f];
   const size_t blk = ((size_t)e * 3 + f) * nb2;
@@ -365,46 +369,65 @@ __global__ void __launch_bounds__(256)
     const S* Pg = pass == 0 ? J + ((size_t)e * 4 + 1 + f) * nb2 : Ainv + (size_t)e2 * nb2;
     const S* Qg = pass == 0 ? Ainv + (size_t)e2 * nb2 : J + ((size_t)e2 * 4 + 1 + m.nbrface[3 * e + f]) * nb2;
     __syncthreads();
-    for (int i = threadIdx.x; i < nb2; i += 256) {
-      P[i] = Pg[i];
-      Q[i] = Qg[i];
-    }
-    if (threadIdx.x < NB) rmax[threadIdx.x] = 0;
+    if (threadIdx.x < NB) emax[0][threadIdx.x] = emax[1][threadIdx.x] = emax[2][threadIdx.x] = 0;
     __syncthreads();
+    // column-major in: entry (row i % NB, column i / NB)
+#pragma unroll
+    for (int t = 0; t < NV; ++t) {
+      const int i = threadIdx.x + 256 * t, r = i % NB, k = i / NB;
+      if (i >= nb2) continue;
+      const S pv = Pg[i], qv = Qg[i];
+      P[r * LD + k] = pv;
+      Q[k * LD + r] = qv;
+      if constexpr (sizeof(S) == 8) {
+        atomicMax(&emax[0][r], fix_exponent(pv));
+        atomicMax(&emax[1][k], fix_exponent(qv));
+      }
+    }
+    __syncthreads();
+    if constexpr (sizeof(S) == 8) {
+#pragma unroll
+      for (int t = 0; t < NV; ++t) {
+        const int i = threadIdx.x + 256 * t, r = i % NB, k = i / NB;
+        if (i >= nb2) continue;
+        reinterpret_cast<Fix*>(P)[r * LD + k] = fix_encode(P[r * LD + k], emax[0][r]);
+        reinterpret_cast<Fix*>(Q)[k * LD + r] = fix_encode(Q[k * LD + r], emax[1][k]);
+      }
+      __syncthreads();
+    }
     S val[NV];
 #pragma unroll
     for (int t = 0; t < NV; ++t) {
-      const int idx = threadIdx.x + 256 * t;
+      // output (r, cc) of the block that is stored: entry (r, cc) of P Q (pass 0) or of (P Q)^T
+      const int idx = threadIdx.x + 256 * t, cc = idx / NB, r = idx - cc * NB;
       if (idx >= nb2) continue;
-      const int cc = idx / NB, r = idx - cc * NB;  // output (r, cc), column-major
-      S a0 = S(0), a1 = S(0);
-      if (pass == 0) {
-        // (P Q)(r, cc) = sum_k P(r, k) Q(k, cc)
-#pragma unroll 8
-        for (int k = 0; k < NB; k += 2) {
-          a0 += P[k * NB + r] * Q[cc * NB + k];
-          a1 += P[(k + 1) * NB + r] * Q[cc * NB + k + 1];
-        }
+      const int pr = pass == 0 ? r : cc, qc = pass == 0 ? cc : r;
+      if constexpr (sizeof(S) == 8) {
+        const Fix *p = reinterpret_cast<const Fix*>(P) + pr * LD, *q = reinterpret_cast<const Fix*>(Q) + qc * LD;
+        FixDot acc;
+        acc.clear();
+#pragma unroll 12
+        for (int k = 0; k < NB; ++k) acc.add(p[k], q[k]);
+        val[t] = -c * acc.result(emax[0][pr], emax[1][qc]);
+        atomicMax(&emax[2][r], fix_exponent(val[t]));
       } else {
-        // ((P Q)^T)(r, cc) = (P Q)(cc, r) = sum_k P(cc, k) Q(k, r)
-#pragma unroll 8
+        S a0 = S(0), a1 = S(0);
+#pragma unroll 12
         for (int k = 0; k < NB; k += 2) {
-          a0 += P[k * NB + cc] * Q[r * NB + k];
-          a1 += P[(k + 1) * NB + cc] * Q[r * NB + k + 1];
+          a0 += P[pr * LD + k] * Q[qc * LD + k];
+          a1 += P[pr * LD + k + 1] * Q[qc * LD + k + 1];
         }
+        dst[blk + fold_index<S>(NB, r, cc)] = S(-c) * (a0 + a1);
       }
-      val[t] = S(-c) * (a0 + a1);
-      if constexpr (sizeof(S) == 8) atomicMax(&rmax[r], fix_exponent(val[t]));
-      else dst[blk + idx] = val[t];
     }
     if constexpr (sizeof(S) == 8) {
       __syncthreads();
 #pragma unroll
       for (int t = 0; t < NV; ++t) {
         const int idx = threadIdx.x + 256 * t;
-        if (idx < nb2) dst[blk + idx] = fix_encode(val[t], rmax[idx % NB]);
+        if (idx < nb2) dst[blk + fold_index<S>(NB, idx % NB, idx / NB)] = fix_encode(val[t], emax[2][idx % NB]);
       }
-      if (threadIdx.x < NB) exps[((size_t)e * 3 + f) * NB + threadIdx.x] = rmax[threadIdx.x];
+      if (threadIdx.x < NB) exps[((size_t)e * 3 + f) * NB + threadIdx.x] = emax[2][threadIdx.x];
     }
   }
 }
@@ -423,8 +446,8 @@ __global__ void __launch_bounds__(64)
     const size_t blk = (size_t)e * 3 + f;
     for (int c = 0; c < nb; ++c) {
       S b;
-      if constexpr (sizeof(S) == 8) b = fix_decode(B[blk * nb * nb + (size_t)c * nb + r], E[blk * nb + r]);
-      else b = B[blk * nb * nb + (size_t)c * nb + r];
+      if constexpr (sizeof(S) == 8) b = fix_decode(B[blk * nb * nb + fold_index<S>(nb, r, c)], E[blk * nb + r]);
+      else b = B[blk * nb * nb + fold_index<S>(nb, r, c)];
       s += b * x[(size_t)e2 * nb + c];
     }
   }
@@ -1223,7 +1246,7 @@ template <class S>
 cudaError_t launch_fold_blocks(const DevMesh& m, int nb, const S* J, const S* Ainv, double c, const FoldOut<S>& out,
                                cudaStream_t st) {
   ProfScope ps(PP_K_FOLD, st);
-  const size_t smem = sizeof(S) * 2 * nb * nb;
+  const size_t smem = sizeof(S) * 2 * nb * (nb + 1);
 #define PP_FOLD(NBV)                                                                                     \
   case NBV: {                                                                                            \
     static const cudaError_t attr =                                                                      \

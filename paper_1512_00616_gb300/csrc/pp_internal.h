@@ -216,6 +216,17 @@ struct DevMesh {
 // All take the stream explicitly and return the launch error (cudaSuccess on success).
 cudaError_t launch_residual(const DevMesh& m, const DevTables& tb, const Phys& ph, const FrameT<double>& fr,
                             const double* u, double* r, cudaStream_t st);
+// Stage Newton residual R = M k - dt r(u) at u = base + aii k, which is written to us; sums: per
+// element |R|^2, |M u|^2 [ne][2]
+struct StageNewton {
+  const double* base;
+  const double* k;
+  double aii, dt;
+  double* us;
+  double* sums;
+};
+cudaError_t launch_stage_residual(const DevMesh& m, const DevTables& tb, const Phys& ph, const FrameT<double>& fr,
+                                  const StageNewton& nw, double* R, cudaStream_t st);
 // per element kappa . dr/ds [ne][3] for three seeds s (the frame carries the derivatives)
 cudaError_t launch_residual_dframe(const DevMesh& m, const DevTables& tb, const Phys& ph, const FrameT<DualV<3>>& fr,
                                    const double* u, const double* kappa, double* per_elem, cudaStream_t st);
@@ -352,10 +363,12 @@ int stage_gmres_barrier_words();
 // BN = -c J_off Ainv_nbr and BT = (-c Ainv_nbr J_off,nbr)^T (3 blocks per element each; BT may
 // be null): the block-Jacobi preconditioner folded into the stage operator.  FP64 blocks are
 // stored as fixed-point words (fixed.cuh) with one exponent per block row (EN, ET).
+// The blocks interleave groups of VW columns, 16 bytes per row and group (fold_index).
 struct Fix;
 template <class S>
 struct FoldOut {
   using W = float;
+  static constexpr int VW = 4;
   float* BN;
   float* BT;
   int* EN = nullptr;
@@ -364,11 +377,17 @@ struct FoldOut {
 template <>
 struct FoldOut<double> {
   using W = Fix;
+  static constexpr int VW = 2;
   Fix* BN;
   Fix* BT;
   int* EN;
   int* ET;
 };
+// word of entry (row, col) in a folded nb x nb block
+template <class S>
+PP_HD int fold_index(int nb, int row, int col) {
+  return (col / FoldOut<S>::VW * nb + row) * FoldOut<S>::VW + col % FoldOut<S>::VW;
+}
 template <class S>
 cudaError_t launch_fold_blocks(const DevMesh& m, int nb, const S* J, const S* Ainv, double c, const FoldOut<S>& out,
                                cudaStream_t st);
