@@ -141,7 +141,11 @@ __device__ __forceinline__ void fix_put(double* w, int* ge, double v) {
 __device__ __forceinline__ void fix_enc(double* w, int ge) { *reinterpret_cast<Fix*>(w) = fix_encode(*w, ge); }
 
 // ------------------------------------------------------------------------ residual
-// T = double: the residual r.  T = DualV<3>: kappa . dr/ds for three motion seeds s carried by the
+// T = double: the residual r, or (NEWTON) the residual of a stage's Newton iteration,
+//   u = base + a_ii k (written, with its neighbours' values formed on the way in),
+//   R = M k - dt r(u), and per element |R|^2 and |M u|^2,
+// in place of seven launches (two vector combinations, the residual, two mass products, two norms).
+// T = DualV<3>: kappa . dr/ds for three motion seeds s carried by the
 // frame, summed per element (dr itself is not written).
 //
 // A CTA takes groups of elements and deals (element, point) and (element, row) tasks to its threads, so
@@ -151,7 +155,7 @@ __device__ __forceinline__ void fix_enc(double* w, int ge) { *reinterpret_cast<F
 // (fixed.cuh); what remains in FP64 are the fluxes.
 // Phases: A jumps U_hat - U- at the face points; B volume points with the element's own liftings;
 // C face points with the lifted gradient of the side that supplies the viscous flux; D projection.
-template <int PD, class T>
+template <int PD, class T, bool NEWTON>
 struct Res {
   static constexpr int NP = (PD + 1) * (PD + 2) / 2, NB = 4 * NP, NF = PD + 2, NV = NF * NF, F3 = 3 * NF;
   static constexpr bool VAL = sizeof(T) == sizeof(double);
@@ -161,32 +165,33 @@ struct Res {
   static constexpr int EB = THREADS / NV;                     // most elements of a group
   static constexpr int LP = NP | 1;                           // odd table rows: no bank conflicts
   // shared memory in 8-byte words: tables, then per element
-  static constexpr int pv = 0, dv = pv + NV * LP, pf = dv + 2 * NV * LP, df = pf + F3 * LP, elems = df + 2 * F3 * LP;
+  static constexpr int pv = 0, dv = pv + NV * LP, pf = dv + 2 * NV * LP, df = pf + F3 * LP,
+                       ms = df + 2 * F3 * LP, elems = ms + (NEWTON ? NP * LP : 0);
   static constexpr int su = 0, Uf = su + 4 * NB, Js = Uf + F3 * 8, G = Js + F3 * 4 * W, H = G + NC * 4 * 2 * NV,
-                       per = (H + NC * 4 * F3) | 1;
+                       ks = H + NC * 4 * F3, per = (ks + (NEWTON ? NB : 0)) | 1;
   static constexpr int words = elems + EB * per;
 };
-template <int PD, class T>
+template <int PD, class T, bool NEWTON>
 struct ResExp {
-  using L = Res<PD, T>;
-  int tab[4];
-  int u[L::EB][4][4], G[L::EB][L::NC][4], H[L::EB][L::NC][4];
+  using L = Res<PD, T, NEWTON>;
+  int tab[5];
+  int u[L::EB][4][4], k[L::EB][4], G[L::EB][L::NC][4], H[L::EB][L::NC][4];
 };
 
 __device__ __forceinline__ double part(double a, int) { return a; }
 __device__ __forceinline__ double part(const DualV<3>& a, int k) { return a.d[k]; }
 
-template <int PD, class T>
-__global__ void __launch_bounds__(Res<PD, T>::THREADS, 2)
+template <int PD, class T, bool NEWTON>
+__global__ void __launch_bounds__(Res<PD, T, NEWTON>::THREADS, 2)
     k_residual(DevMesh m, DevTables tb, Phys ph, FrameT<T> fr, const double* __restrict__ u,
-               const double* __restrict__ kappa, double* __restrict__ out, int eb) {
-  using L = Res<PD, T>;
+               const double* __restrict__ kappa, double* __restrict__ out, StageNewton nw, int eb) {
+  using L = Res<PD, T, NEWTON>;
   constexpr int NP = L::NP, NB = L::NB, NF = L::NF, NV = L::NV, F3 = L::F3, NT = L::THREADS, NC = L::NC, LP = L::LP;
   extern __shared__ double smem[];
-  __shared__ ResExp<PD, T> ex;
+  __shared__ ResExp<PD, T, NEWTON> ex;
   const int tid = threadIdx.x;
   // tables, one exponent each
-  if (tid < 4) ex.tab[tid] = 0;
+  if (tid < 5) ex.tab[tid] = 0;
   __syncthreads();
   auto each_table = [&](auto&& f) {
     for (int i = tid; i < NV * NP; i += NT) {
@@ -201,6 +206,8 @@ __global__ void __launch_bounds__(Res<PD, T>::THREADS, 2)
       f(smem + L::df + q * LP + j, &ex.tab[3], tb.dphi_f + 2 * i);
       f(smem + L::df + (F3 + q) * LP + j, &ex.tab[3], tb.dphi_f + 2 * i + 1);
     }
+    if constexpr (NEWTON)
+      for (int i = tid; i < NP * NP; i += NT) f(smem + L::ms + i / NP * LP + i % NP, &ex.tab[4], tb.Mref + i);
   };
   each_table([](double* w, int* ge, const double* v) { fix_put(w, ge, *v); });
   __syncthreads();
@@ -210,7 +217,8 @@ __global__ void __launch_bounds__(Res<PD, T>::THREADS, 2)
   for (int e0 = blockIdx.x * eb; e0 < m.ne; e0 += gridDim.x * eb) {
     const int n = min(eb, m.ne - e0);
     __syncthreads();
-    for (int k = tid; k < (int)((sizeof(ex.u) + sizeof(ex.G) + sizeof(ex.H)) / 4); k += NT) (&ex.u[0][0][0])[k] = 0;
+    for (int k = tid; k < (int)((sizeof(ex.u) + sizeof(ex.k) + sizeof(ex.G) + sizeof(ex.H)) / 4); k += NT)
+      (&ex.u[0][0][0])[k] = 0;
     __syncthreads();
     for (int idx = tid; idx < n * 4 * NB; idx += NT) {
       const int el = idx / (4 * NB), r = idx - el * 4 * NB, slot = r / NB, k = r - slot * NB;
@@ -219,12 +227,25 @@ __global__ void __launch_bounds__(Res<PD, T>::THREADS, 2)
         const int nn = m.nbr[3 * src + slot - 1];
         src = nn >= 0 ? nn : src;
       }
-      fix_put(smem + L::elems + el * L::per + L::su + r, &ex.u[el][slot][k / NP], u[(size_t)src * NB + k]);
+      const size_t at = (size_t)src * NB + k;
+      double v;
+      if constexpr (NEWTON) {
+        const double kv = nw.k[at];
+        v = nw.base[at] + nw.aii * kv;
+        if (slot == 0) {
+          nw.us[at] = v;
+          fix_put(smem + L::elems + el * L::per + L::ks + k, &ex.k[el][k / NP], kv);
+        }
+      } else {
+        v = u[at];
+      }
+      fix_put(smem + L::elems + el * L::per + L::su + r, &ex.u[el][slot][k / NP], v);
     }
     __syncthreads();
     for (int idx = tid; idx < n * 4 * NB; idx += NT) {
       const int el = idx / (4 * NB), r = idx - el * 4 * NB, slot = r / NB, k = r - slot * NB;
       fix_enc(smem + L::elems + el * L::per + L::su + r, ex.u[el][slot][k / NP]);
+      if (NEWTON && slot == 0) fix_enc(smem + L::elems + el * L::per + L::ks + k, ex.k[el][k / NP]);
     }
     __syncthreads();
     // phase A: both traces and the jumps
@@ -353,7 +374,17 @@ __global__ void __launch_bounds__(Res<PD, T>::THREADS, 2)
         acc[c] = -fix_dot<F3>(fix(L::pf) + i, H, ex.tab[2], ex.H[el][c][a], 0.0, LP);
         acc[c] = fix_dot<2 * NV>(fix(L::dv) + i, G, ex.tab[1], ex.G[el][c][a], acc[c], LP);
       }
-      if constexpr (L::VAL) {
+      if constexpr (NEWTON) {
+        const double detB = m.detB[e0 + el];
+        const Fix* mi = fix(L::ms) + i * LP;
+        const double mk = detB * fix_dot<NP>(mi, reinterpret_cast<const Fix*>(S + L::ks) + a * NP, ex.tab[4], ex.k[el][a], 0.0);
+        const double mu = detB * fix_dot<NP>(mi, reinterpret_cast<const Fix*>(S + L::su) + a * NP, ex.tab[4], ex.u[el][0][a], 0.0);
+        const double R = mk - nw.dt * acc[0];
+        out[(size_t)(e0 + el) * NB + o] = R;
+        // in place of the neighbours' states
+        S[L::su + NB + o] = R;
+        S[L::su + 2 * NB + o] = mu;
+      } else if constexpr (L::VAL) {
         out[(size_t)(e0 + el) * NB + o] = acc[0];
       } else {
         // kappa times the rows, in place of the states
@@ -362,18 +393,22 @@ __global__ void __launch_bounds__(Res<PD, T>::THREADS, 2)
         for (int c = 0; c < NC; ++c) S[L::su + c * NB + o] = kp * acc[c];
       }
     }
-    if constexpr (!L::VAL) {
+    if constexpr (!L::VAL || NEWTON) {
       __syncthreads();
-      // eight lanes per (element, seed), then a butterfly over them
+      // per-element sums: eight lanes per (element, seed or norm), then a butterfly over them
+      constexpr int NS = NEWTON ? 2 : 3;
+      double* const sums = NEWTON ? nw.sums : out;
       const int l = tid & 7;
-      for (int g8 = tid >> 3; g8 < (n * NC + 3) / 4 * 4; g8 += NT / 8) {
-        const int el = g8 / NC, c = g8 - el * NC;
+      for (int g8 = tid >> 3; g8 < (n * NS + 3) / 4 * 4; g8 += NT / 8) {
+        const int el = g8 / NS, c = g8 - el * NS;
         double s = 0.0;
-        if (el < n)
-          for (int o = l; o < NB; o += 8) s += smem[L::elems + el * L::per + L::su + c * NB + o];
+        if (el < n) {
+          const double* v = smem + L::elems + el * L::per + L::su + (NEWTON ? c + 1 : c) * NB;
+          for (int o = l; o < NB; o += 8) s += NEWTON ? v[o] * v[o] : v[o];
+        }
 #pragma unroll
         for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (l == 0 && el < n) out[(size_t)(e0 + el) * NC + c] = s;
+        if (l == 0 && el < n) sums[(size_t)(e0 + el) * NS + c] = s;
       }
     }
   }
@@ -1106,10 +1141,11 @@ __global__ void __launch_bounds__(RES_WARPS * 32)
 
 static int res_blocks(int ne) { return (ne + RES_WARPS - 1) / RES_WARPS; }
 
-template <int PD, class T>
+template <int PD, class T, bool NEWTON = false>
 static cudaError_t run_residual(const DevMesh& m, const DevTables& tb, const Phys& ph, const FrameT<T>& fr,
-                                const double* u, const double* kappa, double* out, cudaStream_t st) {
-  using L = Res<PD, T>;
+                                const double* u, const double* kappa, double* out, cudaStream_t st,
+                                const StageNewton& nw = {}) {
+  using L = Res<PD, T, NEWTON>;
   struct Setup {
     cudaError_t err;
     int resident;
@@ -1117,10 +1153,10 @@ static cudaError_t run_residual(const DevMesh& m, const DevTables& tb, const Phy
   // one device per process (see pp_create)
   static const Setup setup = [] {
     Setup r{cudaSuccess, 0};
-    r.err = cudaFuncSetAttribute(k_residual<PD, T>, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * L::words);
+    r.err = cudaFuncSetAttribute(k_residual<PD, T, NEWTON>, cudaFuncAttributeMaxDynamicSharedMemorySize, 8 * L::words);
     if (r.err != cudaSuccess) return r;
     int per_sm = 0, dev = 0, sms = 0;
-    r.err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_residual<PD, T>, L::THREADS, 8 * L::words);
+    r.err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_residual<PD, T, NEWTON>, L::THREADS, 8 * L::words);
     if (r.err == cudaSuccess) r.err = cudaGetDevice(&dev);
     if (r.err == cudaSuccess) r.err = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     if (r.err == cudaSuccess && per_sm < 1) r.err = cudaErrorInvalidConfiguration;
@@ -1132,7 +1168,7 @@ static cudaError_t run_residual(const DevMesh& m, const DevTables& tb, const Phy
   int eb = (m.ne + setup.resident - 1) / setup.resident;
   eb = eb < 1 ? 1 : eb > L::EB ? L::EB : eb;
   const int groups = (m.ne + eb - 1) / eb, grid = groups < setup.resident ? groups : setup.resident;
-  k_residual<PD, T><<<grid, L::THREADS, 8 * L::words, st>>>(m, tb, ph, fr, u, kappa, out, eb);
+  k_residual<PD, T, NEWTON><<<grid, L::THREADS, 8 * L::words, st>>>(m, tb, ph, fr, u, kappa, out, nw, eb);
   return cudaGetLastError();
 }
 
@@ -1144,6 +1180,18 @@ cudaError_t launch_residual(const DevMesh& m, const DevTables& tb, const Phys& p
     case 2: return run_residual<2, double>(m, tb, ph, fr, u, nullptr, r, st);
     case 3: return run_residual<3, double>(m, tb, ph, fr, u, nullptr, r, st);
     case 4: return run_residual<4, double>(m, tb, ph, fr, u, nullptr, r, st);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+cudaError_t launch_stage_residual(const DevMesh& m, const DevTables& tb, const Phys& ph, const FrameT<double>& fr,
+                                  const StageNewton& nw, double* R, cudaStream_t st) {
+  ProfScope ps(PP_K_RESIDUAL, st);
+  switch (tb.p) {
+    case 1: return run_residual<1, double, true>(m, tb, ph, fr, nullptr, nullptr, R, st, nw);
+    case 2: return run_residual<2, double, true>(m, tb, ph, fr, nullptr, nullptr, R, st, nw);
+    case 3: return run_residual<3, double, true>(m, tb, ph, fr, nullptr, nullptr, R, st, nw);
+    case 4: return run_residual<4, double, true>(m, tb, ph, fr, nullptr, nullptr, R, st, nw);
     default: return cudaErrorInvalidValue;
   }
 }

@@ -436,7 +436,6 @@ int run_steps(pp_ctx* ctx, const pp_mesh* mesh, const double* mu, int n_mu, doub
   const double dt = ctx->cfg.T / Nt;
   double* k[3] = {work_vec(ctx, 1), work_vec(ctx, 2), work_vec(ctx, 3)};
   double* base = work_vec(ctx, 4);
-  double* r = work_vec(ctx, 5);
   double* R = work_vec(ctx, 6);
   double* dk = work_vec(ctx, 7);
   // chord Newton: all stages share a_ii = gamma, so the stored matrix of the previous
@@ -464,14 +463,16 @@ int run_steps(pp_ctx* ctx, const pp_mesh* mesh, const double* mu, int n_mu, doub
       int backtracks = 0;
       bool converged = false, refresh = !have_nview;
       for (int it = 0; it <= ctx->cfg.newton_maxit; ++it) {
-        PP_TRY(lincomb(ctx, n, us, {1.0, ctx->A[i][i]}, {base, k[i]}));
-        PP_CK(launch_residual(m, ctx->tb, ctx->ph, fr, us, r, ctx->stream));
-        PP_CK(launch_stage_matvec<double>(m, ctx->tb, nullptr, 1.0, 0.0, k[i], R, 0, ctx->stream));
-        PP_TRY(lincomb(ctx, n, R, {1.0, -dt}, {R, r}));
-        double rn2, mun;
-        PP_TRY(host_dot<double>(ctx, n, R, R, &rn2));
+        // us = base + a_ii k, R = M k - dt r(us), |R|^2 and |M us|^2 with the record of the solves so far
+        PP_CK(launch_stage_residual(m, ctx->tb, ctx->ph, fr, {base, k[i], ctx->A[i][i], dt, us, ctx->d_elem}, R,
+                                    ctx->stream));
+        PP_CK(launch_colsum(mesh->ne, 2, ctx->d_elem, ctx->d_scalar + kDot - 1, ctx->d_partial, ctx->d_counter,
+                            ctx->stream));
+        PP_CK(cudaMemcpyAsync(ctx->h_scalar + kDot - 1, ctx->d_scalar + kDot - 1, 4 * sizeof(double),
+                              cudaMemcpyDeviceToHost, ctx->stream));
+        PP_CK(cudaStreamSynchronize(ctx->stream));
         PP_TRY(take_record(ctx, &ctx->last_gmres_iters));
-        double rn = std::sqrt(rn2);
+        const double rn = std::sqrt(ctx->h_scalar[kDot - 1]), mun = std::sqrt(ctx->h_scalar[kDot]);
         // backtracking safeguard: a step that made the residual non-finite or larger is halved
         if (it > 0 && (!std::isfinite(rn) || rn > prev_res) && backtracks < 8) {
           alpha *= 0.5;
@@ -483,8 +484,7 @@ int run_steps(pp_ctx* ctx, const pp_mesh* mesh, const double* mu, int n_mu, doub
         if (!std::isfinite(rn)) return set_error(ctx, PP_ENAN, "non-finite stage residual");
         if (it > 0 && rn > 0.25 * prev_res) refresh = true;  // slow chord contraction
         alpha = 1.0;
-        PP_CK(launch_stage_matvec<double>(m, ctx->tb, nullptr, 1.0, 0.0, us, dk, 0, ctx->stream));
-        PP_TRY(host_norm(ctx, n, dk, &mun));
+        if (!std::isfinite(mun)) return set_error(ctx, PP_ENAN, "non-finite norm");
         const double tol = ctx->cfg.newton_tol * mun;
         if (rn <= tol || (it > 0 && rn <= 1e3 * tol && rn > 0.5 * prev_res)) {
           converged = true;
