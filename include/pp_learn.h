@@ -25,6 +25,17 @@ int pp_gemm_f32(int m, int n, int k, float alpha, const float* A, int lda, int t
                 float beta, float* C, int ldc, void* stream);
 int pp_gemm_f64(int m, int n, int k, double alpha, const double* A, int lda, int ta, const double* B, int ldb,
                 int tb, double beta, double* C, int ldc, void* stream);
+/* Forward pass of a network of n_layers linear layers on X [rows][sizes[0]]: Z_l = H_(l-1) W_l + b_l
+   [rows][sizes[l+1]], H_l = GELU(Z_l) below the last layer, H_l = Z_l at the last (H_(-1) = X).
+   sizes: HOST [n_layers + 1]; W, b, Z, H: HOST arrays of n_layers DEVICE pointers. */
+int pp_mlp_forward_f32(int n_layers, int rows, const int* sizes, const float* X, const float* const* W,
+                       const float* const* b, float* const* Z, float* const* H, void* stream);
+/* Its backward pass from dY = d loss / d H_last: dW_l = H_(l-1)^T dZ_l, db_l = column sums of dZ_l,
+   dZ_(l-1) = (dZ_l W_l^T) GELU'(Z_(l-1)).  dZ: HOST array of n_layers - 1 DEVICE scratch arrays
+   [rows][sizes[l+1]]; dW, db: HOST arrays of n_layers DEVICE pointers. */
+int pp_mlp_backward_f32(int n_layers, int rows, const int* sizes, const float* X, const float* const* W,
+                        const float* const* Z, const float* const* H, const float* dY, float* const* dZ,
+                        float* const* dW, float* const* db, void* stream);
 /* Z[r][c] += b[c]; H = GELU(Z) (gelu_on = 1, GELU(z) = z Phi(z)) or H = Z (0). */
 int pp_bias_act_f32(int rows, int cols, float* Z, const float* b, float* H, int gelu_on, void* stream);
 /* dZ = dH * GELU'(Z), elementwise over n values. */

@@ -32,7 +32,7 @@ EXPORTED = [
     "pp_periodic_adjoint_multi", "pp_motion_eval",
     "pp_stage_apply", "pp_prof_also", "pp_prof_sample", "pp_prof_read_class", "pp_measure_fp64_peak_clock",
     # include/pp_learn.h
-    "pp_gemm_f32", "pp_gemm_f64", "pp_bias_act_f32", "pp_gelu_backward_f32", "pp_colsum_f32", "pp_mse_f32",
+    "pp_gemm_f32", "pp_gemm_f64", "pp_mlp_forward_f32", "pp_mlp_backward_f32", "pp_bias_act_f32", "pp_gelu_backward_f32", "pp_colsum_f32", "pp_mse_f32",
     "pp_adam_f32", "pp_syevj_f64",
 ]
 PP_K = dict(none=0, jacobian=1, residual=2, stage_matvec=3, block_apply=4, block_inverse=5, krylov=6, other=7,
@@ -116,6 +116,8 @@ def _load():
         "pp_measure_fp64_peak_clock": (I, [I, dp, dp]),
         "pp_gemm_f32": (I, [I, I, I, C.c_float, P, I, I, P, I, I, C.c_float, P, I, P]),
         "pp_gemm_f64": (I, [I, I, I, D, P, I, I, P, I, I, D, P, I, P]),
+        "pp_mlp_forward_f32": (I, [I, I, P, P, P, P, P, P, P]),
+        "pp_mlp_backward_f32": (I, [I, I, P, P, P, P, P, P, P, P, P, P]),
         "pp_bias_act_f32": (I, [I, I, P, P, P, I, P]),
         "pp_gelu_backward_f32": (I, [I, P, P, P, P]),
         "pp_colsum_f32": (I, [I, I, P, P, P]),
@@ -503,6 +505,25 @@ def pp_gemm(A, B, C_out, ta=False, tb=False, alpha=1.0, beta=0.0):
     f = _lib.pp_gemm_f32 if A.dtype == torch.float32 else _lib.pp_gemm_f64
     _lcheck(f(m, n, k, alpha, _ptr(A), A.shape[1], int(ta), _ptr(B), B.shape[1], int(tb), beta, _ptr(C_out),
               C_out.shape[1], _stream()), "pp_gemm")
+
+
+def _ptrs(arrays):
+    """HOST array of device addresses, from addresses or tensors."""
+    return (C.c_void_p * len(arrays))(*[a if isinstance(a, int) else a.data_ptr() for a in arrays])
+
+
+def pp_mlp_forward_f32(sizes, rows, X, W, b, Z, H):
+    """Z_l = H_(l-1) W_l + b_l, H_l = GELU(Z_l) below the last layer; sizes: the len(W) + 1 widths; W, b, Z, H:
+    lists of float32 CUDA tensors or their addresses."""
+    _lcheck(_lib.pp_mlp_forward_f32(len(W), rows, (C.c_int * len(sizes))(*sizes), X.data_ptr(), _ptrs(W), _ptrs(b),
+                                    _ptrs(Z), _ptrs(H), _stream()), "pp_mlp_forward_f32")
+
+
+def pp_mlp_backward_f32(sizes, rows, X, W, Z, H, dY, dZ, dW, db):
+    """Gradients dW, db of the network from dY = d loss / d H_last; dZ: scratch of the hidden layers."""
+    _lcheck(_lib.pp_mlp_backward_f32(len(W), rows, (C.c_int * len(sizes))(*sizes), X.data_ptr(), _ptrs(W), _ptrs(Z),
+                                     _ptrs(H), dY.data_ptr(), _ptrs(dZ), _ptrs(dW), _ptrs(db), _stream()),
+            "pp_mlp_backward_f32")
 
 
 def pp_bias_act_f32(Z, b, H, gelu_on):

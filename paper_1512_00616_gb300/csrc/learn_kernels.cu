@@ -2,7 +2,8 @@
 // coefficients from the motion parameters):
 //  - tiled dense GEMM, FP32 (network) and FP64 (snapshot Gram matrix, modes, projections),
 //    C = alpha op(A) op(B) + beta C, row-major;
-//  - bias + GELU forward (pre-activation kept), GELU backward, bias-gradient column sums;
+//  - whole network passes, one launch per layer forward and two backward (bias, GELU, its derivative and
+//    the bias gradient in the products' epilogues), and the same steps as separate calls;
 //  - mean-squared-error loss and gradient;
 //  - Adam update;
 //  - one-CTA cyclic Jacobi eigensolver for a small symmetric matrix (POD Gram matrix).
@@ -18,43 +19,111 @@
 
 namespace {
 
-constexpr int TILE = 16;
-
-// row-major element of op(A) (m x k): A is m x k (ta = 0) or k x m (ta = 1)
-template <class T>
-__device__ __forceinline__ T at(const T* A, int lda, int r, int c, int trans) {
-  return trans ? A[(size_t)c * lda + r] : A[(size_t)r * lda + c];
-}
-
-template <class T>
-__global__ void k_gemm(int m, int n, int k, T alpha, const T* __restrict__ A, int lda, int ta,
-                       const T* __restrict__ B, int ldb, int tb, T beta, T* __restrict__ C, int ldc) {
-  __shared__ T As[TILE][TILE + 1];
-  __shared__ T Bs[TILE][TILE + 1];
-  const int r = blockIdx.y * TILE + threadIdx.y;
-  const int c = blockIdx.x * TILE + threadIdx.x;
-  T acc = T(0);
-  for (int k0 = 0; k0 < k; k0 += TILE) {
-    const int ka = k0 + threadIdx.x, kb = k0 + threadIdx.y;
-    As[threadIdx.y][threadIdx.x] = (r < m && ka < k) ? at(A, lda, r, ka, ta) : T(0);
-    Bs[threadIdx.y][threadIdx.x] = (kb < k && c < n) ? at(B, ldb, kb, c, tb) : T(0);
-    __syncthreads();
-#pragma unroll
-    for (int t = 0; t < TILE; ++t) acc += As[threadIdx.y][t] * Bs[t][threadIdx.x];
-    __syncthreads();
-  }
-  if (r < m && c < n) {
-    T* out = C + (size_t)r * ldc + c;
-    *out = alpha * acc + (beta != T(0) ? beta * *out : T(0));
-  }
-}
-
 __device__ __forceinline__ float gelu(float z) { return 0.5f * z * (1.0f + erff(z * 0.70710678118654752f)); }
 __device__ __forceinline__ float gelu_grad(float z) {
   // d/dz [z Phi(z)] = Phi(z) + z phi(z)
   const float Phi = 0.5f * (1.0f + erff(z * 0.70710678118654752f));
   const float phi = 0.39894228040143268f * expf(-0.5f * z * z);
   return Phi + z * phi;
+}
+
+// C tile of op(A) op(B), 32 x 32 per CTA of 128 threads, 2 x 4 outputs per thread, depth 32 with the
+// next tiles' words in registers while the current ones are multiplied.  At the network's sizes (512 x
+// 256 x 256) a layer is 128 CTAs and bound by the latency of its 8 depth steps; the 16 x 16 tile with
+// one output per thread before took twice the steps and two shared-memory loads per multiply-add.
+// epi(row, column, sum) is called for every entry; colsum (or null) receives the column sums of op(B),
+// formed by the first row of tiles from the words it has loaded anyway.
+constexpr int TM = 32, TN = 32, TK = 32, GEMM_T = 128;
+
+template <bool TA, bool TB, class T, class Epi>
+__device__ __forceinline__ void gemm_tile(int m, int n, int k, const T* __restrict__ A, int lda,
+                                          const T* __restrict__ B, int ldb, T* colsum, Epi epi) {
+  __shared__ T As[TK][TM + 1];
+  __shared__ T Bs[TK][TN + 1];
+  constexpr int L = TM * TK / GEMM_T;
+  const int tid = threadIdx.x, r0 = blockIdx.y * TM, c0 = blockIdx.x * TN;
+  const int tr = tid / 8 * 2, tc = tid % 8;  // columns tc, tc + 8, tc + 16, tc + 24
+  T a[L], b[L];
+  auto load = [&](int k0) {
+#pragma unroll
+    for (int i = 0; i < L; ++i) {
+      const int idx = tid + GEMM_T * i, lo = idx % 32, hi = idx / 32;
+      const int ar = r0 + (TA ? lo : hi), ak = k0 + (TA ? hi : lo);
+      a[i] = ar < m && ak < k ? (TA ? A[(size_t)ak * lda + ar] : A[(size_t)ar * lda + ak]) : T(0);
+      const int bc = c0 + (TB ? hi : lo), bk = k0 + (TB ? lo : hi);
+      b[i] = bc < n && bk < k ? (TB ? B[(size_t)bc * ldb + bk] : B[(size_t)bk * ldb + bc]) : T(0);
+    }
+  };
+  T acc[2][4] = {}, csum = T(0);
+  load(0);
+  for (int k0 = 0; k0 < k; k0 += TK) {
+    __syncthreads();
+#pragma unroll
+    for (int i = 0; i < L; ++i) {
+      const int idx = tid + GEMM_T * i, lo = idx % 32, hi = idx / 32;
+      As[TA ? hi : lo][TA ? lo : hi] = a[i];
+      Bs[TB ? lo : hi][TB ? hi : lo] = b[i];
+    }
+    __syncthreads();
+    if (k0 + TK < k) load(k0 + TK);
+#pragma unroll
+    for (int t = 0; t < TK; ++t) {
+      const T a0 = As[t][tr], a1 = As[t][tr + 1];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const T bv = Bs[t][tc + 8 * q];
+        acc[0][q] += a0 * bv;
+        acc[1][q] += a1 * bv;
+      }
+    }
+    if (colsum && blockIdx.y == 0 && tid < TN)
+      for (int t = 0; t < TK; ++t) csum += Bs[t][tid];
+  }
+  if (colsum && blockIdx.y == 0 && tid < TN && c0 + tid < n) colsum[c0 + tid] = csum;
+#pragma unroll
+  for (int p = 0; p < 2; ++p)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int r = r0 + tr + p, c = c0 + tc + 8 * q;
+      if (r < m && c < n) epi(r, c, acc[p][q]);
+    }
+}
+
+template <bool TA, bool TB, class T>
+__global__ void __launch_bounds__(GEMM_T)
+    k_gemm(int m, int n, int k, T alpha, const T* __restrict__ A, int lda, const T* __restrict__ B, int ldb, T beta,
+           T* __restrict__ C, int ldc) {
+  gemm_tile<TA, TB, T>(m, n, k, A, lda, B, ldb, nullptr, [&](int r, int c, T s) {
+    T* out = C + (size_t)r * ldc + c;
+    *out = alpha * s + (beta != T(0) ? beta * *out : T(0));
+  });
+}
+
+// Z = X W + b, H = gelu(Z) (act) or Z
+__global__ void __launch_bounds__(GEMM_T)
+    k_linear(int rows, int fo, int fi, const float* __restrict__ X, const float* __restrict__ W,
+             const float* __restrict__ b, float* __restrict__ Z, float* __restrict__ H, int act) {
+  gemm_tile<false, false, float>(rows, fo, fi, X, fi, W, fo, nullptr, [&](int r, int c, float s) {
+    const float z = s + b[c];
+    Z[(size_t)r * fo + c] = z;
+    H[(size_t)r * fo + c] = act ? gelu(z) : z;
+  });
+}
+
+// dW = X^T dZ and db = column sums of dZ
+__global__ void __launch_bounds__(GEMM_T)
+    k_linear_grad(int rows, int fo, int fi, const float* __restrict__ X, const float* __restrict__ dZ,
+                  float* __restrict__ dW, float* __restrict__ db) {
+  gemm_tile<true, false, float>(fi, fo, rows, X, fi, dZ, fo, db, [&](int r, int c, float s) { dW[(size_t)r * fo + c] = s; });
+}
+
+// dZ of the layer below: (dZ W^T) gelu'(Zin)
+__global__ void __launch_bounds__(GEMM_T)
+    k_linear_back(int rows, int fo, int fi, const float* __restrict__ dZ, const float* __restrict__ W,
+                  const float* __restrict__ Zin, float* __restrict__ dZin) {
+  gemm_tile<false, true, float>(rows, fi, fo, dZ, fo, W, fo, nullptr, [&](int r, int c, float s) {
+    dZin[(size_t)r * fi + c] = s * gelu_grad(Zin[(size_t)r * fi + c]);
+  });
 }
 
 // Z[r, c] += b[c]; H = gelu(Z) (act = 1) or H = Z (act = 0)
@@ -81,22 +150,31 @@ __global__ void k_colsum32(int rows, int cols, const float* dZ, float* db) {
   db[c] = s;
 }
 
-// loss = mean((Y - T)^2) over all entries; dY = 2 (Y - T) / count.  One block.
-__global__ void k_mse(int n, const float* Y, const float* Tg, float* dY, float* loss) {
-  __shared__ float red[256];
-  float s = 0.0f;
-  for (int i = threadIdx.x; i < n; i += blockDim.x) {
-    const float d = Y[i] - Tg[i];
-    s += d * d;
-    dY[i] = 2.0f * d / (float)n;
-  }
-  red[threadIdx.x] = s;
+// loss = mean((Y - T)^2) over all entries; dY = 2 (Y - T) / count.  One block, four sums per thread.
+__global__ void __launch_bounds__(1024) k_mse(int n, const float* Y, const float* Tg, float* dY, float* loss) {
+  __shared__ float red[32];
+  float s[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+  const float sc = 2.0f / (float)n;
+  for (int i0 = threadIdx.x; i0 < n; i0 += 4096)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int i = i0 + 1024 * q;
+      if (i >= n) break;
+      const float d = Y[i] - Tg[i];
+      s[q] += d * d;
+      dY[i] = sc * d;
+    }
+  float t = (s[0] + s[1]) + (s[2] + s[3]);
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+  if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = t;
   __syncthreads();
-  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
-    if (threadIdx.x < o) red[threadIdx.x] += red[threadIdx.x + o];
-    __syncthreads();
+  if (threadIdx.x < 32) {
+    t = red[threadIdx.x];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (threadIdx.x == 0) *loss = t / (float)n;
   }
-  if (threadIdx.x == 0) *loss = red[0] / (float)n;
 }
 
 __global__ void k_adam(int n, float* w, const float* g, float* m1, float* m2, float lr, float b1, float b2,
@@ -311,25 +389,63 @@ __global__ void k_identity(int n, double* V) {
 
 int blocks_for(int64_t n, int t) { return (int)((n + t - 1) / t); }
 
+dim3 tiles(int m, int n) { return dim3((n + TN - 1) / TN, (m + TM - 1) / TM); }
+
+template <class T>
+int gemm(int m, int n, int k, T alpha, const T* A, int lda, int ta, const T* B, int ldb, int tb, T beta, T* C, int ldc,
+         void* stream) {
+  if (m <= 0 || n <= 0 || k <= 0 || !A || !B || !C) return PP_LEARN_EINVAL;
+  cudaStream_t st = (cudaStream_t)stream;
+  pp::ProfScope ps(PP_K_OTHER, st);
+  const dim3 g = tiles(m, n);
+  if (ta && tb) k_gemm<true, true, T><<<g, GEMM_T, 0, st>>>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc);
+  else if (ta) k_gemm<true, false, T><<<g, GEMM_T, 0, st>>>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc);
+  else if (tb) k_gemm<false, true, T><<<g, GEMM_T, 0, st>>>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc);
+  else k_gemm<false, false, T><<<g, GEMM_T, 0, st>>>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc);
+  return cudaGetLastError() == cudaSuccess ? 0 : PP_LEARN_ECUDA;
+}
+
 }  // namespace
 
 extern "C" {
 
 int pp_gemm_f32(int m, int n, int k, float alpha, const float* A, int lda, int ta, const float* B, int ldb, int tb,
                 float beta, float* C, int ldc, void* stream) {
-  if (m <= 0 || n <= 0 || k <= 0 || !A || !B || !C) return PP_LEARN_EINVAL;
-  pp::ProfScope ps(PP_K_OTHER, (cudaStream_t)stream);
-  dim3 grid((n + TILE - 1) / TILE, (m + TILE - 1) / TILE), block(TILE, TILE);
-  k_gemm<float><<<grid, block, 0, (cudaStream_t)stream>>>(m, n, k, alpha, A, lda, ta, B, ldb, tb, beta, C, ldc);
-  return cudaGetLastError() == cudaSuccess ? 0 : PP_LEARN_ECUDA;
+  return gemm<float>(m, n, k, alpha, A, lda, ta, B, ldb, tb, beta, C, ldc, stream);
 }
 
 int pp_gemm_f64(int m, int n, int k, double alpha, const double* A, int lda, int ta, const double* B, int ldb, int tb,
                 double beta, double* C, int ldc, void* stream) {
-  if (m <= 0 || n <= 0 || k <= 0 || !A || !B || !C) return PP_LEARN_EINVAL;
-  pp::ProfScope ps(PP_K_OTHER, (cudaStream_t)stream);
-  dim3 grid((n + TILE - 1) / TILE, (m + TILE - 1) / TILE), block(TILE, TILE);
-  k_gemm<double><<<grid, block, 0, (cudaStream_t)stream>>>(m, n, k, alpha, A, lda, ta, B, ldb, tb, beta, C, ldc);
+  return gemm<double>(m, n, k, alpha, A, lda, ta, B, ldb, tb, beta, C, ldc, stream);
+}
+
+int pp_mlp_forward_f32(int n_layers, int rows, const int* sizes, const float* X, const float* const* W,
+                       const float* const* b, float* const* Z, float* const* H, void* stream) {
+  if (n_layers < 1 || rows <= 0 || !sizes || !X || !W || !b || !Z || !H) return PP_LEARN_EINVAL;
+  cudaStream_t st = (cudaStream_t)stream;
+  for (int l = 0; l < n_layers; ++l) {
+    if (sizes[l] <= 0 || sizes[l + 1] <= 0) return PP_LEARN_EINVAL;
+    pp::ProfScope ps(PP_K_OTHER, st);
+    k_linear<<<tiles(rows, sizes[l + 1]), GEMM_T, 0, st>>>(rows, sizes[l + 1], sizes[l], l ? H[l - 1] : X, W[l], b[l],
+                                                           Z[l], H[l], l + 1 < n_layers);
+  }
+  return cudaGetLastError() == cudaSuccess ? 0 : PP_LEARN_ECUDA;
+}
+
+int pp_mlp_backward_f32(int n_layers, int rows, const int* sizes, const float* X, const float* const* W,
+                        const float* const* Z, const float* const* H, const float* dY, float* const* dZ,
+                        float* const* dW, float* const* db, void* stream) {
+  if (n_layers < 1 || rows <= 0 || !sizes || !X || !W || !Z || !H || !dY || !dZ || !dW || !db) return PP_LEARN_EINVAL;
+  cudaStream_t st = (cudaStream_t)stream;
+  for (int l = n_layers - 1; l >= 0; --l) {
+    if (sizes[l] <= 0 || sizes[l + 1] <= 0) return PP_LEARN_EINVAL;
+    const float* d = l + 1 < n_layers ? dZ[l] : dY;
+    pp::ProfScope ps(PP_K_OTHER, st);
+    if (l > 0)
+      k_linear_back<<<tiles(rows, sizes[l]), GEMM_T, 0, st>>>(rows, sizes[l + 1], sizes[l], d, W[l], Z[l - 1], dZ[l - 1]);
+    k_linear_grad<<<tiles(sizes[l], sizes[l + 1]), GEMM_T, 0, st>>>(rows, sizes[l + 1], sizes[l], l ? H[l - 1] : X, d,
+                                                                   dW[l], db[l]);
+  }
   return cudaGetLastError() == cudaSuccess ? 0 : PP_LEARN_ECUDA;
 }
 
@@ -357,7 +473,7 @@ int pp_colsum_f32(int rows, int cols, const float* dZ, float* db, void* stream) 
 int pp_mse_f32(int n, const float* Y, const float* Tg, float* dY, float* loss, void* stream) {
   if (n <= 0) return PP_LEARN_EINVAL;
   pp::ProfScope ps(PP_K_OTHER, (cudaStream_t)stream);
-  k_mse<<<1, 256, 0, (cudaStream_t)stream>>>(n, Y, Tg, dY, loss);
+  k_mse<<<1, 1024, 0, (cudaStream_t)stream>>>(n, Y, Tg, dY, loss);
   return cudaGetLastError() == cudaSuccess ? 0 : PP_LEARN_ECUDA;
 }
 

@@ -7,8 +7,8 @@ produced by the GPU shooter itself.  Every arithmetic step runs in libpp kernels
 * snapshot Gram matrix, modes, projections and reconstructions: FP64 GEMMs
   (pp_gemm_f64);
 * eigen-decomposition of the Gram matrix: one-block Jacobi (pp_syevj_f64);
-* network forward and backward passes and Adam: pp_gemm_f32, pp_bias_act_f32,
-  pp_gelu_backward_f32, pp_colsum_f32, pp_mse_f32, pp_adam_f32.
+* network forward and backward passes and Adam: pp_mlp_forward_f32, pp_mlp_backward_f32,
+  pp_mse_f32, pp_adam_f32.
 
 A prediction is used only if the shooting residual it starts from is small enough.
 The first primal sweep of pp_shoot_nk evaluates that residual.  If it exceeds the
@@ -85,47 +85,44 @@ class MLP:
     def __init__(self, sizes, seed=0, device="cuda"):
         g = np.random.default_rng(seed)
         self.params = []
+        self.widths = [int(w) for w in sizes]
         for fi, fo in zip(sizes[:-1], sizes[1:]):
             lim = np.sqrt(6.0 / (fi + fo))
             W = torch.tensor(g.uniform(-lim, lim, (fi, fo)), dtype=torch.float32, device=device)
             b = torch.zeros(fo, dtype=torch.float32, device=device)
             self.params.append([W, b])
+        self.sizes = [p.numel() for layer in self.params for p in layer]
         self.m = [[torch.zeros_like(p) for p in layer] for layer in self.params]
         self.v = [[torch.zeros_like(p) for p in layer] for layer in self.params]
         self.step = 0
 
+    def _buffer(self, rows, layers):
+        """One uninitialized allocation for a [rows, width] array per layer, and their addresses."""
+        widths = self.widths[1:][:layers]
+        flat = torch.empty(rows * sum(widths), dtype=torch.float32, device=self.params[0][0].device)
+        base, ptrs = flat.data_ptr(), []
+        for w in widths:
+            ptrs.append(base)
+            base += 4 * rows * w
+        return flat, ptrs
+
     def forward(self, X):
-        self.cache = []
-        H = X.contiguous()
-        for li, (W, b) in enumerate(self.params):
-            Z = torch.zeros(H.shape[0], W.shape[1], dtype=torch.float32, device=H.device)
-            A.pp_gemm(H, W, Z)
-            Hn = torch.empty_like(Z)
-            A.pp_bias_act_f32(Z, b, Hn, li < len(self.params) - 1)
-            self.cache.append((H, Z))
-            H = Hn
-        return H
+        X = X.contiguous()
+        rows, n = X.shape[0], len(self.params)
+        Z, zp = self._buffer(rows, n)
+        H, hp = self._buffer(rows, n)
+        A.pp_mlp_forward_f32(self.widths, rows, X, [W for W, _ in self.params], [b for _, b in self.params], zp, hp)
+        self.cache = (X, Z, zp, H, hp)
+        return H[H.numel() - rows * self.widths[-1]:].view(rows, self.widths[-1])
 
     def backward(self, dY):
-        grads = [None] * len(self.params)
-        dH = dY.contiguous()
-        for li in range(len(self.params) - 1, -1, -1):
-            Hin, Z = self.cache[li]
-            if li == len(self.params) - 1:
-                dZ = dH
-            else:
-                dZ = torch.empty_like(Z)
-                A.pp_gelu_backward_f32(Z, dH, dZ)
-            W = self.params[li][0]
-            dW = torch.zeros_like(W)
-            A.pp_gemm(Hin, dZ, dW, ta=True)
-            db = torch.zeros_like(self.params[li][1])
-            A.pp_colsum_f32(dZ, db)
-            grads[li] = (dW, db)
-            if li > 0:
-                dHn = torch.zeros_like(Hin)
-                A.pp_gemm(dZ, W, dHn, tb=True)
-                dH = dHn
+        X, _, zp, _, hp = self.cache
+        flat = torch.empty(sum(self.sizes), dtype=torch.float32, device=X.device)
+        parts = flat.split(self.sizes)
+        grads = [(parts[2 * l].view(W.shape), parts[2 * l + 1]) for l, (W, _) in enumerate(self.params)]
+        dZ, dp = self._buffer(X.shape[0], len(self.params) - 1)
+        A.pp_mlp_backward_f32(self.widths, X.shape[0], X, [W for W, _ in self.params], zp, hp, dY.contiguous(), dp,
+                              [g[0] for g in grads], [g[1] for g in grads])
         return grads
 
     def loss_and_grads(self, X, T):
