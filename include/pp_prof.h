@@ -24,11 +24,11 @@ extern "C" {
 #define PP_K_STAGE_MATVEC32 8  /* FP32 block-sparse product (mixed-precision inner solves) */
 #define PP_K_BLOCK_APPLY32 9   /* FP32 block-Jacobi application */
 #define PP_K_KRYLOV32 10       /* FP32 Krylov reductions */
-#define PP_K_STAGE_OP 11       /* FP64 stage operator with the preconditioner folded in, x + B x */
+#define PP_K_STAGE_OP 11       /* (was: FP64 folded stage operator; now inside PP_K_STAGE_GMRES, never launched) */
 #define PP_K_FOLD 12           /* products B = -c J_off D^-1 forming that operator (FP64 or FP32) */
-#define PP_K_STAGE_OP32 13     /* FP32 folded stage operator of the mixed-precision inner solves */
-#define PP_K_ARNOLDI 14        /* the Gram-Schmidt passes of one FP64 Arnoldi step (3 launches) */
-#define PP_K_ARNOLDI32 15      /* the same in FP32 (mixed-precision inner solves) */
+#define PP_K_STAGE_OP32 13     /* (was: its FP32 twin; now inside PP_K_STAGE_GMRES32, never launched) */
+#define PP_K_ARNOLDI 14        /* one FP64 Arnoldi step of the GMRES levels outside the stage solves */
+#define PP_K_ARNOLDI32 15      /* the same in FP32 (inner solves without room for the folded operator) */
 #define PP_K_STAGE_GMRES 16    /* one whole FP64 stage solve: red-black reduced GMRES and x = D^-1 y */
 #define PP_K_STAGE_GMRES32 17  /* the same in FP32 (mixed-precision inner and Newton solves) */
 #define PP_K_COUNT 18

@@ -28,18 +28,18 @@
 //  - FP64 products run on the integer pipe (fixed.cuh): the FP64 pipe issues one warp instruction
 //    per 19 clocks and SM, so one application of K at 2048 triangles is 19 us of FP64 issue against
 //    10 us for its 79 MB from L2 at the 25 bytes per clock and SM that were measured;
-//  - one thread per matrix row: 3 nb column-major entries (a warp reads 256 contiguous bytes per
-//    column) through a ring in shared memory that cp.async fills ahead, over passes and barriers;
-//    with the columns in registers instead (two chunks of 20) the compiler spilled and a product of
-//    8192 triangles ran at 4.2 TB/s instead of 5.1;
+//  - one thread per matrix row: its 3 nb entries through a ring in shared memory that cp.async fills
+//    ahead, over passes and barriers; with the columns in registers instead (two chunks of 20) the
+//    compiler spilled and a product of 8192 triangles ran at 4.2 TB/s instead of 5.9;
 //  - the own slices of the basis live in shared memory when they fit beside a short ring;
 //  - three barriers per step (v -> B_IR v -> K v and its projections -> next v); every CTA sums
 //    the CTA partials itself in one fixed order, so all CTAs hold bitwise the same coefficients,
 //    take the same decisions, and results are reproducible bit for bit;
 //  - the Givens update runs on a warp of its own during the next step's first product.
 // Measured (GB300), time of a reduced step (which does the work of two steps of the separate
-// kernels): 2048 triangles, p = 3: 27 us (two separate steps 130 us; the first one-launch version
-// with FP64 FMAs 44 us); 8192 triangles: 112 us (330; 155); 32 triangles, p = 1: 17 us (64; 19).
+// kernels): 2048 triangles, p = 3: 25 us (two separate steps 130 us; the first one-launch version
+// with FP64 FMAs 44 us; 10 us are the blocks from L2, 5 us the three barriers); 8192 triangles: 100 us
+// (330; 155; 46 us at the HBM rate); 32 triangles, p = 1: 12 us (64; 19).
 // Barrier waits of the whole grid are bounded (about a second); an expired wait sets the error
 // word and ends the CTA, and every other CTA's wait then expires too.
 #pragma once
@@ -189,7 +189,8 @@ struct Rows {
 // and grid barriers.  ST chunks of U columns: 3 (77 KB) beside a basis in shared memory, 6 without.
 // The blocks interleave VW columns (fold_index), so a copy is 16 bytes per thread and 512
 // contiguous bytes per warp: with one word per copy the SM's outstanding requests, not the bytes,
-// were the limit (8192 triangles: 5.1 TB/s in FP64 words, 3.0 TB/s in FP32 words).
+// were the limit (8192 triangles: a product at 5.1 TB/s instead of 5.9 in FP64 words, mixed-precision
+// sweeps 231 ms instead of 205).
 template <int NB, class S, int ST>
 struct Ring {
   using R = Rows<NB, S>;

@@ -1382,25 +1382,9 @@ cudaError_t launch_mdot(int64_t n, const S* V, int64_t ldv, int k, const S* w, d
 }
 
 template <class S>
-cudaError_t launch_update_mdot(int64_t n, const S* V, int64_t ldv, int k, const double* h, S* w, double* out,
-                               double* partial, unsigned* counter, cudaStream_t st) {
-  return launch_cgs<S>(cgs_args<S>(1, n, V, ldv, k, h, w, out, partial, counter), st);
-}
-
-template <class S>
 cudaError_t launch_update_norm2(int64_t n, const S* V, int64_t ldv, int k, const double* h, S* w, double* out,
                                 double* partial, unsigned* counter, cudaStream_t st) {
   return launch_cgs<S>(cgs_args<S>(2, n, V, ldv, k, h, w, out, partial, counter), st);
-}
-
-template <class S>
-cudaError_t launch_update_norm2_givens(int64_t n, const S* V, int64_t ldv, int k, const double* h, S* w, double* out,
-                                       double* partial, unsigned* counter, int j, int m, const double* h1,
-                                       const double* h2, double* H, double* cs, double* sn, double* g, double* stat,
-                                       cudaStream_t st) {
-  CgsArgs<S> a = cgs_args<S>(2, n, V, ldv, k, h, w, out, partial, counter);
-  a.gv = GivensArgs{j, m, h1, h2, H, cs, sn, g, stat};
-  return launch_cgs<S>(a, st);
 }
 
 template <class S>
@@ -1517,8 +1501,6 @@ cudaError_t launch_scale(int64_t n, double* y, double a, const double* x, cudaSt
   template cudaError_t launch_scale_dev<S>(int64_t, S*, const double*, const S*, cudaStream_t);                     \
   template cudaError_t launch_mdot<S>(int64_t, const S*, int64_t, int, const S*, double*, double*, unsigned*,       \
                                       cudaStream_t);                                                                \
-  template cudaError_t launch_update_mdot<S>(int64_t, const S*, int64_t, int, const double*, S*, double*, double*,  \
-                                             unsigned*, cudaStream_t);                                              \
   template cudaError_t launch_update_norm2<S>(int64_t, const S*, int64_t, int, const double*, S*, double*, double*, \
                                               unsigned*, cudaStream_t);                                             \
   template cudaError_t launch_fold_blocks<S>(const DevMesh&, int, const S*, const S*, double, const FoldOut<S>&,    \
@@ -1531,9 +1513,6 @@ cudaError_t launch_scale(int64_t n, double* y, double a, const double* x, cudaSt
   template cudaError_t launch_arnoldi_ortho<S>(int64_t, const S*, int64_t, int, S*, double*, double*, double*,  \
                                                  double*, unsigned*, int, int, double*, double*, double*, double*,  \
                                                  double*, double, cudaStream_t);                                    \
-  template cudaError_t launch_update_norm2_givens<S>(int64_t, const S*, int64_t, int, const double*, S*, double*,   \
-                                                     double*, unsigned*, int, int, const double*, const double*,    \
-                                                     double*, double*, double*, double*, double*, cudaStream_t);    \
   template cudaError_t launch_dot<S>(int64_t, const S*, const S*, double*, double*, unsigned*, cudaStream_t);
 PP_INST(double)
 PP_INST(float)

@@ -18,7 +18,6 @@ namespace pp {
 constexpr int kMaxP = 4;
 constexpr int kMaxNp = 15;   // (p+1)(p+2)/2 at p = 4
 constexpr int kMaxNb = 60;   // 4 * kMaxNp
-constexpr int kMaxQv = 36;   // (p+2)^2 volume points at p = 4
 constexpr int kMaxQf = 6;    // p+2 face points at p = 4
 constexpr int kStages = 3;
 
@@ -55,8 +54,6 @@ PP_HD Dual& operator*=(Dual& a, Dual b) { a = a * b; return a; }
 
 PP_HD double val(double a) { return a; }
 PP_HD double val(Dual a) { return a.v; }
-PP_HD double der(double) { return 0.0; }
-PP_HD double der(Dual a) { return a.d; }
 __device__ __forceinline__ double sqrtT(double a) { return sqrt(a); }
 __device__ __forceinline__ Dual sqrtT(Dual a) {
   double s = sqrt(a.v);
@@ -277,15 +274,10 @@ cudaError_t launch_gmres_backsolve(int ncols, int m, const double* H, const doub
 template <class S>
 cudaError_t launch_mdot(int64_t n, const S* V, int64_t ldv, int k, const S* w, double* out, double* partial,
                         unsigned* counter, cudaStream_t st);
-// w -= V h[0:k]; then out[0:k] = V_j . w  (fused CGS second pass)
-template <class S>
-cudaError_t launch_update_mdot(int64_t n, const S* V, int64_t ldv, int k, const double* h, S* w, double* out,
-                               double* partial, unsigned* counter, cudaStream_t st);
 // w -= V h[0:k]; then out[0] = w . w
 template <class S>
 cudaError_t launch_update_norm2(int64_t n, const S* V, int64_t ldv, int k, const double* h, S* w, double* out,
                                 double* partial, unsigned* counter, cudaStream_t st);
-// w -= V h[0:k]; out[0] = w . w; then the GMRES Givens update of Hessenberg column j
 // One Arnoldi orthogonalization step against V[0..k) with selective reorthogonalization
 // (classical Gram-Schmidt, a second pass only when more than half of |w|^2 cancels),
 // ending with the Givens update of Hessenberg column j: h1[0..k] <- (V^T w, |w|^2),
@@ -309,11 +301,6 @@ template <class S>
 cudaError_t launch_arnoldi_ortho(int64_t n, const S* V, int64_t ldv, int k, S* w, double* h1, double* h2,
                                  double* nrm, double* partial, unsigned* counter, int j, int m, double* H, double* cs,
                                  double* sn, double* g, double* stat, double shift, cudaStream_t st);
-template <class S>
-cudaError_t launch_update_norm2_givens(int64_t n, const S* V, int64_t ldv, int k, const double* h, S* w, double* out,
-                                       double* partial, unsigned* counter, int j, int m, const double* h1,
-                                       const double* h2, double* H, double* cs, double* sn, double* g, double* stat,
-                                       cudaStream_t st);
 // out[0] = x . y
 template <class S>
 cudaError_t launch_dot(int64_t n, const S* x, const S* y, double* out, double* partial, unsigned* counter,
