@@ -179,14 +179,20 @@ struct Rows {
   static constexpr int CE = E >= 13 ? E : 24 / E * E;  // elements whose coefficients are held at a time
   static constexpr int C = 3 * NB;   // columns of a row of B
   static constexpr int U = (NB <= 24 ? 6 : 10) * (sizeof(S) == 8 ? 1 : 2);  // columns per ring chunk
-  static constexpr int NCH = C / U;  // chunks per row, a multiple of 3; 6 with the deep ring
+  static constexpr int NCH = C / U;  // chunks per row
+  // chunks of the deep ring: a ring runs on from row to row, so its length divides NCH (a slot would
+  // hold another chunk than the one that is read from it otherwise, and a row shorter than the ring
+  // would be read beyond its end)
+  static constexpr int DEEP = NCH % 6 == 0 ? 6 : 3;
+  static_assert(C % U == 0 && NCH % 3 == 0 && NCH % DEEP == 0, "a ring takes whole rows");
   static constexpr int XS = E * C;   // operand entries of a pass
   static constexpr int XP = (XS + GT - 1) / GT;
 };
 
 // Ring of a thread's next columns of B in shared memory, filled by cp.async: a thread copies and
 // reads only its own words, so no barrier is involved, and the ring runs on over passes, products
-// and grid barriers.  ST chunks of U columns: 3 (77 KB) beside a basis in shared memory, 6 without.
+// and grid barriers.  ST chunks of U columns: 3 (at most 77 KB) beside a basis in shared memory,
+// Rows::DEEP without (6, and 3 for FP32 rows of 12 and 60 columns, which 6 chunks do not divide).
 // The blocks interleave VW columns (fold_index), so a copy is 16 bytes per thread and 512
 // contiguous bytes per warp: with one word per copy the SM's outstanding requests, not the bytes,
 // were the limit (8192 triangles: a product at 5.1 TB/s instead of 5.9 in FP64 words, mixed-precision
@@ -332,6 +338,7 @@ __device__ __forceinline__ bool rows_product(const GArgs<S>& a, GShared<NB, S>& 
   using R = Rows<NB, S>;
   using W = typename Wire<S>::T;
   constexpr int NBB = 3 * NB * NB, VW = FoldOut<S>::VW;
+  static_assert(R::NCH % ST == 0, "slot c % ST holds chunk c of every row");
   const Lane<NB> ln;
   // passes of equal size
   const int np = (p1 - p0 + R::E - 1) / R::E, per = np > 0 ? (p1 - p0 + np - 1) / np : 0;
@@ -699,8 +706,10 @@ struct ArgsOf<S, kSingle> {
   using T = GArgs<S>;
 };
 
-template <int NB, class S, int MODE, int ST>
+// VS: the own slices of the basis lie in shared memory
+template <int NB, class S, int MODE, bool VS>
 __global__ void __launch_bounds__(GALL, 1) k_stage_gmres(const __grid_constant__ GArgs<S> args) {
+  constexpr int ST = VS ? 3 : Rows<NB, S>::DEEP;
   __shared__ GShared<NB, S> sh;
   extern __shared__ __align__(16) unsigned char dyn[];
   typename ArgsOf<S, MODE>::T a = args;
@@ -716,7 +725,6 @@ __global__ void __launch_bounds__(GALL, 1) k_stage_gmres(const __grid_constant__
   using W = typename Wire<S>::T;
   // own slices of the basis and their exponents: shared memory, or the slices of V itself
   const Ring<NB, S, ST> ring(dyn);
-  constexpr bool VS = ST == 3;
   W* const Vo = VS ? reinterpret_cast<W*>(dyn) + Ring<NB, S, ST>::WORDS : a.V + (size_t)r0 * NB;
   const size_t ldv = VS ? (size_t)a.own_max * NB : nv;
   int* const Ve = VS ? reinterpret_cast<int*>(Vo + (a.m + 1) * ldv) : a.Vexp + r0;
@@ -1009,9 +1017,10 @@ struct GSetup {
 
 template <int NB, class S>
 cudaError_t launch_gmres(GArgs<S>& a, cudaStream_t st) {
-  const void* const kernels[4] = {(const void*)k_stage_gmres<NB, S, kGrid, 3>, (const void*)k_stage_gmres<NB, S, kGrid, 6>,
-                                  (const void*)k_stage_gmres<NB, S, kClusters, 3>,
-                                  (const void*)k_stage_gmres<NB, S, kSingle, 3>};
+  const void* const kernels[4] = {(const void*)k_stage_gmres<NB, S, kGrid, true>,
+                                  (const void*)k_stage_gmres<NB, S, kGrid, false>,
+                                  (const void*)k_stage_gmres<NB, S, kClusters, true>,
+                                  (const void*)k_stage_gmres<NB, S, kSingle, true>};
   // one device per process (see pp_create); thread-safe static initialization
   static const GSetup setup = [&] {
     GSetup s;
@@ -1028,7 +1037,7 @@ cudaError_t launch_gmres(GArgs<S>& a, cudaStream_t st) {
     return s;
   }();
   if (setup.err != cudaSuccess) return setup.err;
-  const size_t short_bytes = sizeof(S) * Ring<NB, S, 3>::WORDS, deep_bytes = sizeof(S) * Ring<NB, S, 6>::WORDS;
+  const size_t short_bytes = sizeof(S) * Ring<NB, S, 3>::WORDS, deep_bytes = sizeof(S) * Ring<NB, S, Rows<NB, S>::DEEP>::WORDS;
   // the short ring and the basis slices of `own` elements
   auto basis_bytes = [&](int own) {
     return short_bytes + (size_t)(a.m + 1) * own * (sizeof(S) * NB + (sizeof(S) == 8 ? sizeof(int) : 0)) + 8;
