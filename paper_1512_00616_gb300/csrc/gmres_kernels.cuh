@@ -40,8 +40,8 @@
 // kernels): 2048 triangles, p = 3: 25 us (two separate steps 130 us; the first one-launch version
 // with FP64 FMAs 44 us; 10 us are the blocks from L2, 5 us the three barriers); 8192 triangles: 100 us
 // (330; 155; 46 us at the HBM rate); 32 triangles, p = 1: 12 us (64; 19).
-// Barrier waits of the whole grid are bounded (about a second); an expired wait sets the error
-// word and ends the CTA, and every other CTA's wait then expires too.
+// Barrier waits of the whole grid are bounded (about a second); an expired wait ends the CTA, which
+// reports it in the record itself (solve_record.h).  The host then clears the barrier words.
 #pragma once
 
 #include <algorithm>
@@ -50,6 +50,7 @@
 #include "pp_internal.h"
 #include "prof.h"
 #include "reduce.cuh"
+#include "solve_record.h"
 #include "../../include/pp_prof.h"
 
 namespace pp {
@@ -67,7 +68,7 @@ constexpr int kCluster = 8;
 enum Mode { kGrid, kClusters, kSingle };
 constexpr unsigned long long kBarrierNs = 1000000000ull;
 // barrier words, on their own 128-byte lines
-constexpr int BAR_COUNT = 0, BAR_EXIT = 32, BAR_ERROR = 64, BAR_WORDS = 96;
+constexpr int BAR_COUNT = 0, BAR_EXIT = 32, BAR_WORDS = 64;
 constexpr int kSmemMax = 227 * 1024;   // shared memory of a CTA
 
 // Blocks and exchanged vectors: FP64 ones travel as 58-bit fixed-point words with one exponent
@@ -150,7 +151,6 @@ struct Barrier {
           if ((++it & 255u) == 0u) {
             if (t0 == 0) t0 = now_ns();
             else if (now_ns() - t0 > kBarrierNs) {
-              atomicExch(bar + BAR_ERROR, 1u);
               ok = 0;
               break;
             }
@@ -1000,11 +1000,11 @@ __global__ void __launch_bounds__(GALL, 1) k_stage_gmres(const __grid_constant__
       }
     }
   }
-  if (bi == 0 && tid == 0) {
-    a.rec[1] += (double)total;
-    if (!alive) a.rec[0] = 8.0;
-    else if (flag == 4) a.rec[0] = 4.0;
-    else if (a.need_conv && flag != 1 && flag != 2) a.rec[0] = 1.0;
+  if (tid == 0) {
+    if (bi == 0) a.rec[1] += (double)total;
+    // codes are positive doubles, which order as their bits do
+    if (const int code = solve_code(alive, flag, a.need_conv != 0, bi == 0))
+      atomicMax(reinterpret_cast<unsigned long long*>(a.rec), (unsigned long long)__double_as_longlong((double)code));
   }
   if (alive) bar.leave();
 }

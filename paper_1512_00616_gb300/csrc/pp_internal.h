@@ -319,7 +319,7 @@ cudaError_t launch_stream_rows(const DevMesh& m, const DevTables& tb, int nb, in
 cudaError_t stream_rows_error(int* flag, bool reset);  // bounded-wait expiry flag of those kernels
 // One stage solve (gmres_kernels.cuh): restarted GMRES on (I + B) y = b with the folded blocks B
 // and the eliminated elements taken out, then x = D y.  Nothing is read back: failures (1 the cap
-// with need_conv set, 4 non-finite, 8 an expired barrier wait) stay in rec[0], which makes later
+// with need_conv set, 4 non-finite, 8 an expired barrier wait; solve_record.h) stay in rec[0], which makes later
 // solves return at once, and rec[1] counts the Krylov steps.  V holds m + 1 vectors; ywarm (kept elements, or null) is the initial guess when warm is set and receives y.
 template <class S>
 struct StageGmres {

@@ -26,6 +26,7 @@
 
 #include "context.h"
 #include "prof.h"
+#include "solve_record.h"
 #include "../../include/pp_prof.h"
 
 namespace pp {
@@ -62,8 +63,8 @@ int take_record(pp_ctx* ctx, int64_t* steps) {
   PP_CK(cudaMemsetAsync(ctx->d_scalar + kDot + 1, 0, 2 * sizeof(double), ctx->stream));
   PP_CK(cudaMemsetAsync(ctx->d_gm_bar, 0, sizeof(unsigned) * stage_gmres_barrier_words(), ctx->stream));
   PP_CK(cudaStreamSynchronize(ctx->stream));
-  if (code == 1.0) return set_error(ctx, PP_ENOCONV, "stage GMRES hit gmres_maxit");
-  if (code == 4.0) return set_error(ctx, PP_ENAN, "GMRES: non-finite Arnoldi quantity");
+  if (code == kSolveCap) return set_error(ctx, PP_ENOCONV, "stage GMRES hit gmres_maxit");
+  if (code == kSolveNonFinite) return set_error(ctx, PP_ENAN, "GMRES: non-finite Arnoldi quantity");
   return set_error(ctx, PP_ECUDA, "stage GMRES: grid barrier wait expired");
 }
 
