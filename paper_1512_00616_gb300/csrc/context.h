@@ -82,6 +82,7 @@ struct pp_ctx {
   double* d_gm = nullptr;      // stage solves: CTA partials
   unsigned* d_gm_bar = nullptr;   // stage solves: barrier words
   double steps_seen = 0.0;     // Krylov steps already counted from the record in d_scalar
+  bool record_open = false;    // a sweep has launched solves since the record was last known to be clean
   double* d_gterm = nullptr;   // adjoint-sweep gradient terms, 9 per stage [3 * Nt][9]
   size_t gterm_cap = 0;        // capacity in stages
 

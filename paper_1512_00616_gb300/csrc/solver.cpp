@@ -51,6 +51,22 @@ int host_dot(pp_ctx* ctx, int64_t n, const S* x, const S* y, double* out) {
   return PP_OK;
 }
 
+int clear_record(pp_ctx* ctx) {
+  ctx->steps_seen = 0.0;
+  PP_CK(cudaMemsetAsync(ctx->d_scalar + kDot + 1, 0, 2 * sizeof(double), ctx->stream));
+  PP_CK(cudaMemsetAsync(ctx->d_gm_bar, 0, sizeof(unsigned) * stage_gmres_barrier_words(), ctx->stream));
+  ctx->record_open = false;
+  return PP_OK;
+}
+
+// Start of a sweep: one that left early before may have left a failure (which would stop every solve
+// of this one) or uncounted steps behind.
+int open_record(pp_ctx* ctx) {
+  if (ctx->record_open) PP_TRY(clear_record(ctx));
+  ctx->record_open = true;
+  return PP_OK;
+}
+
 // The record of the stage solves as the last synchronized copy has it (host_dot, read_record):
 // adds the steps since the last call to *steps, and turns a failure into its status, clearing it
 // for the next sweep.
@@ -59,9 +75,7 @@ int take_record(pp_ctx* ctx, int64_t* steps) {
   *steps += (int64_t)(done - ctx->steps_seen);
   ctx->steps_seen = done;
   if (code == 0.0) return PP_OK;
-  ctx->steps_seen = 0.0;
-  PP_CK(cudaMemsetAsync(ctx->d_scalar + kDot + 1, 0, 2 * sizeof(double), ctx->stream));
-  PP_CK(cudaMemsetAsync(ctx->d_gm_bar, 0, sizeof(unsigned) * stage_gmres_barrier_words(), ctx->stream));
+  PP_TRY(clear_record(ctx));
   PP_CK(cudaStreamSynchronize(ctx->stream));
   if (code == kSolveCap) return set_error(ctx, PP_ENOCONV, "stage GMRES hit gmres_maxit");
   if (code == kSolveNonFinite) return set_error(ctx, PP_ENAN, "GMRES: non-finite Arnoldi quantity");
@@ -73,6 +87,13 @@ int read_record(pp_ctx* ctx, int64_t* steps) {
                         ctx->stream));
   PP_CK(cudaStreamSynchronize(ctx->stream));
   return take_record(ctx, steps);
+}
+
+// End of a sweep.
+int close_record(pp_ctx* ctx, int64_t* steps) {
+  PP_TRY(read_record(ctx, steps));
+  ctx->record_open = false;
+  return PP_OK;
 }
 
 int host_norm(pp_ctx* ctx, int64_t n, const double* x, double* out) {
@@ -321,6 +342,11 @@ int stage_solve(pp_ctx* ctx, const pp_mesh* mesh, const StageView& sv, int trans
     int outer = 0;
     int st = gmres<double>(ctx, ctx->kin, A, P, b, x, rtol, atol, ctx->cfg.gmres_maxit, &outer, nullptr, true);
     if (iters) *iters = outer + inner_total;
+    if (st != PP_OK) {
+      // what stopped the inner solves, if anything did, is the cause
+      int64_t steps = 0;
+      PP_TRY(read_record(ctx, &steps));
+    }
     if (st == PP_ENOCONV) return set_error(ctx, PP_ENOCONV, "stage FGMRES hit gmres_maxit");
     return st;
   }
@@ -568,6 +594,7 @@ int ensure_segment(pp_ctx* ctx, int step, int64_t* steps) {
 int primal_sweep(pp_ctx* ctx, const pp_mesh* mesh, const double* mu, int n_mu, const double* u0, int Nt,
                  double* u_traj, double* u_final, double* qoi) {
   PP_TRY(ensure_store(ctx, mesh, Nt));
+  PP_TRY(open_record(ctx));
   ctx->lin_valid = false;
   ctx->lin_mesh = mesh;
   ctx->lin_mu.assign(mu, mu + n_mu);
@@ -597,6 +624,7 @@ int primal_sweep(pp_ctx* ctx, const pp_mesh* mesh, const double* mu, int n_mu, c
       ctx->seg_cur = seg;
     }
   }
+  ctx->record_open = false;  // read after the last solve of every stage
   double W = 0.0, Jx = 0.0;
   for (int step = 0; step < Nt; ++step)
     for (int i = 0; i < 3; ++i) {
@@ -630,6 +658,7 @@ int tangent_sweep(pp_ctx* ctx, const double* v, double* out) {
   double* w = work_vec(ctx, 13);
   double* rhs = work_vec(ctx, 14);
   double* v0 = work_vec(ctx, 15);
+  PP_TRY(open_record(ctx));
   PP_TRY(copy(ctx, n, v0, v));
   PP_TRY(copy(ctx, n, du, v));
   ctx->last_gmres_tangent = 0;
@@ -653,7 +682,7 @@ int tangent_sweep(pp_ctx* ctx, const double* v, double* out) {
     }
     PP_TRY(lincomb(ctx, n, du, {1.0, ctx->b[0], ctx->b[1], ctx->b[2]}, {du, dk[0], dk[1], dk[2]}));
   }
-  PP_TRY(read_record(ctx, &ctx->last_gmres_tangent));
+  PP_TRY(close_record(ctx, &ctx->last_gmres_tangent));
   PP_TRY(lincomb(ctx, n, out, {1.0, -1.0}, {v0, du}));
   PP_CK(cudaStreamSynchronize(ctx->stream));
   PP_TRY(check_stream_kernels(ctx));
@@ -692,6 +721,7 @@ int adjoint_sweep(pp_ctx* ctx, const double* lam_Nt, const double* weights, doub
     }
     ds_host.assign(n_st * 3 * (size_t)n_mu, 0.0);
   }
+  PP_TRY(open_record(ctx));
   PP_TRY(copy(ctx, n, lam, lam_Nt));
   ctx->last_gmres_adjoint = 0;
   for (int step = Nt - 1; step >= 0; --step) {
@@ -762,7 +792,7 @@ int adjoint_sweep(pp_ctx* ctx, const double* lam_Nt, const double* weights, doub
     if (withF)
       PP_TRY(lincomb(ctx, n, lam, {1.0, dt * ctx->b[0], dt * ctx->b[1], dt * ctx->b[2]}, {lam, g[0], g[1], g[2]}));
   }
-  PP_TRY(read_record(ctx, &ctx->last_gmres_adjoint));
+  PP_TRY(close_record(ctx, &ctx->last_gmres_adjoint));
   PP_TRY(copy(ctx, n, lam0, lam));
   std::vector<double> gterm;
   if (withF && dFdmu) {
@@ -1294,7 +1324,9 @@ int stage_apply(pp_ctx* ctx, int step, int i, int kind, int trans, int prec, con
   if (prec == 1 && ctx->cfg.precision != PP_PREC_MIXED)
     return set_error(ctx, PP_EINVAL, "pp_stage_apply: FP32 copies exist in PP_PREC_MIXED only");
   int64_t steps = 0;
+  PP_TRY(open_record(ctx));
   PP_TRY(ensure_segment(ctx, step, &steps));
+  ctx->record_open = false;
   const pp_mesh* mesh = ctx->lin_mesh;
   const DevMesh& m = mesh->dev;
   const int64_t n = ctx->ws_nu;
