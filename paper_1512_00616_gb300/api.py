@@ -508,22 +508,57 @@ def pp_gemm(A, B, C_out, ta=False, tb=False, alpha=1.0, beta=0.0):
 
 
 def _ptrs(arrays):
-    """HOST array of device addresses, from addresses or tensors."""
+    """HOST array of device addresses, from addresses (whose sizes are the caller's) or tensors."""
     return (C.c_void_p * len(arrays))(*[a if isinstance(a, int) else a.data_ptr() for a in arrays])
+
+
+def _f32(name, a, count):
+    """Refuses a tensor with fewer than `count` contiguous float32 values on the GPU."""
+    import torch
+    if a.dtype is not torch.float32 or not a.is_cuda or a.numel() < count or not a.is_contiguous():
+        raise ValueError(f"{name}: {a.dtype} {tuple(a.shape)} on {a.device}, not {count} contiguous float32 values on the GPU")
+
+
+def _network(sizes, rows, X, *lists):
+    """Checks the arrays of a network's pass; lists: (name, arrays, rows of a layer's array or None for its inputs)."""
+    n = len(sizes) - 1
+    if n < 1 or any(len(v) != n for _, v, _ in lists):
+        raise ValueError(f"network of {n} layers: lists of {[len(v) for _, v, _ in lists]}")
+    _f32("X", X, rows * sizes[0])
+    for name, v, per in lists:
+        for l in range(n):
+            if not isinstance(v[l], int):
+                _f32(name, v[l], sizes[l + 1] * (sizes[l] if per is None else per))
 
 
 def pp_mlp_forward_f32(sizes, rows, X, W, b, Z, H):
     """Z_l = H_(l-1) W_l + b_l, H_l = GELU(Z_l) below the last layer; sizes: the len(W) + 1 widths; W, b, Z, H:
-    lists of float32 CUDA tensors or their addresses."""
-    _lcheck(_lib.pp_mlp_forward_f32(len(W), rows, (C.c_int * len(sizes))(*sizes), X.data_ptr(), _ptrs(W), _ptrs(b),
-                                    _ptrs(Z), _ptrs(H), _stream()), "pp_mlp_forward_f32")
+    lists of contiguous float32 CUDA tensors of those sizes, or their addresses."""
+    _network(sizes, rows, X, ("W", W, None), ("b", b, 1), ("Z", Z, rows), ("H", H, rows))
+    _mlp_forward(sizes, rows, X.data_ptr(), *map(_ptrs, (W, b, Z, H)))
 
 
 def pp_mlp_backward_f32(sizes, rows, X, W, Z, H, dY, dZ, dW, db):
     """Gradients dW, db of the network from dY = d loss / d H_last; dZ: scratch of the hidden layers."""
-    _lcheck(_lib.pp_mlp_backward_f32(len(W), rows, (C.c_int * len(sizes))(*sizes), X.data_ptr(), _ptrs(W), _ptrs(Z),
-                                     _ptrs(H), dY.data_ptr(), _ptrs(dZ), _ptrs(dW), _ptrs(db), _stream()),
-            "pp_mlp_backward_f32")
+    _network(sizes, rows, X, ("W", W, None), ("Z", Z, rows), ("H", H, rows), ("dW", dW, None), ("db", db, 1))
+    _f32("dY", dY, rows * sizes[-1])
+    if len(dZ) != len(W) - 1:
+        raise ValueError(f"network of {len(W)} layers: {len(dZ)} scratch arrays")
+    for l, z in enumerate(dZ):
+        if not isinstance(z, int):
+            _f32("dZ", z, rows * sizes[l + 1])
+    _mlp_backward(sizes, rows, X.data_ptr(), *map(_ptrs, (W, Z, H)), dY.data_ptr(), *map(_ptrs, (dZ, dW, db)))
+
+
+# the calls themselves, on addresses and HOST arrays of addresses that the caller has checked
+def _mlp_forward(sizes, rows, *arrays):
+    n = len(sizes)
+    _lcheck(_lib.pp_mlp_forward_f32(n - 1, rows, (C.c_int * n)(*sizes), *arrays, _stream()), "pp_mlp_forward_f32")
+
+
+def _mlp_backward(sizes, rows, *arrays):
+    n = len(sizes)
+    _lcheck(_lib.pp_mlp_backward_f32(n - 1, rows, (C.c_int * n)(*sizes), *arrays, _stream()), "pp_mlp_backward_f32")
 
 
 def pp_bias_act_f32(Z, b, H, gelu_on):

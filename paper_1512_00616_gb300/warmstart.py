@@ -21,6 +21,7 @@ generates data with the GPU shooter, trains, then compares NK iterations and wal
 on held-out mu against the steady-state cold start.
 """
 import argparse
+import ctypes as C
 import json
 import time
 
@@ -79,50 +80,96 @@ class POD:
 
 
 # ------------------------------------------------------------------------------ network
+_F32 = torch.float32
+
+
+def _addresses(*ptrs):
+    """HOST array of device addresses."""
+    return (C.c_void_p * len(ptrs))(*ptrs)
+
+
 class MLP:
     """sizes[0] -> ... -> sizes[-1] with GELU hidden activations, FP32, row-major."""
 
     def __init__(self, sizes, seed=0, device="cuda"):
         g = np.random.default_rng(seed)
         self.params = []
-        self.widths = [int(w) for w in sizes]
         for fi, fo in zip(sizes[:-1], sizes[1:]):
             lim = np.sqrt(6.0 / (fi + fo))
             W = torch.tensor(g.uniform(-lim, lim, (fi, fo)), dtype=torch.float32, device=device)
             b = torch.zeros(fo, dtype=torch.float32, device=device)
             self.params.append([W, b])
-        self.sizes = [p.numel() for layer in self.params for p in layer]
         self.m = [[torch.zeros_like(p) for p in layer] for layer in self.params]
         self.v = [[torch.zeros_like(p) for p in layer] for layer in self.params]
         self.step = 0
 
-    def _buffer(self, rows, layers):
+    def _layers(self, dev):
+        """The layers that `params` holds now as contiguous arrays, the addresses of their weights and biases, and
+        the widths: the passes take every size from them, and refuse what the kernels would read as something else."""
+        keep, wp, bp, widths = [], [], [], []
+        for W, b in self.params:
+            shape = W.shape
+            if len(shape) != 2 or b.numel() != shape[1] or widths and shape[0] != widths[-1]:
+                raise ValueError(f"MLP: layer {len(wp)} has weights {tuple(shape)} and bias {tuple(b.shape)}")
+            if W.dtype is not _F32 or b.dtype is not _F32 or W.get_device() != dev or b.get_device() != dev:
+                raise ValueError(f"MLP: layer {len(wp)} is {W.dtype}, {b.dtype} on {W.device}, {b.device}, "
+                                 "not float32 beside the input")
+            if not (W.is_contiguous() and b.is_contiguous()):
+                W, b = W.contiguous(), b.contiguous()
+                keep.append((W, b))
+            if not widths:
+                widths.append(shape[0])
+            widths.append(shape[1])
+            wp.append(W.data_ptr())
+            bp.append(b.data_ptr())
+        return keep, _addresses(*wp), _addresses(*bp), widths
+
+    @staticmethod
+    def _checked(x, name, rows, cols):
+        shape = x.shape
+        if len(shape) != 2 or shape[1] != cols or rows is not None and shape[0] != rows or x.dtype is not _F32:
+            raise ValueError(f"MLP: {name} is {x.dtype} {tuple(shape)}, not float32 [{rows or 'rows'}, {cols}]")
+        return x if x.is_contiguous() else x.contiguous()
+
+    @staticmethod
+    def _buffer(rows, widths, device):
         """One uninitialized allocation for a [rows, width] array per layer, and their addresses."""
-        widths = self.widths[1:][:layers]
-        flat = torch.empty(rows * sum(widths), dtype=torch.float32, device=self.params[0][0].device)
+        flat = torch.empty(rows * sum(widths), dtype=_F32, device=device)
         base, ptrs = flat.data_ptr(), []
         for w in widths:
             ptrs.append(base)
             base += 4 * rows * w
-        return flat, ptrs
+        return flat, _addresses(*ptrs)
 
     def forward(self, X):
-        X = X.contiguous()
-        rows, n = X.shape[0], len(self.params)
-        Z, zp = self._buffer(rows, n)
-        H, hp = self._buffer(rows, n)
-        A.pp_mlp_forward_f32(self.widths, rows, X, [W for W, _ in self.params], [b for _, b in self.params], zp, hp)
-        self.cache = (X, Z, zp, H, hp)
-        return H[H.numel() - rows * self.widths[-1]:].view(rows, self.widths[-1])
+        keep, wp, bp, widths = self._layers(X.get_device())
+        X = self._checked(X, "the input", None, widths[0])
+        rows = X.shape[0]
+        Z, zp = self._buffer(rows, widths[1:], X.device)
+        H, hp = self._buffer(rows, widths[1:], X.device)
+        A._mlp_forward(widths, rows, X.data_ptr(), wp, bp, zp, hp)
+        self.cache = (X, Z, zp, H, hp, widths)
+        return H[H.numel() - rows * widths[-1]:].view(rows, widths[-1])
 
     def backward(self, dY):
-        X, _, zp, _, hp = self.cache
-        flat = torch.empty(sum(self.sizes), dtype=torch.float32, device=X.device)
-        parts = flat.split(self.sizes)
-        grads = [(parts[2 * l].view(W.shape), parts[2 * l + 1]) for l, (W, _) in enumerate(self.params)]
-        dZ, dp = self._buffer(X.shape[0], len(self.params) - 1)
-        A.pp_mlp_backward_f32(self.widths, X.shape[0], X, [W for W, _ in self.params], zp, hp, dY.contiguous(), dp,
-                              [g[0] for g in grads], [g[1] for g in grads])
+        X, _, zp, _, hp, widths = self.cache
+        rows = X.shape[0]
+        keep, wp, _, now = self._layers(X.get_device())
+        if now != widths:
+            raise ValueError(f"MLP: layers of widths {now} in the backward pass, {widths} in the forward pass")
+        dY = self._checked(dY, "the output's gradient", rows, widths[-1])
+        if dY.get_device() != X.get_device():
+            raise ValueError(f"MLP: the output's gradient is on {dY.device}, the input on {X.device}")
+        shapes = list(zip(widths[:-1], widths[1:]))
+        sizes = [n for fi, fo in shapes for n in (fi * fo, fo)]
+        flat = torch.empty(sum(sizes), dtype=_F32, device=X.device)
+        parts, ptrs = flat.split(sizes), [flat.data_ptr()]
+        for n in sizes:
+            ptrs.append(ptrs[-1] + 4 * n)
+        grads = [(parts[2 * l].view(shape), parts[2 * l + 1]) for l, shape in enumerate(shapes)]
+        dZ, dp = self._buffer(rows, widths[1:-1], X.device)
+        A._mlp_backward(widths, rows, X.data_ptr(), wp, zp, hp, dY.data_ptr(), dp, _addresses(*ptrs[:-1:2]),
+                        _addresses(*ptrs[1::2]))
         return grads
 
     def loss_and_grads(self, X, T):
