@@ -81,6 +81,7 @@ struct pp_ctx {
   unsigned* d_arn_bar = nullptr;  // fused Arnoldi step: arrival count, release epoch, error word
   double* d_gm = nullptr;      // stage solves: CTA partials
   unsigned* d_gm_bar = nullptr;   // stage solves: barrier words
+  pp::FoldScale wscale;        // powers of two of the FP64 stage solves' words
   double steps_seen = 0.0;     // Krylov steps already counted from the record in d_scalar
   bool record_open = false;    // a sweep has launched solves since the record was last known to be clean
   double* d_gterm = nullptr;   // adjoint-sweep gradient terms, 9 per stage [3 * Nt][9]

@@ -94,7 +94,7 @@ struct GArgs {
   int d_row, d_col;    // strides of a row / column of D
   const S* b;          // [ne][nb] right-hand side
   S* x;                // [ne][nb] solution
-  S* ywarm;            // [nR nb] y of the kept elements: initial guess (warm), written at the end; or null
+  S* ywarm;            // [nR nb] (scaled) y of the kept elements: initial guess (warm), written at the end; or null
   int warm;
   double rtol, atol;
   int maxit, m, need_conv;
@@ -107,6 +107,7 @@ struct GArgs {
   unsigned* bar;
   double* rec;         // [0] failure: 1 cap, 4 non-finite, 8 barrier; [1] steps taken
   int own_max;         // most kept elements of a CTA
+  VarScale scale;      // FP64: B and all vectors but b and x are scaled by these powers of two
 };
 
 __device__ __forceinline__ unsigned long long now_ns() {
@@ -259,10 +260,21 @@ struct Lane {
   __device__ Lane() : el(threadIdx.x / NB), row(threadIdx.x - threadIdx.x / NB * NB) {}
 };
 
+// Word of a row in an own slice of the basis in global memory (FP64): the eight lanes that share a slice in
+// cta_dots, two per variable, read consecutive words.  In shared memory the rows lie in their order: the
+// lanes' words two apart then fall into different banks as they are.
+template <int NB, bool VS>
+__host__ __device__ constexpr int slice_at(int row) {
+  constexpr int NP = NB / 4;
+  if (VS) return row;
+  const int var = row / NP, j = row - var * NP;
+  return j / 2 * 8 + (NP % 2 == 1 && j == NP - 1 ? var : 2 * var + j % 2);
+}
+
 // Writes a pass's rows (one value per thread, `on` where there is one) to the exchanged operand
 // (shared = true) and to the own slice `slot` of the basis (with exponents at slot_e, element
 // index own_el) unless that is null.
-template <int NB, class S>
+template <int NB, class S, bool VS>
 __device__ __forceinline__ void publish(const GArgs<S>& a, GShared<NB, S>& sh, int& turn, bool on, int el, int row,
                                         int pos, S val, bool shared, typename Wire<S>::T* slot = nullptr,
                                         int* slot_e = nullptr, int own_el = 0) {
@@ -280,7 +292,7 @@ __device__ __forceinline__ void publish(const GArgs<S>& a, GShared<NB, S>& sh, i
         if (row == 0) a.wexp[pos] = e;
       }
       if (slot) {
-        slot[own_el * NB + row] = q;
+        slot[own_el * NB + slice_at<NB, VS>(row)] = q;
         if (row == 0) slot_e[own_el] = e;
       }
     }
@@ -288,7 +300,7 @@ __device__ __forceinline__ void publish(const GArgs<S>& a, GShared<NB, S>& sh, i
     if (threadIdx.x < Rows<NB, S>::E) sh.emax[clear][threadIdx.x] = 0;
   } else if (on) {
     if (shared) a.wire[(size_t)pos * NB + row] = val;
-    if (slot) slot[own_el * NB + row] = val;
+    if (slot) slot[own_el * NB + slice_at<NB, VS>(row)] = val;
   }
 }
 
@@ -478,23 +490,25 @@ __device__ __forceinline__ void own_dots(const float* V, size_t ldv, int k, int 
 }
 
 // `from`: first vector (0, or k for |w|^2 alone), written from region row 0 on.
-template <int NB>
-__device__ __forceinline__ void cta_dots(const float* V, const int*, size_t ldv, size_t, int k, int from, int nel,
-                                         double* region, int rs, double (*)[GLD]) {
+template <int NB, bool VS>
+__device__ __forceinline__ void cta_dots(const float* V, const int*, const VarScale&, size_t ldv, size_t, int k,
+                                         int from, int nel, double* region, int rs, double (*)[GLD]) {
   const int nk = k - from, n = nel * NB;
   if (nk < GW) own_dots<1>(V, ldv, k, from, n, region, rs);
   else if (nk < 2 * GW) own_dots<2>(V, ldv, k, from, n, region, rs);
   else own_dots<4>(V, ldv, k, from, n, region, rs);
 }
 
-// FP64: eight lanes per vector; they share the entries of a slice (coalesced), and each lane turns
-// its exact integer sum over them into a double, so the FP64 pipe sees two instructions per slice.
-// A warp takes four vectors; with few vectors up to three warps share the elements of four.
-template <int NB>
-__device__ __forceinline__ void cta_dots(const Fix* V, const int* Vexp, size_t ldv, size_t lde, int k, int from,
-                                         int nel, double* region, int rs, double (*dpart)[GLD]) {
-  constexpr int P = (NB + 7) / 8;
-  const int lane = threadIdx.x & 31, l = lane & 7, warp = threadIdx.x >> 5;
+// FP64: eight lanes per vector, two per variable, so that a lane's words have one scale; each lane turns
+// its exact integer sum over every other entry of its variable into a double, so the FP64 pipe sees two
+// instructions per slice.  A warp takes four vectors; with few vectors up to three warps share the elements
+// of four.
+template <int NB, bool VS>
+__device__ __forceinline__ void cta_dots(const Fix* V, const int* Vexp, const VarScale& scale, size_t ldv, size_t lde,
+                                         int k, int from, int nel, double* region, int rs, double (*dpart)[GLD]) {
+  constexpr int NP = NB / 4, P = (NP + 1) / 2;
+  const int lane = threadIdx.x & 31, l = lane & 7, warp = threadIdx.x >> 5, var = l >> 1, half = l & 1;
+  const int unscale = -2 * scale[var];
   const int groups = (k - from) / 4 + 1, share = min(3, max(1, GW / groups));
   const Fix* w = V + (size_t)k * ldv;
   const int* we = Vexp + (size_t)k * lde;
@@ -510,11 +524,13 @@ __device__ __forceinline__ void cta_dots(const Fix* V, const int* Vexp, size_t l
         acc.clear();
 #pragma unroll
         for (int c = 0; c < P; ++c) {
-          const int i = el * NB + l + 8 * c;
-          if (NB % 8 == 0 || l + 8 * c < NB) acc.add(v[i], w[i]);
+          // slice_at of row var NP + 2 c + half
+          const bool odd = NP % 2 == 1 && c == P - 1;
+          const int i = el * NB + (VS ? var * NP + 2 * c + half : 8 * c + (odd ? var : l));
+          if (!odd || half == 0) acc.add(v[i], w[i]);
         }
         const int e1 = ve[el], e2 = we[el];
-        s = acc.result(e1 + e2, e1 == 0x7ff || e2 == 0x7ff, s);
+        s = acc.result(e1 + e2 + unscale, e1 == 0x7ff || e2 == 0x7ff, s);
       }
     }
 #pragma unroll
@@ -602,7 +618,7 @@ template <int NB>
 __device__ __forceinline__ void set_coefficients(GShared<NB, float>&, const double*, int, const int*, size_t, int,
                                                  int) {}
 
-// sum_t c_t V_t at one own row (of own element el, own row i)
+// sum_t c_t V_t at one own row (of own element el, word i of the own slices)
 template <int NB>
 __device__ __forceinline__ double combine(const GShared<NB, double>& sh, const double*, int k, const Fix* V,
                                           size_t ldv, int el, int i) {
@@ -631,7 +647,7 @@ __device__ __forceinline__ float combine(const GShared<NB, float>&, const double
   return (s[0] + s[1]) + (s[2] + s[3]);
 }
 
-// own entry i of a basis slot
+// word i of a basis slot
 __device__ __forceinline__ double entry(const Fix* slot, const int* slot_e, int el, int i) {
   return fix_decode(slot[i], slot_e[el]);
 }
@@ -746,12 +762,16 @@ __global__ void __launch_bounds__(GALL, 1) k_stage_gmres(const __grid_constant__
   const W* const rowR = first_row_of<NB, S>(a, r0, r1);
   auto wait = [&] { return bar.wait(); };
   auto idle = [] {};
-  auto rhs = [&](int pos, int row) { return a.b[(size_t)a.list[pos] * NB + row]; };
-  // f(on, element of the pass, own element, own row index) over passes of the own kept elements
+  auto raw = [&](int pos, int row) { return a.b[(size_t)a.list[pos] * NB + row]; };
+  auto rhs = [&](int pos, int row) {
+    if constexpr (sizeof(S) == 8) return raw(pos, row) * fix_pow2(a.scale[row / (NB / 4)]);
+    else return raw(pos, row);
+  };
+  // f(on, own element, word of the own slices) over passes of the own kept elements
   auto passes = [&](auto&& before, auto&& f) {
     for (int q = 0; q < nel; q += E) {
       before(q);
-      f(ln.el < E && q + ln.el < nel, q + ln.el, (q + ln.el) * NB + ln.row);
+      f(ln.el < E && q + ln.el < nel, q + ln.el, (q + ln.el) * NB + slice_at<NB, VS>(ln.row));
     }
   };
   auto none = [](int) {};
@@ -766,26 +786,27 @@ __global__ void __launch_bounds__(GALL, 1) k_stage_gmres(const __grid_constant__
     ring.prime(start, start != nullptr);
   }
   // the initial guess (zero without one) to the exchanged operand
-  passes(none, [&](bool on, int oe, int i) {
+  passes(none, [&](bool on, int oe, int) {
     S v = S(0);
     if (on) {
+      const int i = oe * NB + ln.row;
       if (guess) v = a.ywarm[(size_t)r0 * NB + i];
       yo[i] = v;
     }
-    publish<NB, S>(a, sh, turn, on, ln.el, ln.row, r0 + oe, v, true);
+    publish<NB, S, VS>(a, sh, turn, on, ln.el, ln.row, r0 + oe, v, true);
   });
   bar.arrive();
   for (bool first = true; alive; first = false) {
     // ---- residual of the reduced system: z = b_I - B_IR y, r = b_R - y - B_RR y - B_RI z
     if (guess) {
       alive = rows_product<NB, S, ST, MODE>(a, sh, ring, i0, i1, rowI, rowR, wait, idle, [&](bool on, int el, int row, int pos, S s) {
-        publish<NB, S>(a, sh, turn, on, el, row, pos, on ? rhs(pos, row) - s : S(0), true);
+        publish<NB, S, VS>(a, sh, turn, on, el, row, pos, on ? rhs(pos, row) - s : S(0), true);
       });
     } else {
       alive = bar.wait();
       for (int q = i0; alive && q < i1; q += E) {
         const bool on = ln.el < E && q + ln.el < i1;
-        publish<NB, S>(a, sh, turn, on, ln.el, ln.row, q + ln.el, on ? rhs(q + ln.el, ln.row) : S(0), true);
+        publish<NB, S, VS>(a, sh, turn, on, ln.el, ln.row, q + ln.el, on ? rhs(q + ln.el, ln.row) : S(0), true);
       }
     }
     if (!alive) break;
@@ -795,7 +816,7 @@ __global__ void __launch_bounds__(GALL, 1) k_stage_gmres(const __grid_constant__
       S s = S(0);
       for (int i = wt; i < (nel + i1 - i0) * NB; i += GT) {
         const int pos = i < nel * NB ? r0 + i / NB : i0 + i / NB - nel;
-        const S v = rhs(pos, i % NB);
+        const S v = raw(pos, i % NB);
         s += v * v;
       }
       S t[1] = {s};
@@ -804,7 +825,7 @@ __global__ void __launch_bounds__(GALL, 1) k_stage_gmres(const __grid_constant__
     }
     bar.arrive();
     alive = rows_product<NB, S, ST, MODE>(a, sh, ring, r0, r1, rowR, rowI, wait, idle, [&](bool on, int el, int row, int pos, S s) {
-      publish<NB, S>(a, sh, turn, on, el, row, pos, on ? rhs(pos, row) - yo[(pos - r0) * NB + row] - s : S(0), false,
+      publish<NB, S, VS>(a, sh, turn, on, el, row, pos, on ? rhs(pos, row) - yo[(pos - r0) * NB + row] - s : S(0), false,
                      Vo, Ve, pos - r0);
     });
     if (!alive) break;
@@ -815,7 +836,7 @@ __global__ void __launch_bounds__(GALL, 1) k_stage_gmres(const __grid_constant__
       for (int w = 0; w < GW; ++w) s += sh.coef[w];
       region0[rs + bi] = s;
     }
-    cta_dots<NB>(Vo, Ve, ldv, lde, 0, 0, nel, region0, rs, sh.dpart);
+    cta_dots<NB, VS>(Vo, Ve, a.scale, ldv, lde, 0, 0, nel, region0, rs, sh.dpart);
     bar.arrive();
     if (!(alive = bar.wait())) break;
     sum_partials<MODE>(first ? 2 : 1, region0, sh.red);
@@ -832,7 +853,7 @@ __global__ void __launch_bounds__(GALL, 1) k_stage_gmres(const __grid_constant__
     if (flag == 0) {
       const S inv0 = S(sh.inv);
       passes(none, [&](bool on, int oe, int i) {
-        publish<NB, S>(a, sh, turn, on, ln.el, ln.row, r0 + oe, on ? entry(Vo, Ve, oe, i) * inv0 : S(0), true, Vo, Ve,
+        publish<NB, S, VS>(a, sh, turn, on, ln.el, ln.row, r0 + oe, on ? entry(Vo, Ve, oe, i) * inv0 : S(0), true, Vo, Ve,
                        oe);
       });
       bar.arrive();
@@ -846,7 +867,7 @@ __global__ void __launch_bounds__(GALL, 1) k_stage_gmres(const __grid_constant__
             [&] {
               if (j > 0) givens<NB, S>(sh, j - 1, total + j >= a.maxit);
             },
-            [&](bool on, int el, int row, int pos, S s) { publish<NB, S>(a, sh, turn, on, el, row, pos, -s, true); });
+            [&](bool on, int el, int row, int pos, S s) { publish<NB, S, VS>(a, sh, turn, on, el, row, pos, -s, true); });
         if (!alive) break;
         bar.arrive();
         // ---- w = B_RR v_j + B_RI z, unless the step before was the last
@@ -860,7 +881,7 @@ __global__ void __launch_bounds__(GALL, 1) k_stage_gmres(const __grid_constant__
               return !stopped;
             },
             idle, [&](bool on, int el, int row, int pos, S s) {
-              publish<NB, S>(a, sh, turn, on, el, row, pos, s, false, slot, slot_e, pos - r0);
+              publish<NB, S, VS>(a, sh, turn, on, el, row, pos, s, false, slot, slot_e, pos - r0);
             });
         if (stopped) {
           alive = ended = true;
@@ -874,7 +895,7 @@ __global__ void __launch_bounds__(GALL, 1) k_stage_gmres(const __grid_constant__
         k = j + 1;
         __syncthreads();
         // ---- projections and |w|^2
-        cta_dots<NB>(Vo, Ve, ldv, lde, k, 0, nel, region1, rs, sh.dpart);
+        cta_dots<NB, VS>(Vo, Ve, a.scale, ldv, lde, k, 0, nel, region1, rs, sh.dpart);
         bar.arrive();
         if (!(alive = bar.wait())) break;
         sum_partials<MODE>(k + 1, region1, sh.red);
@@ -906,12 +927,12 @@ __global__ void __launch_bounds__(GALL, 1) k_stage_gmres(const __grid_constant__
                  [&](bool on, int oe, int i) {
                    const S s = on && pass < 2 ? entry(slot, slot_e, oe, i) - combine<NB>(sh, sh.red, k, Vo, ldv, oe, i)
                                               : S(0);
-                   publish<NB, S>(a, sh, turn, on, ln.el, ln.row, r0 + oe, s, false, slot, slot_e, oe);
+                   publish<NB, S, VS>(a, sh, turn, on, ln.el, ln.row, r0 + oe, s, false, slot, slot_e, oe);
                  });
           __syncthreads();
           double* region = pass == 0 ? region0 : region1;
-          if (pass == 0) cta_dots<NB>(Vo, Ve, ldv, lde, k, 0, nel, region, rs, sh.dpart);
-          else cta_dots<NB>(Vo, Ve, ldv, lde, k, k, nel, region + (size_t)k * rs, rs, sh.dpart);
+          if (pass == 0) cta_dots<NB, VS>(Vo, Ve, a.scale, ldv, lde, k, 0, nel, region, rs, sh.dpart);
+          else cta_dots<NB, VS>(Vo, Ve, a.scale, ldv, lde, k, k, nel, region + (size_t)k * rs, rs, sh.dpart);
           bar.arrive();
           if (!(alive = bar.wait())) break;
           if (pass == 0) {
@@ -928,7 +949,7 @@ __global__ void __launch_bounds__(GALL, 1) k_stage_gmres(const __grid_constant__
                [&](bool on, int oe, int i) {
                  const S s = on ? (entry(slot, slot_e, oe, i) - combine<NB>(sh, sh.red, k, Vo, ldv, oe, i)) * inv
                                 : S(0);
-                 publish<NB, S>(a, sh, turn, on, ln.el, ln.row, r0 + oe, s, true, slot, slot_e, oe);
+                 publish<NB, S, VS>(a, sh, turn, on, ln.el, ln.row, r0 + oe, s, true, slot, slot_e, oe);
                });
         bar.arrive();
       }
@@ -962,11 +983,12 @@ __global__ void __launch_bounds__(GALL, 1) k_stage_gmres(const __grid_constant__
            [&](bool on, int oe, int i) {
              S s = S(0);
              if (on) {
-               s = yo[i] + combine<NB>(sh, sh.coef, k, Vo, ldv, oe, i);
-               yo[i] = s;
-               if (a.ywarm) a.ywarm[(size_t)r0 * NB + i] = s;
+               const int r = oe * NB + ln.row;
+               s = yo[r] + combine<NB>(sh, sh.coef, k, Vo, ldv, oe, i);
+               yo[r] = s;
+               if (a.ywarm) a.ywarm[(size_t)r0 * NB + r] = s;
              }
-             publish<NB, S>(a, sh, turn, on, ln.el, ln.row, r0 + oe, s, true);
+             publish<NB, S, VS>(a, sh, turn, on, ln.el, ln.row, r0 + oe, s, true);
            });
     bar.arrive();
     guess = true;
@@ -986,7 +1008,9 @@ __global__ void __launch_bounds__(GALL, 1) k_stage_gmres(const __grid_constant__
       __syncthreads();
       for (int idx = wt; idx < E * NB && q0 + idx / NB < nown; idx += GT) {
         const int q = q0 + idx / NB, pos = q < nel ? r0 + q : i0 + q - nel;
-        ys[idx] = a.y[(size_t)pos * NB + idx % NB];
+        S y = a.y[(size_t)pos * NB + idx % NB];
+        if constexpr (sizeof(S) == 8) y *= fix_pow2(-a.scale[idx % NB / (NB / 4)]);
+        ys[idx] = y;
       }
       __syncthreads();
       if (ln.el < E && q0 + ln.el < nown) {
@@ -1113,6 +1137,7 @@ cudaError_t launch_stage_gmres(const DevMesh& m, int nb, const StageGmres<S>& q,
   a.partial = q.partial;
   a.bar = q.bar;
   a.rec = q.rec;
+  a.scale = q.scale;
   switch (nb) {
     case 12: return launch_gmres<12, S>(a, st);
     case 24: return launch_gmres<24, S>(a, st);

@@ -342,14 +342,15 @@ __global__ void __launch_bounds__(256)
 // [e][f][row]; FP32 blocks as floats (EN, ET unused).
 // FP64: both factors go to fixed point as well (one exponent per row of P and column of Q) and an
 // entry is one exact integer sum, two FP64 instructions instead of nb: with FP64 FMAs the kernel sat
-// at the FP64 pipe's floor (2048 triangles, p = 3: 1.06 ms a stage, normal and transposed blocks).
+// at the FP64 pipe's floor (2048 triangles, p = 3: 1.06 ms a stage, normal and transposed blocks).  The factors are
+// scaled as the words are (VarScale): (S P S^-1) (S Q S^-1), for the transposed blocks S^-1 in place of S.
 // Rows are padded to an odd number of words, so that lanes over rows read different banks.
 template <int NB, class S>
 __global__ void __launch_bounds__(256, 2)
-    k_fold_blocks(DevMesh m, const S* __restrict__ J, const S* __restrict__ Ainv, double c, FoldOut<S> out) {
+    k_fold_blocks(DevMesh m, const S* __restrict__ J, const S* __restrict__ Ainv, double c, FoldScale sc, FoldOut<S> out) {
   extern __shared__ __align__(16) unsigned char fsm_raw[];
   __shared__ int emax[3][NB];  // rows of P, columns of Q, rows of the product
-  constexpr int nb2 = NB * NB, LD = NB + 1;
+  constexpr int nb2 = NB * NB, LD = NB + 1, NP = NB / 4;
   constexpr int NV = (nb2 + 255) / 256;
   S* P = reinterpret_cast<S*>(fsm_raw);  // [row][k]
   S* Q = P + NB * LD;                    // [column][k]
@@ -376,7 +377,12 @@ __global__ void __launch_bounds__(256, 2)
     for (int t = 0; t < NV; ++t) {
       const int i = threadIdx.x + 256 * t, r = i % NB, k = i / NB;
       if (i >= nb2) continue;
-      const S pv = Pg[i], qv = Qg[i];
+      S pv = Pg[i], qv = Qg[i];
+      if constexpr (sizeof(S) == 8) {
+        const int d = pass == 0 ? sc.n[r / NP] - sc.n[k / NP] : sc.t[k / NP] - sc.t[r / NP];
+        pv *= fix_pow2(d);
+        qv *= fix_pow2(d);
+      }
       P[r * LD + k] = pv;
       Q[k * LD + r] = qv;
       if constexpr (sizeof(S) == 8) {
@@ -436,7 +442,7 @@ __global__ void __launch_bounds__(256, 2)
 template <class S>
 __global__ void __launch_bounds__(64)
     k_folded_apply(DevMesh m, int nb, const typename FoldOut<S>::W* __restrict__ B, const int* __restrict__ E,
-                   const S* __restrict__ x, S* __restrict__ y) {
+                   VarScale sc, const S* __restrict__ x, S* __restrict__ y) {
   const int e = blockIdx.x, r = threadIdx.x;
   if (r >= nb) return;
   S s = x[(size_t)e * nb + r];
@@ -446,7 +452,9 @@ __global__ void __launch_bounds__(64)
     const size_t blk = (size_t)e * 3 + f;
     for (int c = 0; c < nb; ++c) {
       S b;
-      if constexpr (sizeof(S) == 8) b = fix_decode(B[blk * nb * nb + fold_index<S>(nb, r, c)], E[blk * nb + r]);
+      if constexpr (sizeof(S) == 8)
+        b = fix_decode(B[blk * nb * nb + fold_index<S>(nb, r, c)], E[blk * nb + r]) *
+            fix_pow2(sc[c / (nb / 4)] - sc[r / (nb / 4)]);
       else b = B[blk * nb * nb + fold_index<S>(nb, r, c)];
       s += b * x[(size_t)e2 * nb + c];
     }
@@ -1243,8 +1251,8 @@ cudaError_t launch_block_apply(const DevMesh& m, int nb, const S* Ainv, const S*
 }
 
 template <class S>
-cudaError_t launch_fold_blocks(const DevMesh& m, int nb, const S* J, const S* Ainv, double c, const FoldOut<S>& out,
-                               cudaStream_t st) {
+cudaError_t launch_fold_blocks(const DevMesh& m, int nb, const S* J, const S* Ainv, double c, const FoldScale& sc,
+                               const FoldOut<S>& out, cudaStream_t st) {
   ProfScope ps(PP_K_FOLD, st);
   const size_t smem = sizeof(S) * 2 * nb * (nb + 1);
 #define PP_FOLD(NBV)                                                                                     \
@@ -1252,7 +1260,7 @@ cudaError_t launch_fold_blocks(const DevMesh& m, int nb, const S* J, const S* Ai
     static const cudaError_t attr =                                                                      \
         cudaFuncSetAttribute(k_fold_blocks<NBV, S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem); \
     if (attr != cudaSuccess) return attr;                                                                \
-    k_fold_blocks<NBV, S><<<m.ne * 3, 256, smem, st>>>(m, J, Ainv, c, out);                              \
+    k_fold_blocks<NBV, S><<<m.ne * 3, 256, smem, st>>>(m, J, Ainv, c, sc, out);                          \
     break;                                                                                               \
   }
   switch (nb) {
@@ -1268,10 +1276,10 @@ cudaError_t launch_fold_blocks(const DevMesh& m, int nb, const S* J, const S* Ai
 }
 
 template <class S>
-cudaError_t launch_folded_apply(const DevMesh& m, int nb, const typename FoldOut<S>::W* B, const int* E, const S* x,
-                                S* y, cudaStream_t st) {
+cudaError_t launch_folded_apply(const DevMesh& m, int nb, const typename FoldOut<S>::W* B, const int* E,
+                                const VarScale& sc, const S* x, S* y, cudaStream_t st) {
   ProfScope ps(PP_K_OTHER, st);
-  k_folded_apply<S><<<m.ne, 64, 0, st>>>(m, nb, B, E, x, y);
+  k_folded_apply<S><<<m.ne, 64, 0, st>>>(m, nb, B, E, sc, x, y);
   return cudaGetLastError();
 }
 
@@ -1503,10 +1511,10 @@ cudaError_t launch_scale(int64_t n, double* y, double a, const double* x, cudaSt
                                       cudaStream_t);                                                                \
   template cudaError_t launch_update_norm2<S>(int64_t, const S*, int64_t, int, const double*, S*, double*, double*, \
                                               unsigned*, cudaStream_t);                                             \
-  template cudaError_t launch_fold_blocks<S>(const DevMesh&, int, const S*, const S*, double, const FoldOut<S>&,    \
-                                             cudaStream_t);                                                         \
+  template cudaError_t launch_fold_blocks<S>(const DevMesh&, int, const S*, const S*, double, const FoldScale&,     \
+                                             const FoldOut<S>&, cudaStream_t);                                      \
   template cudaError_t launch_folded_apply<S>(const DevMesh&, int, const typename FoldOut<S>::W*, const int*,       \
-                                              const S*, S*, cudaStream_t);                                          \
+                                              const VarScale&, const S*, S*, cudaStream_t);                                          \
   template cudaError_t launch_arnoldi_step<S>(int64_t, const S*, int64_t, int, S*, S*, double*, double*, double*,    \
                                              double*, unsigned*, double*, int, int, double*, double*, double*,      \
                                              double*, double*, double, cudaStream_t);                               \

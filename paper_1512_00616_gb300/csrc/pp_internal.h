@@ -317,6 +317,19 @@ template <class S>
 cudaError_t launch_stream_rows(const DevMesh& m, const DevTables& tb, int nb, int nblk, const S* B, double alpha,
                                double beta, const S* x, S* y, cudaStream_t st);
 cudaError_t stream_rows_error(int* flag, bool reset);  // bounded-wait expiry flag of those kernels
+// FP64 blocks and vectors of the stage solves are fixed-point words with one exponent for all four variables
+// of a group (fixed.cuh).  The energy is 1 / M^2 of the density (M: Mach number), so the words hold the system
+// scaled by powers of two, which is exact: B' = S B S^-1, y' = S y with S = diag(1, 2^mom, 2^mom, 2^energy);
+// inner products and norms are those of the unscaled vectors.
+struct VarScale {
+  int mom = 0, energy = 0;
+  PP_HD int operator[](int var) const { return var == 0 ? 0 : var == 3 ? energy : mom; }
+};
+// for the normal and the transposed system
+struct FoldScale {
+  VarScale n, t;
+};
+FoldScale fold_scale(double mach);
 // One stage solve (gmres_kernels.cuh): restarted GMRES on (I + B) y = b with the folded blocks B
 // and the eliminated elements taken out, then x = D y.  Nothing is read back: failures (1 the cap
 // with need_conv set, 4 non-finite, 8 an expired barrier wait; solve_record.h) stay in rec[0], which makes later
@@ -340,6 +353,7 @@ struct StageGmres {
   double* partial;   // stage_gmres_partial_words()
   unsigned* bar;     // stage_gmres_barrier_words(), zero before the first launch
   double* rec;
+  VarScale scale;    // of the blocks (FP64)
 };
 constexpr int kGmresMaxRestart = 60;
 constexpr int kClusterRows = 2560;  // most kept rows solved by one cluster of 8 CTAs (one pass each)
@@ -349,7 +363,7 @@ size_t stage_gmres_partial_words();
 int stage_gmres_barrier_words();
 // BN = -c J_off Ainv_nbr and BT = (-c Ainv_nbr J_off,nbr)^T (3 blocks per element each; BT may
 // be null): the block-Jacobi preconditioner folded into the stage operator.  FP64 blocks are
-// stored as fixed-point words (fixed.cuh) with one exponent per block row (EN, ET).
+// stored as fixed-point words (fixed.cuh), scaled by sc, with one exponent per block row (EN, ET).
 // The blocks interleave groups of VW columns, 16 bytes per row and group (fold_index).
 struct Fix;
 template <class S>
@@ -376,12 +390,12 @@ PP_HD int fold_index(int nb, int row, int col) {
   return (col / FoldOut<S>::VW * nb + row) * FoldOut<S>::VW + col % FoldOut<S>::VW;
 }
 template <class S>
-cudaError_t launch_fold_blocks(const DevMesh& m, int nb, const S* J, const S* Ainv, double c, const FoldOut<S>& out,
-                               cudaStream_t st);
-// y = x + B x with those blocks
+cudaError_t launch_fold_blocks(const DevMesh& m, int nb, const S* J, const S* Ainv, double c, const FoldScale& sc,
+                               const FoldOut<S>& out, cudaStream_t st);
+// y = x + B x with those blocks (unscaled)
 template <class S>
-cudaError_t launch_folded_apply(const DevMesh& m, int nb, const typename FoldOut<S>::W* B, const int* E, const S* x,
-                                S* y, cudaStream_t st);
+cudaError_t launch_folded_apply(const DevMesh& m, int nb, const typename FoldOut<S>::W* B, const int* E,
+                                const VarScale& sc, const S* x, S* y, cudaStream_t st);
 int reduction_blocks();  // number of partial sums used by the reductions
 
 }  // namespace pp

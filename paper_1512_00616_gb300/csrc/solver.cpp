@@ -286,7 +286,7 @@ int stage_solve32(pp_ctx* ctx, const pp_mesh* mesh, const StageView& sv, int tra
     KrylovT<float>& K = ctx->k32;
     PP_CK(launch_stage_gmres<float>(m, ctx->tb.nb,
                                     {Bf, nullptr, trans ? sv.AT32 : sv.A32, 0, b, x, nullptr, 0, rtol, 0.0, maxit, K.m, 0,
-                                     K.V, K.t, K.w, ctx->d_wexp, ctx->d_gm, ctx->d_gm_bar, ctx->d_scalar + kDot + 1},
+                                     K.V, K.t, K.w, ctx->d_wexp, ctx->d_gm, ctx->d_gm_bar, ctx->d_scalar + kDot + 1, {}},
                                     ctx->stream));
     return PP_OK;
   }
@@ -359,7 +359,8 @@ int stage_solve(pp_ctx* ctx, const pp_mesh* mesh, const StageView& sv, int trans
     PP_CK(launch_stage_gmres<double>(m, ctx->tb.nb,
                                      {Bf, trans ? sv.ET : sv.EN, at ? sv.AinvT : sv.Ainv, trans && !at, b, x, ywarm,
                                       use_warm ? 1 : 0, rtol, atol, ctx->cfg.gmres_maxit, K.m, exact ? 1 : 0, K.V,
-                                      K.t, K.w, ctx->d_wexp, ctx->d_gm, ctx->d_gm_bar, ctx->d_scalar + kDot + 1},
+                                      K.t, K.w, ctx->d_wexp, ctx->d_gm, ctx->d_gm_bar, ctx->d_scalar + kDot + 1,
+                                      trans ? ctx->wscale.t : ctx->wscale.n},
                                      ctx->stream));
     return PP_OK;
   }
@@ -430,7 +431,7 @@ int finalize_stage_slot(pp_ctx* ctx, const pp_mesh* mesh, const StageView& sv, b
     }
     if (sv.BN32)
       PP_CK(launch_fold_blocks<float>(
-          m, nb, sv.J32, sv.A32, sv.c,
+          m, nb, sv.J32, sv.A32, sv.c, {},
           {const_cast<float*>(sv.BN32), full && sv.BT32 ? const_cast<float*>(sv.BT32) : nullptr}, ctx->stream));
     return PP_OK;
   }
@@ -439,7 +440,7 @@ int finalize_stage_slot(pp_ctx* ctx, const pp_mesh* mesh, const StageView& sv, b
   if (full && sv.JT)
     PP_CK(launch_transpose_blocks<double, double>(m, nb, sv.J, const_cast<double*>(sv.JT), ctx->stream));
   if (sv.BN)
-    PP_CK(launch_fold_blocks<double>(m, nb, sv.J, sv.Ainv, sv.c,
+    PP_CK(launch_fold_blocks<double>(m, nb, sv.J, sv.Ainv, sv.c, ctx->wscale,
                                      {(Fix*)sv.BN, full && sv.BT ? (Fix*)sv.BT : nullptr, const_cast<int*>(sv.EN),
                                       const_cast<int*>(sv.ET)},
                                      ctx->stream));
@@ -1343,7 +1344,8 @@ int stage_apply(pp_ctx* ctx, int step, int i, int kind, int trans, int prec, con
     } else {
       const uint64_t* Bf = trans ? sv.BT : sv.BN;
       if (!Bf) return set_error(ctx, PP_ESTATE, "pp_stage_apply: no FP64 folded operator stored");
-      PP_CK(launch_folded_apply<double>(m, nb, (const Fix*)Bf, trans ? sv.ET : sv.EN, x, y, ctx->stream));
+      PP_CK(launch_folded_apply<double>(m, nb, (const Fix*)Bf, trans ? sv.ET : sv.EN,
+                                        trans ? ctx->wscale.t : ctx->wscale.n, x, y, ctx->stream));
     }
   } else {
     if (!sv.J32) return set_error(ctx, PP_ESTATE, "pp_stage_apply: no FP32 copies stored");
@@ -1357,7 +1359,7 @@ int stage_apply(pp_ctx* ctx, int step, int i, int kind, int trans, int prec, con
     } else {
       const float* Bf = trans ? sv.BT32 : sv.BN32;
       if (!Bf) return set_error(ctx, PP_ESTATE, "pp_stage_apply: no FP32 folded operator stored");
-      PP_CK(launch_folded_apply<float>(m, nb, Bf, nullptr, x32, y32, ctx->stream));
+      PP_CK(launch_folded_apply<float>(m, nb, Bf, nullptr, {}, x32, y32, ctx->stream));
     }
     PP_CK(launch_cast<float, double>(n, y, y32, ctx->stream));
   }
