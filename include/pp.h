@@ -26,6 +26,9 @@
  *   context); small meshes use one CTA or one cluster of 8.  Two contexts solving at the same time
  *   on one device compete for the SMs; a barrier wait is bounded (about one
  *   second), after which the call fails with PP_ECUDA instead of hanging.
+ * - The FP64 stage solves resolve right-hand sides whose squared norm is in the
+ *   FP64 range (norms from about 1e-154); smaller ones count as zero, and so does
+ *   every number below 2^-1022 (subnormal).
  * - Nondimensionalization: chord 1, leading edge at the origin, free stream
  *   rho = 1, velocity (1, 0), p = 1/(gamma Mach^2), viscosity 1/Re.
  */

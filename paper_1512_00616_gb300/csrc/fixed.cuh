@@ -30,6 +30,15 @@ __device__ __forceinline__ double fix_pow2(int e) {
   return __hiloint2double((e > 1023 ? 2046 : e + 1023) << 20, 0);
 }
 
+// s + w 2^e for |w| < 2^63, rounded as one operation also where 2^e is below the normal range
+__device__ __forceinline__ double fix_scale(double w, int e, double s) {
+  if (e < -1022) {  // w and 2^e exchange a factor 2^128, which is exact
+    w *= 0x1p-128;
+    e += 128;
+  }
+  return fma(w, fix_pow2(e), s);
+}
+
 __device__ __forceinline__ int fix_exponent(double v) { return (__double2hiint(v) >> 20) & 0x7ff; }
 
 // The signed 53-bit significand of v (biased exponent ex) shifted right by d - 4, rounded: d = emax - ex
@@ -75,7 +84,10 @@ struct FixDot {
     hl += (long long)a.lo * b.hi;
     ll += (long long)a.lo * b.lo;
   }
-  // s + (hh 2^58 + hl 2^29 + ll) 2^(e2 - 2158), e2 the sum of the two group exponents; NaN if bad
+  // s + (hh 2^58 + hl 2^29 + ll) 2^(e2 - 2158), e2 the sum of the two group exponents; NaN if bad.  The unit of
+  // the sum is 2^60 below it, so sums under 2^-960 become zero; Small keeps them (squared norms of small vectors;
+  // its branch costs the products 3 %).
+  template <bool Small = false>
   __device__ __forceinline__ double result(int e2, bool bad, double s) const {
     const long long mid = hl + (ll >> 29);                 // units of 2^29; what ll loses is 2^-85 of the scale
     const long long top = hh + (mid >> 29);                // units of 2^58
@@ -84,7 +96,12 @@ struct FixDot {
     const int n = __clzll(top ^ (top >> 63)) - 1;          // leading bits that may be shifted out
     const int sh = n < 29 ? n : 29;
     const long long w = (top << sh) | (long long)(rest >> (29 - sh));
-    double scale = fix_pow2(e2 - 2158 + 58 - sh);          // w's unit
+    const int e = e2 - 2158 + 58 - sh;                     // of w's unit
+    if constexpr (Small) {
+      const double r = fix_scale((double)w, e, s);
+      return bad ? __longlong_as_double(0x7ff8000000000000LL) : r;
+    }
+    double scale = fix_pow2(e);
     if (bad) scale = __longlong_as_double(0x7ff8000000000000LL);
     return fma((double)w, scale, s);
   }

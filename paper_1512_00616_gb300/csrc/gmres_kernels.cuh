@@ -490,7 +490,7 @@ __device__ __forceinline__ void own_dots(const float* V, size_t ldv, int k, int 
 }
 
 // `from`: first vector (0, or k for |w|^2 alone), written from region row 0 on.
-template <int NB, bool VS>
+template <int NB, bool VS, bool Small = false>
 __device__ __forceinline__ void cta_dots(const float* V, const int*, const VarScale&, size_t ldv, size_t, int k,
                                          int from, int nel, double* region, int rs, double (*)[GLD]) {
   const int nk = k - from, n = nel * NB;
@@ -502,8 +502,8 @@ __device__ __forceinline__ void cta_dots(const float* V, const int*, const VarSc
 // FP64: eight lanes per vector, two per variable, so that a lane's words have one scale; each lane turns
 // its exact integer sum over every other entry of its variable into a double, so the FP64 pipe sees two
 // instructions per slice.  A warp takes four vectors; with few vectors up to three warps share the elements
-// of four.
-template <int NB, bool VS>
+// of four.  Small: the vector may be small (residuals; the basis is normalized).
+template <int NB, bool VS, bool Small = false>
 __device__ __forceinline__ void cta_dots(const Fix* V, const int* Vexp, const VarScale& scale, size_t ldv, size_t lde,
                                          int k, int from, int nel, double* region, int rs, double (*dpart)[GLD]) {
   constexpr int NP = NB / 4, P = (NP + 1) / 2;
@@ -530,7 +530,7 @@ __device__ __forceinline__ void cta_dots(const Fix* V, const int* Vexp, const Va
           if (!odd || half == 0) acc.add(v[i], w[i]);
         }
         const int e1 = ve[el], e2 = we[el];
-        s = acc.result(e1 + e2 + unscale, e1 == 0x7ff || e2 == 0x7ff, s);
+        s = acc.result<Small>(e1 + e2 + unscale, e1 == 0x7ff || e2 == 0x7ff, s);
       }
     }
 #pragma unroll
@@ -547,7 +547,7 @@ __device__ __forceinline__ void cta_dots(const Fix* V, const int* Vexp, const Va
 
 // out[t] = sum over the CTAs of region[t][.], t < nk, the same in every CTA: a warp per output, the
 // partials as integers against their largest exponent (exact sums, no FP64 additions).
-template <int MODE>
+template <int MODE, bool Small = false>
 __device__ __forceinline__ void sum_partials(int nk, const double* region, double* out) {
   if constexpr (MODE == kSingle) {
     for (int t = threadIdx.x; t < nk; t += GALL) out[t] = region[t];
@@ -585,7 +585,9 @@ __device__ __forceinline__ void sum_partials(int nk, const double* region, doubl
 #pragma unroll
     for (int p = 0; p < Q; ++p)
       if (lane == p && t0 + p * GW < nk)
-        out[t0 + p * GW] = e[p] == 0x7ff ? __longlong_as_double(0x7ff8000000000000LL) : (double)q[p] * fix_pow2(e[p] - 1076);
+        out[t0 + p * GW] = e[p] == 0x7ff ? __longlong_as_double(0x7ff8000000000000LL)
+                           : Small       ? fix_scale((double)q[p], e[p] - 1076, 0.0)
+                                         : (double)q[p] * fix_pow2(e[p] - 1076);
   }
   __syncthreads();
 }
@@ -836,10 +838,10 @@ __global__ void __launch_bounds__(GALL, 1) k_stage_gmres(const __grid_constant__
       for (int w = 0; w < GW; ++w) s += sh.coef[w];
       region0[rs + bi] = s;
     }
-    cta_dots<NB, VS>(Vo, Ve, a.scale, ldv, lde, 0, 0, nel, region0, rs, sh.dpart);
+    cta_dots<NB, VS, true>(Vo, Ve, a.scale, ldv, lde, 0, 0, nel, region0, rs, sh.dpart);
     bar.arrive();
     if (!(alive = bar.wait())) break;
-    sum_partials<MODE>(first ? 2 : 1, region0, sh.red);
+    sum_partials<MODE, true>(first ? 2 : 1, region0, sh.red);
     if (tid == 0) {
       const double beta = sqrt(fmax(sh.red[0], 0.0));
       if (first) sh.tol = fmax(a.rtol * sqrt(fmax(sh.red[1], 0.0)), a.atol);
