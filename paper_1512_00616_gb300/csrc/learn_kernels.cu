@@ -10,6 +10,7 @@
 // The C ABI is declared in include/pp_learn.h.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cmath>
 #include <cstdint>
 
@@ -97,6 +98,38 @@ __global__ void __launch_bounds__(GEMM_T)
     T* out = C + (size_t)r * ldc + c;
     *out = alpha * s + (beta != T(0) ? beta * *out : T(0));
   });
+}
+
+// The same with a 16 x 16 tile and one output per thread of 256 (see gemm for when).
+constexpr int TS = 16;
+template <bool TA, bool TB, class T>
+__global__ void __launch_bounds__(TS * TS)
+    k_gemm_small(int m, int n, int k, T alpha, const T* __restrict__ A, int lda, const T* __restrict__ B, int ldb,
+                 T beta, T* __restrict__ C, int ldc) {
+  __shared__ T As[TS][TS + 1];
+  __shared__ T Bs[TS][TS + 1];
+  const int x = threadIdx.x % TS, y = threadIdx.x / TS, c0 = blockIdx.x * TS;
+  for (int r0 = blockIdx.y * TS; r0 < m; r0 += gridDim.y * TS) {
+    T acc = T(0);
+    for (int k0 = 0; k0 < k; k0 += TS) {
+      // x runs along the stored rows of both operands
+      const int ar = r0 + (TA ? x : y), ak = k0 + (TA ? y : x);
+      const int bc = c0 + (TB ? y : x), bk = k0 + (TB ? x : y);
+      const T a = ar < m && ak < k ? (TA ? A[(size_t)ak * lda + ar] : A[(size_t)ar * lda + ak]) : T(0);
+      const T b = bc < n && bk < k ? (TB ? B[(size_t)bc * ldb + bk] : B[(size_t)bk * ldb + bc]) : T(0);
+      __syncthreads();
+      As[TA ? x : y][TA ? y : x] = a;  // [row][depth]
+      Bs[TB ? x : y][TB ? y : x] = b;  // [depth][column]
+      __syncthreads();
+#pragma unroll
+      for (int t = 0; t < TS; ++t) acc += As[y][t] * Bs[t][x];
+    }
+    const int r = r0 + y, c = c0 + x;
+    if (r < m && c < n) {
+      T* out = C + (size_t)r * ldc + c;
+      *out = alpha * acc + (beta != T(0) ? beta * *out : T(0));
+    }
+  }
 }
 
 // Z = X W + b, H = gelu(Z) (act) or Z
@@ -398,10 +431,26 @@ int gemm(int m, int n, int k, T alpha, const T* A, int lda, int ta, const T* B, 
   cudaStream_t st = (cudaStream_t)stream;
   pp::ProfScope ps(PP_K_OTHER, st);
   const dim3 g = tiles(m, n);
-  if (ta && tb) k_gemm<true, true, T><<<g, GEMM_T, 0, st>>>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc);
-  else if (ta) k_gemm<true, false, T><<<g, GEMM_T, 0, st>>>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc);
-  else if (tb) k_gemm<false, true, T><<<g, GEMM_T, 0, st>>>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc);
-  else k_gemm<false, false, T><<<g, GEMM_T, 0, st>>>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc);
+  // The small tile in FP64, whose issue rate is per SM (a warp instruction per 19 clocks): a CTA of the 32 x 32
+  // tile issues four times the FMAs per depth, so while there are fewer tiles than SMs it takes four times as
+  // long (snapshot Gram matrix 48 x 48, depth 81,920: 24.6 ms against 5.9 ms; projection 48 x 47: 24.5 against 5.8 ms;
+  // one reconstruction, 81,920 columns, depth 64: 282 against 142 us), and with many it is no faster (1500 x 1500 x
+  // 1500: 5.65 against 5.54 ms).  In FP32 the small tile with B transposed up to 240 large tiles (256 x 256, depth 4096:
+  // 271 against 101 us; 480 x 480, 225 tiles: 283 against 269 us; 512 x 512, 256 tiles: 283 against 312 us), 112 with
+  // both transposed (352 x 352, 121 tiles: 189 against 195 us).  Otherwise the large one (1024 x 1024 x 4096: 421 us;
+  // 1275 us with the 16 x 16 tile before).
+  if (sizeof(T) == 8 || (tb && g.x * g.y <= (ta ? 112u : 240u))) {
+    const dim3 h((n + TS - 1) / TS, std::min((m + TS - 1) / TS, 65535));
+    if (ta && tb) k_gemm_small<true, true, T><<<h, TS * TS, 0, st>>>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc);
+    else if (ta) k_gemm_small<true, false, T><<<h, TS * TS, 0, st>>>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc);
+    else if (tb) k_gemm_small<false, true, T><<<h, TS * TS, 0, st>>>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc);
+    else k_gemm_small<false, false, T><<<h, TS * TS, 0, st>>>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc);
+  } else if constexpr (sizeof(T) == 4) {
+    if (ta && tb) k_gemm<true, true, T><<<g, GEMM_T, 0, st>>>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc);
+    else if (ta) k_gemm<true, false, T><<<g, GEMM_T, 0, st>>>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc);
+    else if (tb) k_gemm<false, true, T><<<g, GEMM_T, 0, st>>>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc);
+    else k_gemm<false, false, T><<<g, GEMM_T, 0, st>>>(m, n, k, alpha, A, lda, B, ldb, beta, C, ldc);
+  }
   return cudaGetLastError() == cudaSuccess ? 0 : PP_LEARN_ECUDA;
 }
 
