@@ -115,7 +115,7 @@ __device__ __forceinline__ const double* lift_row(const DevTables& tb, int side,
 template <int N>
 __device__ __forceinline__ double fix_dot(const Fix* a, const Fix* b, int ea, int eb, double s, int stride = 1) {
   constexpr int parts = (N + 59) / 60, M = (N + parts - 1) / parts;
-  static_assert(parts == 1 || parts * M == N, "equal parts");
+  static_assert((parts == 1 || parts * M == N) && M <= kFixTerms, "equal parts, one exact sum each");
 #pragma unroll
   for (int p = 0; p < parts; ++p) {
     FixDot acc;

@@ -8,7 +8,7 @@
 // so entries within a factor 16 of the largest keep all 53 bits and the others are rounded at
 // 2^-58 of the group's scale (a DFMA chain rounds every partial sum at 2^-53 of itself).
 // q is stored as hi 2^29 + lo with |hi| <= 2^28 and -2^28 <= lo < 2^28, and the dot product over
-// up to 64 terms is exact in three 64-bit sums (hi hi, hi lo + lo hi, lo lo): 2^56 2^6 = 2^62.
+// up to kFixTerms terms is exact in three 64-bit sums (hi hi, hi lo + lo hi, lo lo).
 // The one rounding is the conversion of the sum to double.
 // Entries more than a factor 16 below the largest hold fewer than 53 bits, so a group that mixes variables is
 // scaled first (VarScale: the energy is 1 / M^2 of the density at Mach number M).  Error of a product with the
@@ -19,6 +19,9 @@
 #pragma once
 
 namespace pp {
+
+// the cross sum takes two products of up to 2^56 a term: 2 63 2^56 < 2^63
+constexpr int kFixTerms = 63;
 
 struct __align__(8) Fix {
   int hi, lo;

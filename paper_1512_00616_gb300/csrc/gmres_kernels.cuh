@@ -351,6 +351,7 @@ __device__ __forceinline__ bool rows_product(const GArgs<S>& a, GShared<NB, S>& 
   using W = typename Wire<S>::T;
   constexpr int NBB = 3 * NB * NB, VW = FoldOut<S>::VW;
   static_assert(R::NCH % ST == 0, "slot c % ST holds chunk c of every row");
+  static_assert(NB <= kFixTerms, "a block row is one exact sum");
   const Lane<NB> ln;
   // passes of equal size
   const int np = (p1 - p0 + R::E - 1) / R::E, per = np > 0 ? (p1 - p0 + np - 1) / np : 0;
@@ -624,6 +625,7 @@ __device__ __forceinline__ void set_coefficients(GShared<NB, float>&, const doub
 template <int NB>
 __device__ __forceinline__ double combine(const GShared<NB, double>& sh, const double*, int k, const Fix* V,
                                           size_t ldv, int el, int i) {
+  static_assert(GM <= kFixTerms, "the vectors of a cycle are one exact sum");
   FixDot acc;
   acc.clear();
   el %= Rows<NB, double>::CE;

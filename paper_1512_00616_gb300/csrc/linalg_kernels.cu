@@ -349,6 +349,7 @@ template <int NB, class S>
 __global__ void __launch_bounds__(256, 2)
     k_fold_blocks(DevMesh m, const S* __restrict__ J, const S* __restrict__ Ainv, double c, FoldScale sc, FoldOut<S> out) {
   extern __shared__ __align__(16) unsigned char fsm_raw[];
+  static_assert(NB <= kFixTerms, "an entry is one exact sum");
   __shared__ int emax[3][NB];  // rows of P, columns of Q, rows of the product
   constexpr int nb2 = NB * NB, LD = NB + 1, NP = NB / 4;
   constexpr int NV = (nb2 + 255) / 256;
