@@ -86,8 +86,11 @@ typedef struct pp_config {
   double newton_tol;  /* stop when ||dk||_2 <= newton_tol * max(1, ||u_i||_2) */
   int newton_maxit;
   double gmres_rtol;  /* relative tolerance of the Newton-step GMRES */
-  int gmres_restart;
-  int gmres_maxit;    /* cap on GMRES iterations per linear solve */
+  int gmres_restart;  /* basis vectors per cycle */
+  int gmres_maxit;    /* cap on GMRES steps per linear solve.  With the folded operator (the case while
+                         device memory allows) a step is one of the red-black reduced system: it reads
+                         the operator once, as a step of the whole system does, and advances as far as
+                         two of those */
   /* tangent and adjoint stage solves (linear, must be tight for exact sensitivities) */
   double lin_rtol;
   /* shooting (Algorithm primal) */
@@ -101,7 +104,7 @@ typedef struct pp_config {
   int adj_maxit;
   /* precision of the stage linear solves (PP_PREC_*) */
   int precision;
-  int inner_maxit;    /* PP_PREC_MIXED: FP32 GMRES iterations per preconditioner application */
+  int inner_maxit;    /* PP_PREC_MIXED: FP32 GMRES steps (as gmres_maxit) per preconditioner application */
   double inner_rtol;  /* PP_PREC_MIXED: relative tolerance of that inner solve */
   /* 0: the primal sweep keeps the stage linearization of the whole period in HBM.
      K > 0: it keeps the state and Newton predictor every K steps and one K-step segment

@@ -54,9 +54,11 @@ int pp_prof_read_class(int kind, int64_t* launches, double* total_ms, double* by
 /* Counts launches of every class since the last pp_prof_select (no events). */
 int pp_prof_counts(int64_t* counts /* [PP_K_COUNT] */);
 
-/* Iteration counts of the last sweeps on ctx: stage Newton iterations and GMRES
-   iterations of the last primal sweep; GMRES iterations of the last tangent and of
-   the last adjoint sweep.  Any pointer may be NULL. */
+/* Iteration counts of the last sweeps on ctx: stage Newton iterations and GMRES steps of
+   the last primal sweep; GMRES steps of the last tangent and of the last adjoint sweep.
+   A step is one of the red-black reduced system, worth two of the whole system, except where
+   the folded operator is not stored (pp_config.gmres_maxit); mixed precision adds the FP64
+   outer iterations to the inner steps.  Any pointer may be NULL. */
 struct pp_ctx;
 int pp_sweep_counts(const struct pp_ctx* ctx, int64_t* newton, int64_t* gmres_primal, int64_t* gmres_tangent,
                     int64_t* gmres_adjoint);

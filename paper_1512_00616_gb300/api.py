@@ -470,6 +470,7 @@ def pp_measure_fp64_peak_clock(device=0):
 
 
 def pp_sweep_counts(ctx):
+    """Newton iterations and GMRES steps (of the reduced system, include/pp_prof.h) of the last sweeps."""
     v = [C.c_int64() for _ in range(4)]
     _check(ctx, _lib.pp_sweep_counts(ctx, *[C.byref(x) for x in v]))
     return dict(newton=v[0].value, gmres_primal=v[1].value, gmres_tangent=v[2].value, gmres_adjoint=v[3].value)
