@@ -155,8 +155,7 @@ int copy(pp_ctx* ctx, int64_t n, S* y, const S* x) {
 // enqueued past convergence is simply not used (its column is beyond ncols).
 template <class S>
 int gmres(pp_ctx* ctx, KrylovT<S>& K, const OpT<S>& A, const OpT<S>& prec, const S* b, S* x, double rtol,
-          double atol, int maxit, int* iters, double* res_out, bool flexible = false, bool warm = false,
-          double shift = 0.0) {
+          double atol, int maxit, int* iters, double* res_out, bool flexible = false) {
   const int64_t n = K.n;
   const int m = K.m;
   double* d_h1 = K.d_h;
@@ -164,19 +163,8 @@ int gmres(pp_ctx* ctx, KrylovT<S>& K, const OpT<S>& A, const OpT<S>& prec, const
   double* d_nrm = K.d_h + 2 * (m + 2);
   const bool flex = flexible && K.Z && prec;
   bool first = true;
-  if (warm) {
-    // initial guess in x: the tolerance stays relative to |b| (set here), the first cycle
-    // starts from r = b - A x
-    PP_CK(launch_dot<S>(n, b, b, d_nrm, ctx->d_partial, ctx->d_counter, ctx->stream));
-    PP_CK(launch_gmres_init(d_nrm, rtol, atol, 1, m, K.d_g, K.d_stat, ctx->stream));
-    PP_TRY(A(x, K.w));
-    if (shift != 0.0) PP_TRY(lincomb<S>(ctx, n, K.r, {1.0, -1.0, -shift}, {b, K.w, x}));
-    else PP_TRY(lincomb<S>(ctx, n, K.r, {1.0, -1.0}, {b, K.w}));
-    first = false;
-  } else {
-    PP_CK(cudaMemsetAsync(x, 0, sizeof(S) * n, ctx->stream));
-    PP_TRY(copy<S>(ctx, n, K.r, b));
-  }
+  PP_CK(cudaMemsetAsync(x, 0, sizeof(S) * n, ctx->stream));
+  PP_TRY(copy<S>(ctx, n, K.r, b));
   int total = 0;
   double res = 0.0;
   int status = PP_ENOCONV;
@@ -202,11 +190,11 @@ int gmres(pp_ctx* ctx, KrylovT<S>& K, const OpT<S>& A, const OpT<S>& prec, const
         // one cooperative launch: orthogonalization, Givens, scaling, record into the ring
         PP_CK(launch_arnoldi_step<S>(n, K.V, n, j + 1, K.w, vnext, d_h1, d_h2, d_nrm, ctx->d_arn, ctx->d_arn_bar,
                                      K.h_h_dev + 8 * (j % kRing), j, m, K.d_H, K.d_cs, K.d_sn, K.d_g, K.d_stat,
-                                     shift, ctx->stream));
+                                     ctx->stream));
         PP_CK(cudaEventRecord(K.ev[j % kRing], ctx->stream));
       } else {
         PP_CK(launch_arnoldi_ortho<S>(n, K.V, n, j + 1, K.w, d_h1, d_h2, d_nrm, ctx->d_partial, ctx->d_counter, j,
-                                      m, K.d_H, K.d_cs, K.d_sn, K.d_g, K.d_stat, shift, ctx->stream));
+                                      m, K.d_H, K.d_cs, K.d_sn, K.d_g, K.d_stat, ctx->stream));
         PP_CK(cudaMemcpyAsync(slot, K.d_stat, 8 * sizeof(double), cudaMemcpyDeviceToHost, ctx->stream));
         PP_CK(cudaEventRecord(K.ev[j % kRing], ctx->stream));
         PP_CK(launch_scale_dev<S>(n, vnext, K.d_stat + 3, K.w, ctx->stream));
@@ -250,8 +238,7 @@ int gmres(pp_ctx* ctx, KrylovT<S>& K, const OpT<S>& A, const OpT<S>& prec, const
     if (total >= maxit) break;
     // restart from the true residual r = b - A x
     PP_TRY(A(x, K.w));
-    if (shift != 0.0) PP_TRY(lincomb<S>(ctx, n, K.r, {1.0, -1.0, -shift}, {b, K.w, x}));
-    else PP_TRY(lincomb<S>(ctx, n, K.r, {1.0, -1.0}, {b, K.w}));
+    PP_TRY(lincomb<S>(ctx, n, K.r, {1.0, -1.0}, {b, K.w}));
   }
   if (iters) *iters = total;
   if (res_out) *res_out = res;
