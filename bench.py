@@ -336,6 +336,7 @@ def run_ours(args, rank, world, local_rank):
 
 # kernel classes timed by the bench: (one-launch stage solves, block Jacobian)
 KERNELS = {"fp64": ("stage_gmres", "jacobian"), "mixed": ("stage_gmres32", "jacobian")}
+L2_BYTES_PER_CLK_SM = 25.0  # what L2 delivered to the products of the stage solves (2048 triangles, p = 3)
 PROF_STRIDE = 1   # every launch is bracketed by CUDA events (about 1,200 launches of these classes a step)
 
 
@@ -364,30 +365,30 @@ def roofline_for(kernel, res, peaks, fp64_tflops, c, sustained):
                 "note": "basis of one stage solve (<= 41 x N_u words) is L2-resident: a low fraction means "
                         "latency-bound grid reductions, not HBM"}
     if kernel == "jacobian":
-        # basis contraction of the 4 blocks plus the two tables W = C T per variable pair; the flux
-        # derivatives at the points are not counted
-        nqv, nqf = (p + 2) ** 2, 3 * (p + 2)
-        flops = 2.0 * ne * 16 * (Np * Np * (2 * nqv + 2 * nqf) + 3 * Np * (2 * nqv + 2 * nqf))
-        ach = flops / t / 1e12
-        return {"bound": "alu", "achieved": ach, "peak": fp64_tflops, "unit": "TFLOP/s",
-                "frac": ach / fp64_tflops if fp64_tflops else None, "traffic": None,
-                "kernel": "k_jacobian (element block Jacobian)", "launches": launches, "avg_us": t * 1e6}
+        # bytes written once: 4 blocks per element.  What bounds it is FP64 issue of the fluxes and factors and
+        # the barriers between them; the contractions run on the integer pipe, so no rate of products does.
+        ach = 8.0 * ne * 4 * nb * nb / t / 1e9
+        return {"bound": "latency", "achieved": ach, "peak": hbm, "unit": "GB/s", "frac": ach / hbm, "traffic": None,
+                "kernel": "k_jacobian (element block Jacobian)", "launches": launches, "avg_us": t * 1e6,
+                "note": "blocks written; bound by FP64 issue of the fluxes and by barriers, not by bytes"}
     word = 4 if kernel.endswith("32") else 8
     if kernel.startswith("stage_gmres"):
         # one launch = one solve of `steps` Krylov steps (mean over the last bench step's solves); a
         # step reads the 3 blocks and operand slices of every element once
+        # (FP64 and FP32 words alike; the FP64 products run on the integer pipe).  Held against what delivers
+        # the blocks: L2 while they fit, else HBM
         steps = res["steps_per_solve"]
-        byts = steps * ne * (3 * nb * nb + 5 * nb) * word
-        note = "%.1f steps per solve; blocks of one solve %.0f MB" % (steps, ne * 3 * nb * nb * word / 1e6)
-        common = {"traffic": MEASURED_TRAFFIC.get((kernel, res["config"])), "launches": launches, "avg_us": t * 1e6,
-                  "kernel": "k_stage_gmres<%d,%s> (whole stage solve, eliminated elements taken out)"
-                  % (nb, "double" if word == 8 else "float"), "hbm_gbs_equiv": byts / t / 1e9, "note": note}
-        if word == 8:
-            ach = 2.0 * steps * ne * 3 * nb * nb / t / 1e12
-            return {"bound": "alu", "achieved": ach, "peak": fp64_tflops, "unit": "TFLOP/s",
-                    "frac": ach / fp64_tflops if fp64_tflops else None, **common}
-        ach = byts / t / 1e9
-        return {"bound": "hbm", "achieved": ach, "peak": hbm, "unit": "GB/s", "frac": ach / hbm, **common}
+        blocks = ne * 3 * nb * nb * word
+        ach = steps * ne * (3 * nb * nb + 5 * nb) * word / t / 1e9
+        sm_mhz = (res.get("clocks") or {}).get("sm_mhz") or 2070.0
+        in_l2 = blocks <= 100e6
+        peak = L2_BYTES_PER_CLK_SM * 152 * sm_mhz * 1e6 / 1e9 if in_l2 else hbm
+        return {"bound": "l2" if in_l2 else "hbm", "achieved": ach, "peak": peak, "unit": "GB/s", "frac": ach / peak,
+                "traffic": MEASURED_TRAFFIC.get((kernel, res["config"])), "launches": launches, "avg_us": t * 1e6,
+                "kernel": "k_stage_gmres<%d,%s> (whole stage solve, eliminated elements taken out)"
+                % (nb, "double" if word == 8 else "float"),
+                "note": "%.1f steps per solve; blocks of one solve %.0f MB; the rest of a step are grid exchanges, "
+                        "projections and update" % (steps, blocks / 1e6)}
     # folded operator: 3 blocks + 3 neighbour slices + own slice + output per element
     byts = ne * (3 * nb * nb * word + 5 * nb * word)
     if word == 8:
