@@ -548,10 +548,10 @@ int ensure_store(pp_ctx* ctx, const pp_mesh* mesh, int Nt) {
 // Exponents of the powers nearest to (momentum, energy) M^1/2, M^2 for the normal system and M^-1/2, M^-3/2
 // for the transposed one, 1 above Mach 1.  Taken from a scan of both exponents in steps of 1/2 at M = 0.001 .. 0.05:
 // error of a product with the folded blocks per variable, relative to an FP64 FMA chain's, p = 1 .. 4, random,
-// one-variable and Krylov vectors (largest over all): M = 0.2: 0.3 .. 0.8; 0.05: 1.1; 0.01: 2.2; 0.002: 6.4.
-// Unscaled: 5.9; 81; 1900; 43,000.
+// one-variable and Krylov vectors (largest over all): M = 0.2: 0.2 .. 0.8 (once 2.0, 1.7e-16 against 8.7e-17);
+// 0.05: 1.1; 0.01: 2.2; 0.002: 6.4.  Unscaled: 5.9; 81; 1900; 43,000.
 FoldScale fold_scale(double mach) {
-  const double l = std::log2(std::min(mach, 1.0));
+  const double l = std::max(std::log2(std::min(mach, 1.0)), -250.0);  // the powers stay within the FP64 range
   FoldScale s;
   s.n = {(int)std::lround(0.5 * l), (int)std::lround(2.0 * l)};
   s.t = {-(int)std::lround(0.5 * l), -(int)std::lround(1.5 * l)};
