@@ -83,6 +83,10 @@ class POD:
 _F32 = torch.float32
 
 
+def _on_gpu(x):
+    return x.is_cuda
+
+
 def _addresses(*ptrs):
     """HOST array of device addresses."""
     return (C.c_void_p * len(ptrs))(*ptrs)
@@ -127,8 +131,10 @@ class MLP:
     @staticmethod
     def _checked(x, name, rows, cols):
         shape = x.shape
-        if len(shape) != 2 or shape[1] != cols or rows is not None and shape[0] != rows or x.dtype is not _F32:
-            raise ValueError(f"MLP: {name} is {x.dtype} {tuple(shape)}, not float32 [{rows or 'rows'}, {cols}]")
+        if (len(shape) != 2 or shape[1] != cols or rows is not None and shape[0] != rows or x.dtype is not _F32
+                or not _on_gpu(x)):
+            raise ValueError(f"MLP: {name} is {x.dtype} {tuple(shape)} on {x.device}, not float32 "
+                             f"[{rows or 'rows'}, {cols}] on the GPU")
         return x if x.is_contiguous() else x.contiguous()
 
     @staticmethod

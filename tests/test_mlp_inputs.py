@@ -7,6 +7,7 @@ import pytest
 
 torch = pytest.importorskip("torch")
 api = pytest.importorskip("paper_1512_00616_gb300.api")
+from paper_1512_00616_gb300 import warmstart  # noqa: E402
 from paper_1512_00616_gb300.warmstart import MLP  # noqa: E402
 
 
@@ -16,6 +17,7 @@ def calls(monkeypatch):
     call = lambda name: lambda n, rows, sizes, *a: got.append((name, list(sizes), rows)) or 0  # noqa: E731
     monkeypatch.setattr(api, "_lib", types.SimpleNamespace(pp_mlp_forward_f32=call("forward"), pp_mlp_backward_f32=call("backward")))
     monkeypatch.setattr(api, "_stream", lambda: None)
+    monkeypatch.setattr(warmstart, "_on_gpu", lambda x: True)
     return got
 
 
@@ -64,6 +66,14 @@ def test_layers_changed_between_the_passes_are_refused(calls):
     net.params[0] = [torch.zeros(6, 9), torch.zeros(9)]
     with pytest.raises(ValueError):
         net.backward(torch.zeros(5, 4))
+
+
+def test_inputs_on_the_cpu_are_refused(calls, monkeypatch):
+    net = MLP([6, 8, 4], device="cpu")
+    monkeypatch.setattr(warmstart, "_on_gpu", lambda x: x.is_cuda)
+    with pytest.raises(ValueError):
+        net.forward(torch.zeros(5, 6))
+    assert not calls
 
 
 def test_the_calls_check_their_tensors():
